@@ -16,7 +16,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libamgp2.so")
-SOURCES = ["api.cu", "setup.cu", "cycle.cu", "flow.cu", "krylov.cu", "batched.cu", "noalloc.cu",
+SOURCES = ["api.cu", "setup.cu", "cycle.cu", "flow.cu", "coarse_map.cu", "krylov.cu", "batched.cu", "noalloc.cu",
            "learned.cu", "mlp.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",

@@ -247,6 +247,13 @@ struct amg_handle {
   amgp2::DBuf<unsigned char> full_ph32, full_ph64;
   int full_n32 = 0, full_n64 = 0;
   amgp2::DBuf<unsigned> grid_bar;
+  // the cycle from level map_from down as one stored matrix (coarse_map.cu; -1: off),
+  // map_m x map_m row-major with rows map_ld apart, in the cycle's precision
+  int map_from = -1;
+  int map_m = 0, map_ld = 0;
+  amgp2::DBuf<float> map32;
+  amgp2::DBuf<double> map64;
+  std::vector<double> map_w;         // the weights that it was built with
   // batched (multi-right-hand-side) solves
   std::vector<amgp2::BatchLevel> B;
   amgp2::DBuf<double> mb, mx, mr, mz, mp, mq, mro, bred, bscal;
@@ -298,6 +305,15 @@ void level_transfer(amg_handle* h, int l, bool restrict_, bool f32);
 void autotune_levels(amg_handle* h);
 // records the cluster sub-cycle from level `from` (0 disables it)
 void set_subcycle(amg_handle* h, int from);
+
+// coarse_map.cu: the cycle below a level as one stored matrix
+// picks the level and allocates the matrix (before autotune_levels)
+void map_plan(amg_handle* h);
+// fills the matrix for the level weights w (host, 4 a level); again when they changed
+void map_build(amg_handle* h, const double* w);
+// x = (the cycle from level map_from) b, vectors of that level in the padded layout
+template <typename T, typename IO>
+void map_apply(amg_handle* h, const IO* b, IO* x);
 
 // krylov (krylov.cu)
 int solve_device(amg_handle* h, const double* b, double* x, double tol, amg_stats* st);

@@ -1,0 +1,632 @@
+// The cycle below a level as one stored matrix.
+//
+// From x = 0, what Algorithm 1 does on level l and below (every sweep, transfer and the
+// coarsest solve, nu times) is linear in the level's right-hand side: x_l = M b_l with a
+// dense m x m matrix M, m the level's unknowns.  Run operation by operation it is a chain
+// of about 2 x 30 colours and 5 other launches a level, each a few microseconds whatever
+// the level's size (elasticity 32^3, FP32: 280 us of the 774 us preconditioner below
+// level 1, for 8,538 unknowns; FP64 24^3: 690 us of 1317 us for 3,144).  M b instead reads
+// m^2 values once.  M is filled at setup, and again when the level weights change, by
+// running the cycle's own recorded operations on blocks of unit vectors, so it is the same
+// operator, weights, smoother and cycle type, in the cycle's precision.
+#include <cuda_bf16.h>
+
+#include <algorithm>
+#include <type_traits>
+#include <vector>
+
+#include "amg_internal.cuh"
+#include "phase.cuh"
+#include "vec.cuh"
+
+namespace amgp2 {
+
+namespace {
+
+// ------------------------------------------------------------------- blocks of vectors
+
+// A block of W vectors is stored entry by entry: entry k of vector c at k * W + c, so
+// consecutive threads take consecutive vectors and every value of an operator is one
+// broadcast load for a warp.  A thread holds 2 vectors (16 bytes an entry).
+//
+// FP64 handles build in FP64.  FP32 handles build in FP32 pairs (hi + lo, as the Krylov
+// operator) with the cycle's own FP32 (or BF16) operator values: M is then the cycle of
+// those operators to about 2^-48, rounded once, and M b is no further from the 64-bit
+// cycle than the FP32 operations were.  Built in plain FP32, M doubled that error (32^3:
+// 7.1e-7 against 3.4e-7 relative).  FP64 would take the m nnz FMAs of three sweeps at
+// 0.5e12 a second (87 ms at 32^3); the pairs issue at the FP32 rate.
+constexpr int kColThreads = 128;
+constexpr int kColN = 2;                             // vectors of a thread
+constexpr int kColBlock = kColThreads * kColN;       // vectors of a CTA
+constexpr int kColMax = 16 * kColBlock;              // vectors of one pass
+
+struct Pair {
+  float h, l;
+};
+__device__ __forceinline__ void mac(double& s, double a, double x) { s = fma(a, x, s); }
+// s += a x: the rounded sum and its error, exact where |s| >= |a x| (FastTwoSum with the
+// product unrounded); a step where the product is the larger one may lose its rounding
+// error, as a plain FP32 step does, which the result, rounded to FP32, can bear
+__device__ __forceinline__ void mac(Pair& s, float a, Pair x) {
+  const float t = fmaf(a, x.h, s.h);
+  const float e = fmaf(a, x.h, __fsub_rn(s.h, t));
+  s.l = fmaf(a, x.l, s.l) + e;
+  s.h = t;
+}
+__device__ __forceinline__ void add(double& s, double x) { s += x; }
+__device__ __forceinline__ void add(Pair& s, Pair x) { pair_add(s.h, s.l, x.h, x.l); }
+__device__ __forceinline__ double scaled(double om, double s, double d) { return om * s / d; }
+__device__ __forceinline__ Pair scaled(float om, Pair s, float d) {   // om s / d
+  Pair t{0.f, 0.f};
+  mac(t, om, s);
+  const float q = t.h / d;
+  return {q, (fmaf(-q, d, t.h) + t.l) / d};
+}
+__device__ __forceinline__ double wide(double x) { return x; }
+__device__ __forceinline__ double wide(Pair x) { return (double)x.h + (double)x.l; }
+__device__ __forceinline__ void narrow(double& x, double v) { x = v; }
+__device__ __forceinline__ void narrow(Pair& x, double v) {
+  x.h = (float)v;
+  x.l = (float)(v - (double)x.h);
+}
+__device__ __forceinline__ double normal(double x) { return x; }
+__device__ __forceinline__ Pair normal(Pair x) {   // |h| >= |l| (FastTwoSum)
+  const float h = __fadd_rn(x.h, x.l);
+  return {h, __fsub_rn(x.l, __fsub_rn(h, x.h))};
+}
+__device__ __forceinline__ double round_to(double, double x) { return x; }
+__device__ __forceinline__ float round_to(float, Pair x) { return x.h; }
+
+template <typename T>
+struct alignas(16) Cell {   // an entry of neighbouring vectors
+  T v[kColN];
+};
+template <typename T>
+__device__ __forceinline__ Cell<T> ldc(const T* p) {
+  union { float4 f; Cell<T> c; } u;
+  u.f = *reinterpret_cast<const float4*>(p);
+  return u.c;
+}
+template <typename T>
+__device__ __forceinline__ void stc(T* p, const Cell<T>& c) {
+  union { float4 f; Cell<T> c; } u;
+#pragma unroll
+  for (int q = 0; q < kColN; ++q) u.c.v[q] = normal(c.v[q]);
+  *reinterpret_cast<float4*>(p) = u.f;
+}
+template <typename T>
+__device__ __forceinline__ Cell<T> zero() {
+  return Cell<T>{};
+}
+template <typename T, typename S>
+__device__ __forceinline__ void axpy(Cell<T>& s, S a, const Cell<T>& x) {
+#pragma unroll
+  for (int q = 0; q < kColN; ++q) mac(s.v[q], a, x.v[q]);
+}
+template <typename T>
+__device__ __forceinline__ void add(Cell<T>& s, const Cell<T>& x) {
+#pragma unroll
+  for (int q = 0; q < kColN; ++q) add(s.v[q], x.v[q]);
+}
+template <typename S, typename V>
+__device__ __forceinline__ S value(const V* p) {
+  if constexpr (std::is_same<S, V>::value) return __ldg(p);
+  else return __bfloat162float(__ldg(p));
+}
+// unpadded unknown j -> entry of the padded layout
+__device__ __forceinline__ int pad_index(int j, int n3) {
+  return j < n3 ? 4 * (j / 3) + j % 3 : j + n3 / 3;
+}
+
+// block rows of A (rows_body of the cycle): CTA per row and column block.  T: entries of
+// the vectors; S: operator scalars; V: storage of the block values
+template <typename T, typename S, typename V>
+__global__ void __launch_bounds__(kColThreads) k_cols_rows(const Phase P, int W) {
+  const int g = blockIdx.x;
+  const int64_t c = (int64_t)blockIdx.y * kColBlock + threadIdx.x * kColN;
+  const T* x = (const T*)P.x + c;
+  const V* val = (const V*)P.val;
+  const int i = P.rows ? __ldg(P.rows + g) : g;
+  const int a = __ldg(P.rowptr + g), e = __ldg(P.rowptr + g + 1);
+  // the row's columns and values staged in shared memory, kStage blocks at a time; A sums
+  // of every A-th block each, whose loads are in flight together
+  constexpr int A = 4, kStage = 64;
+  __shared__ int sj[kStage];
+  __shared__ S sv[kStage][9];
+  Cell<T> s[A][3];
+#pragma unroll
+  for (int u = 0; u < A; ++u)
+#pragma unroll
+    for (int q = 0; q < 3; ++q) s[u][q] = zero<T>();
+  for (int k0 = a; k0 < e; k0 += kStage) {
+    const int n = min(kStage, e - k0);
+    __syncthreads();
+    for (int t = threadIdx.x; t < 9 * n; t += kColThreads)
+      sv[t % n][t / n] = value<S>(val + (t / n) * P.nnz + k0 + t % n);
+    for (int t = threadIdx.x; t < n; t += kColThreads) sj[t] = 4 * __ldg(P.col + k0 + t);
+    __syncthreads();
+    int k = 0;
+    for (; k + A <= n; k += A) {
+      Cell<T> xv[A][3];
+#pragma unroll
+      for (int u = 0; u < A; ++u)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) xv[u][q] = ldc(x + (int64_t)(sj[k + u] + q) * W);
+#pragma unroll
+      for (int u = 0; u < A; ++u)
+#pragma unroll
+        for (int q = 0; q < 9; ++q) axpy(s[u][q / 3], sv[k + u][q], xv[u][q % 3]);
+    }
+    for (; k < n; ++k)
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const Cell<T> v = ldc(x + (int64_t)(sj[k] + q) * W);
+#pragma unroll
+        for (int p = 0; p < 3; ++p) axpy(s[0][p], sv[k][3 * p + q], v);
+      }
+  }
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    add(s[0][q], s[1][q]);
+    add(s[2][q], s[3][q]);
+    add(s[0][q], s[2][q]);
+  }
+  T* y = (T*)P.y + c;
+  const int64_t o = 4 * (int64_t)i * W;
+  if (P.mode == kApply) {
+#pragma unroll
+    for (int q = 0; q < 3; ++q) stc(y + o + q * W, s[0][q]);
+    return;
+  }
+  const T* b = (const T*)P.b + c;
+  Cell<T> r[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    r[q] = ldc(b + o + q * W);
+#pragma unroll
+    for (int w = 0; w < kColN; ++w) s[0][q].v[w] = normal(s[0][q].v[w]);
+    axpy(r[q], S(-1), s[0][q]);
+    if (P.mode == kResid) stc(y + o + q * W, r[q]);
+#pragma unroll
+    for (int w = 0; w < kColN; ++w) r[q].v[w] = normal(r[q].v[w]);
+  }
+  if (P.mode == kResid) return;
+  const S om = P.wt ? (S)(P.omega * P.wt[0]) : (S)P.omega;
+  const S* d = (const S*)P.dinv + 12 * (int64_t)i;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    Cell<T> t = zero<T>(), xi = ldc(x + o + q * W);
+#pragma unroll
+    for (int p = 0; p < 3; ++p) axpy(t, __ldg(d + 4 * q + p), r[p]);
+#pragma unroll
+    for (int w = 0; w < kColN; ++w) t.v[w] = normal(t.v[w]);
+    axpy(xi, om, t);
+    stc(y + o + q * W, xi);
+  }
+}
+
+// the other operations of the cycle, CTA per item (row, node or entry) and column block
+template <typename T, typename S>
+__global__ void __launch_bounds__(kColThreads) k_cols_phase(const Phase P, int W) {
+  const int i = blockIdx.x;
+  const int64_t c = (int64_t)blockIdx.y * kColBlock + threadIdx.x * kColN;
+  const T* x = (const T*)P.x + c;
+  const T* b = (const T*)P.b + c;
+  T* y = (T*)P.y + c;
+  const S* val = (const S*)P.val;
+  const int64_t o = (int64_t)i * W, o4 = 4 * (int64_t)i * W;
+  auto norm = [](Cell<T> v) {
+#pragma unroll
+    for (int w = 0; w < kColN; ++w) v.v[w] = normal(v.v[w]);
+    return v;
+  };
+  switch (P.type) {
+    case PH_COPY: stc(y + o, ldc(x + o)); break;
+    case PH_RESTRICT:
+    case PH_PROLONG: {
+      Cell<T> s[3] = {zero<T>(), zero<T>(), zero<T>()};
+      for (int t = P.rowptr[i]; t < P.rowptr[i + 1]; ++t) {
+        const int64_t j = 4 * (int64_t)P.col[t] * W;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) axpy(s[q], val[t], ldc(x + j + q * W));
+      }
+      const S wc = P.wt ? (S)P.wt[1] : S(1);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        if (P.type == PH_PROLONG) {
+          Cell<T> v = ldc(y + o4 + q * W);
+          axpy(v, wc, norm(s[q]));
+          s[q] = v;
+        }
+        stc(y + o4 + q * W, s[q]);
+      }
+      break;
+    }
+    case PH_RESTRICT1:
+    case PH_PROLONG1: {
+      Cell<T> s = zero<T>();
+      for (int t = P.rowptr[i]; t < P.rowptr[i + 1]; ++t)
+        axpy(s, val[t], ldc(x + (int64_t)P.col[t] * W));
+      if (P.type == PH_PROLONG1) {
+        Cell<T> v = ldc(y + o);
+        axpy(v, P.wt ? (S)P.wt[1] : S(1), norm(s));
+        s = v;
+      }
+      stc(y + o, s);
+      break;
+    }
+    case PH_COARSE: {   // the generalised inverse in FP64, as in the cycle
+      double s[kColN] = {};
+      for (int j = 0; j < P.m; ++j) {
+        const double X = P.X[(int64_t)i * P.m + j];
+        const Cell<T> v = ldc(b + (int64_t)pad_index(j, P.n3) * W);
+#pragma unroll
+        for (int q = 0; q < kColN; ++q) s[q] = fma(X, wide(v.v[q]), s[q]);
+      }
+      Cell<T> t;
+#pragma unroll
+      for (int q = 0; q < kColN; ++q) narrow(t.v[q], s[q]);
+      stc(y + (int64_t)pad_index(i, P.n3) * W, t);
+      break;
+    }
+    case PH_BT_ADD: {
+      Cell<T> s[3] = {zero<T>(), zero<T>(), zero<T>()};
+      for (int t = P.rowptr[i]; t < P.rowptr[i + 1]; ++t) {
+        const Cell<T> p = ldc(x + (int64_t)P.col[t] * W);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) axpy(s[q], val[q * P.nnz + t], p);
+      }
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        Cell<T> v = ldc(y + o4 + q * W);
+        axpy(v, (S)P.omega, norm(s[q]));
+        stc(y + o4 + q * W, v);
+      }
+      break;
+    }
+    case PH_PROWS: {
+      const T* p = (const T*)P.p + c;
+      Cell<T> s = zero<T>(), cp = zero<T>();
+      for (int t = P.rowptr[i]; t < P.rowptr[i + 1]; ++t) {
+        const int64_t j = 4 * (int64_t)P.col[t] * W;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) axpy(s, val[q * P.nnz + t], ldc(x + j + q * W));
+      }
+      if (P.mode != 3)
+        for (int t = P.crow[i]; t < P.crow[i + 1]; ++t)
+          axpy(cp, ((const S*)P.cval)[t], ldc(p + (int64_t)P.ccol[t] * W));
+      axpy(s, S(-1), norm(cp));                        // B u - C p
+      if (P.mode == 1) {
+        Cell<T> g = ldc(b + o);
+        axpy(g, S(-1), norm(s));
+        s = g;
+      } else if (P.mode == 3) {
+        axpy(s, S(-1), ldc(b + o));
+      } else if (P.mode == 2) {
+        const S om = P.wt ? (S)(P.omega * P.wt[2]) : (S)P.omega;
+        const S d = ((const S*)P.sd)[i];
+        axpy(s, S(-1), ldc(b + o));
+        s = norm(s);
+        Cell<T> v = ldc(p + o);
+        if (d != S(0)) {
+#pragma unroll
+          for (int q = 0; q < kColN; ++q) add(v.v[q], scaled(om, s.v[q], d));
+        }
+        s = v;
+      }
+      stc(y + o, s);
+      break;
+    }
+    case PH_SROWS: {
+      Cell<T> s = ldc(b + o);
+      for (int t = P.rowptr[i]; t < P.rowptr[i + 1]; ++t)
+        axpy(s, -val[t], ldc(x + (int64_t)P.col[t] * W));
+      if (P.mode == 1) {
+        Cell<T> v = ldc(x + o);
+        axpy(v, (S)P.omega * ((const S*)P.dinv)[i], norm(s));
+        s = v;
+      }
+      stc(y + o, s);
+      break;
+    }
+    case PH_VEC: {
+      Cell<T> v = zero<T>();
+      if (P.mode == 0) {
+        axpy(v, (S)P.omega * ((const S*)P.dinv)[i], ldc(x + o));
+      } else {
+        v = ldc(y + o);
+        add(v, ldc(x + o));
+        if (P.mode == 2) axpy(v, -((const S*)P.dinv)[i], ldc(b + o));
+      }
+      stc(y + o, v);
+      break;
+    }
+    default:
+      break;
+  }
+}
+
+// unit vectors first, first + 1, ... of the level's m unknowns (the block is zero before)
+template <typename T>
+__global__ void k_cols_unit(T* b, int first, int m, int n3, int W) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c < W && first + c < m) narrow(b[(int64_t)pad_index(first + c, n3) * W + c], 1.0);
+}
+
+// columns first.. of M from the block's solution vectors
+template <typename T, typename S>
+__global__ void k_cols_store(const T* __restrict__ x, S* __restrict__ M, int first, int m, int ld,
+                             int n3, int W) {
+  const int j = blockIdx.x;
+  for (int c = threadIdx.x; c < W && first + c < m; c += blockDim.x)
+    M[(int64_t)j * ld + first + c] = round_to(S(0), x[(int64_t)pad_index(j, n3) * W + c]);
+}
+
+// The blocks of vectors that stand for the level work vectors while phases run on W
+// columns: a phase's vector operand is found by the level vector that it points into.
+template <typename T, typename S>
+struct ColVectors {
+  struct Range {
+    const S* base;
+    int64_t n;
+    int64_t at;
+  };
+  std::vector<Range> ranges;
+  int64_t total = 0;
+  DBuf<T> mem;
+
+  void add(const DBuf<S>& v) {
+    if (v.p) ranges.push_back({v.p, (int64_t)v.n, -1});
+  }
+  Range* find(const void* p) {
+    const S* q = static_cast<const S*>(p);
+    for (Range& r : ranges)
+      if (q >= r.base && q < r.base + r.n) return &r;
+    return nullptr;
+  }
+  void use(const void* p) {   // gives the vector of p its place
+    Range* r = p ? find(p) : nullptr;
+    if (r && r->at < 0) {
+      r->at = total;
+      total += r->n;
+    }
+  }
+  T* map(const void* p, int W) {
+    Range* r = find(p);
+    return r ? mem.p + (r->at + (static_cast<const S*>(p) - r->base)) * W : nullptr;
+  }
+};
+
+void add_level(ColVectors<double, double>& v, const Level& l) {
+  v.add(l.x64); v.add(l.b64); v.add(l.r64); v.add(l.t64);
+  for (const auto& s : l.S) { v.add(s->x64); v.add(s->b64); v.add(s->r64); }
+}
+void add_level(ColVectors<Pair, float>& v, const Level& l) {
+  v.add(l.x32); v.add(l.b32); v.add(l.r32); v.add(l.t32);
+  for (const auto& s : l.S) { v.add(s->x32); v.add(s->b32); v.add(s->r32); }
+}
+
+template <typename T, typename S>
+void run_cols(amg_handle* h, const Phase& P, int W) {
+  cudaStream_t s = h->stream;
+  if (P.type == PH_ZERO) {
+    if (P.n > 0) AMG_CUDA(cudaMemsetAsync(P.y, 0, (size_t)P.n * W * sizeof(T), s));
+    return;
+  }
+  const int items = P.type == PH_COARSE ? P.m : P.n;
+  if (items <= 0) return;
+  const dim3 grid(items, W / kColBlock);
+  if (P.type != PH_ROWS) {
+    k_cols_phase<T, S><<<grid, kColThreads, 0, s>>>(P, W);
+  } else if (P.vbf) {
+    if constexpr (std::is_same<S, float>::value)
+      k_cols_rows<T, float, __nv_bfloat16><<<grid, kColThreads, 0, s>>>(P, W);
+  } else {
+    k_cols_rows<T, S, S><<<grid, kColThreads, 0, s>>>(P, W);
+  }
+  h->launches++;
+}
+
+// M (the handle's precision S) from the cycle's operations on blocks of T vectors
+template <typename T, typename S>
+void build(amg_handle* h, S* M) {
+  // all columns at once up to kColMax: a launch's CTAs go over the rows of a colour first,
+  // so a block of 256 columns keeps its vectors in L2, and the small colours still fill the
+  // chip (512 columns a pass at 32^3: 97 ms, all but a few launches waiting on latency)
+  const int from = h->map_from, m = h->map_m;
+  const int nchunk = div_up(m, kColMax);
+  const int W = div_up(div_up(m, nchunk), kColBlock) * kColBlock;
+  std::vector<Phase> ph;
+  record_map_phases<S>(h, from, ph);
+  ColVectors<T, S> v;
+  for (size_t l = from; l < h->L.size(); ++l) add_level(v, *h->L[l]);
+  const Level& lv = *h->L[from];
+  constexpr bool f32 = std::is_same<S, float>::value;
+  const void* lb = f32 ? (const void*)lv.b32.p : lv.b64.p;
+  const void* lx = f32 ? (const void*)lv.x32.p : lv.x64.p;
+  v.use(lb);
+  v.use(lx);
+  for (const Phase& P : ph)
+    for (const void* q : {P.x, P.b, P.p, (const void*)P.y}) v.use(q);
+  v.mem.alloc((size_t)v.total * W);
+  T* b = v.map(lb, W);
+  T* x = v.map(lx, W);
+  for (Phase& P : ph) {
+    for (const void** q : {&P.x, &P.b, &P.p})
+      if (*q) *q = v.map(*q, W);
+    P.y = v.map(P.y, W);
+  }
+  AMG_CUDA(cudaMemsetAsync(v.mem.p, 0, v.mem.bytes(), h->stream));
+  const int n3 = 3 * lv.n;
+  for (int first = 0; first < m; first += W) {
+    AMG_CUDA(cudaMemsetAsync(b, 0, (size_t)lv.dofs4() * W * sizeof(T), h->stream));
+    k_cols_unit<T><<<div_up(W, 256), 256, 0, h->stream>>>(b, first, m, n3, W);
+    for (const Phase& P : ph) run_cols<T, S>(h, P, W);
+    k_cols_store<T, S><<<m, 256, 0, h->stream>>>(x, M, first, m, h->map_ld, n3, W);
+    h->launches += 2;
+  }
+  AMG_LAUNCH_CHECK();
+  AMG_CUDA(cudaStreamSynchronize(h->stream));   // the blocks are freed here
+}
+
+// ------------------------------------------------------------------- application
+
+constexpr int kMapThreads = 256;
+
+// the products of 16 bytes of a row, added to a running sum (FP32: with its rounding
+// error, TwoSum, so that a row's sum of thousands of terms loses no more than the short
+// sums of the cycle's sparse rows)
+template <typename T> struct Stream16;
+template <> struct Stream16<float> {
+  using type = float4;
+  struct Sum {
+    float s = 0.f, e = 0.f;
+    __device__ void add(float4 a, float4 b) {
+      const float d = fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, __fmul_rn(a.x, b.x))));
+      pair_add(s, e, d, 0.f);
+    }
+    __device__ void join(const Sum& o) { pair_add(s, e, o.s, o.e); }
+    __device__ void lane(int o) {
+      const float t = __shfl_xor_sync(0xffffffffu, s, o);
+      const float u = __shfl_xor_sync(0xffffffffu, e, o);
+      pair_add(s, e, t, u);
+    }
+    __device__ float value() const { return s + e; }
+  };
+};
+template <> struct Stream16<double> {
+  using type = double2;
+  struct Sum {
+    double s = 0.0;
+    __device__ void add(double2 a, double2 b) { s = fma(a.y, b.y, fma(a.x, b.x, s)); }
+    __device__ void join(const Sum& o) { s += o.s; }
+    __device__ void lane(int o) { s += __shfl_xor_sync(0xffffffffu, s, o); }
+    __device__ double value() const { return s; }
+  };
+};
+
+// x = M b, padded vectors of IO converted to T (FP32 handles at level 0 take the outer
+// FP64 vectors directly).  One warp a row at a time; b is staged unpadded in shared memory
+// by every CTA; the row's values stream with U 16-byte loads in flight a lane.  STREAM:
+// evict-first loads for a matrix beyond the L2 capacity, so that it does not push out the
+// vectors; a smaller one is left to stay in L2 from one application to the next.
+template <typename T, typename IO, bool STREAM>
+__global__ void __launch_bounds__(kMapThreads) k_map_apply(int m, int ld, int n3,
+                                                           const T* __restrict__ M,
+                                                           const IO* __restrict__ b,
+                                                           IO* __restrict__ x) {
+  using V = typename Stream16<T>::type;
+  constexpr int N = 16 / sizeof(T), U = 8;
+  extern __shared__ __align__(16) unsigned char map_smem[];
+  T* sb = reinterpret_cast<T*>(map_smem);
+  for (int j = threadIdx.x; j < ld; j += kMapThreads)
+    sb[j] = j < m ? (T)b[pad_index(j, n3)] : T(0);
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  const int nw = gridDim.x * (kMapThreads / 32);
+  const V* sv = reinterpret_cast<const V*>(sb);
+  const int nv = ld / N;
+  for (int i = blockIdx.x * (kMapThreads / 32) + (threadIdx.x >> 5); i < m; i += nw) {
+    const V* row = reinterpret_cast<const V*>(M + (int64_t)i * ld);
+    typename Stream16<T>::Sum s[4];
+    for (int k = lane; k < nv; k += 32 * U) {
+      V a[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (k + 32 * u < nv) a[u] = STREAM ? __ldcs(row + k + 32 * u) : __ldg(row + k + 32 * u);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (k + 32 * u < nv) s[u & 3].add(a[u], sv[k + 32 * u]);
+    }
+    s[0].join(s[1]);
+    s[2].join(s[3]);
+    s[0].join(s[2]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s[0].lane(o);
+    if (lane == 0) {
+      const int o = pad_index(i, n3);
+      x[o] = (IO)s[0].value();
+      if (i < n3 && (o & 3) == 2) x[o + 1] = IO(0);   // the node's padding
+    }
+  }
+}
+
+template <typename T>
+const T* matrix(const amg_handle* h) {
+  if constexpr (std::is_same<T, float>::value) return h->map32.p;
+  else return h->map64.p;
+}
+
+}  // namespace
+
+// The largest level stored as a matrix.  Below these sizes M b is faster than the chain
+// of launches that it replaces: reading M takes 4 m^2 bytes at about 6 TB/s in FP32 (63 us
+// at 10,240) against 65 launches of 2 to 5 us and the levels below; in FP64 the m^2 FMAs
+// take 75 us at 6,144 (0.5e12 a second on this GPU).  They also bound the memory (420 and
+// 300 MB) and the time of the construction.
+constexpr int kMapMax32 = 10240;
+constexpr int kMapMax64 = 6144;
+// and the share of the coarsest solve (FP64) in the construction
+constexpr int64_t kMapCoarseWork = 4000000000ll;
+
+void map_plan(amg_handle* h) {
+  const amg_options& o = h->opt;
+  h->map_from = -1;
+  // a launch variant that the caller forces keeps its levels; the Vanka phases are not recorded
+  if (o.cluster_from != -1 || o.cycle_kernel != 0 || o.gs_cluster != -1 || o.gs_flow != -1 ||
+      o.gs_stream != -1 || o.gs_tma != -1 || o.smoother == AMG_SMOOTHER_VANKA)
+    return;
+  const bool f32 = o.precision == AMG_FP32;
+  for (int l = 0; l + 1 < (int)h->L.size(); ++l) {
+    const int m = h->L[l]->dofs();
+    if (m > (f32 ? kMapMax32 : kMapMax64) ||
+        (int64_t)h->coarse_m * h->coarse_m * m > kMapCoarseWork)
+      continue;
+    h->map_m = m;
+    h->map_ld = (m + 31) / 32 * 32;
+    const size_t count = (size_t)m * h->map_ld;
+    try {
+      if (f32) h->map32.alloc(count);
+      else h->map64.alloc(count);
+    } catch (const Error& e) {
+      if (e.code != AMG_ERR_NOMEM) throw;
+      return;   // no room: the cycle runs operation by operation
+    }
+    // the padding of the rows stays 0
+    if (f32) AMG_CUDA(cudaMemsetAsync(h->map32.p, 0, h->map32.bytes(), h->stream));
+    else AMG_CUDA(cudaMemsetAsync(h->map64.p, 0, h->map64.bytes(), h->stream));
+    h->map_from = l;
+    return;
+  }
+}
+
+void map_build(amg_handle* h, const double* w) {
+  if (h->map_from < 0) return;
+  // the weights of the levels that M holds (4 a level): nothing to do if they are as built
+  const std::vector<double> now(w + 4 * h->map_from, w + 4 * h->L.size());
+  if (now == h->map_w) return;
+  h->map_w.clear();
+  if (h->map32.p) build<Pair, float>(h, h->map32.p);
+  else build<double, double>(h, h->map64.p);
+  h->map_w = now;
+}
+
+template <typename T, typename IO>
+void map_apply(amg_handle* h, const IO* b, IO* x) {
+  const int m = h->map_m, ld = h->map_ld, n3 = 3 * h->L[h->map_from]->n;
+  const T* M = matrix<T>(h);
+  const int smem = ld * (int)sizeof(T);
+  const bool stream = (int64_t)m * ld * sizeof(T) > (64ll << 20);
+  const auto k = stream ? k_map_apply<T, IO, true> : k_map_apply<T, IO, false>;
+  max_dynamic_smem((const void*)k, (sizeof(T) == 4 ? kMapMax32 : kMapMax64) * (int)sizeof(T));
+  // a warp a row where the rows allow it, at most four CTAs an SM
+  const int grid = std::max(1, std::min(div_up(m, kMapThreads / 32), 4 * 152));
+  k<<<grid, kMapThreads, smem, h->stream>>>(m, ld, n3, M, b, x);
+  h->launches++;
+}
+
+template void map_apply<float, float>(amg_handle*, const float*, float*);
+template void map_apply<float, double>(amg_handle*, const double*, double*);
+template void map_apply<double, double>(amg_handle*, const double*, double*);
+
+}  // namespace amgp2

@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "amg_internal.cuh"
+#include "phase.cuh"
 #include "vec.cuh"
 
 namespace cg = cooperative_groups;
@@ -24,8 +25,6 @@ namespace cg = cooperative_groups;
 namespace amgp2 {
 
 namespace {
-
-enum RowMode { kApply = 0, kResid = 1, kGS = 2, kJacobi = 3 };
 
 template <typename T>
 __device__ __forceinline__ T ldg(const T* p) { return __ldg(p); }
@@ -464,42 +463,6 @@ __global__ void __launch_bounds__(256) k_vanka(int npatch, const int* __restrict
 }
 
 // ------------------------------------------------------------------- phases
-
-enum PhaseType : int {
-  PH_ZERO = 0, PH_COPY, PH_ROWS, PH_RESTRICT, PH_PROLONG, PH_RESTRICT1, PH_PROLONG1,
-  PH_COARSE, PH_BT_ADD, PH_PROWS, PH_SROWS, PH_VEC, PH_VANKA
-};
-
-// One operation of the cycle with its operands (a plain record, copied to the
-// device for the cluster launch or passed by value to a single launch).
-struct Phase {
-  int type, mode, G, n;   // n: rows / nodes / entries
-  const int* rows;
-  const int* rowptr;
-  const int* col;
-  const void* val;
-  int64_t nnz;
-  const void* dinv;
-  const void* x;
-  const void* b;
-  void* y;
-  const int* crow;
-  const int* ccol;
-  const void* cval;
-  const void* sd;
-  const void* p;          // pressure iterate (PH_PROWS)
-  const double* X;
-  int m, n3;
-  double omega;
-  const double* wt;       // the level's learned weights (null: plain method)
-  int vbf;                // PH_ROWS: values stored as BF16 (FP32 arithmetic)
-  int sctas;              // PH_ROWS, Gauss-Seidel: CTAs per SM of the streaming colour
-                          // kernel (0: one group of lanes per row, k_gs_pdl)
-  int xnc;                // PH_ROWS, Gauss-Seidel (k_gs_pdl): x through the L1 path
-  int tma;                // PH_ROWS, Gauss-Seidel, FP32: the TMA-staged colour kernel
-  int* err;               // the handle's error word (bounded waits that gave up)
-  const long long* off;   // PH_VANKA: offsets of the patch inverses
-};
 
 template <typename T, bool COH, typename V = T>
 __device__ void dispatch_rows_v(const Phase& P, int warp, int nwarps) {
@@ -2180,6 +2143,10 @@ void cycle_rec(Emit<T>& e, amg_handle* h, int l, T* x, const T* b, bool x_is_zer
 template <typename T>
 void coarse_calls(Emit<T>& e, amg_handle* h, int l, T* xc, const T* bc) {
   const int L = (int)h->L.size() - 1;
+  if (!e.rec && h->map_from > 0 && l == h->map_from) {
+    map_apply<T, T>(h, bc, xc);
+    return;
+  }
   if (!e.rec && h->sub_from > 0 && l == h->sub_from) {
     SubCycle<T>::launch(h);
     return;
@@ -2391,9 +2358,27 @@ void vcycle(amg_handle* h, int l, bool x_is_zero) {
   cycle_rec<T>(e, h, l, LvVec<T>::x(lv), LvVec<T>::b(lv), x_is_zero);
 }
 
+template <typename T>
+void record_map_phases(amg_handle* h, int l, std::vector<Phase>& ph) {
+  Emit<T> e{h, &ph};
+  Level& lv = *h->L[l];
+  if (l > 0) {
+    coarse_calls<T>(e, h, l, LvVec<T>::x(lv), LvVec<T>::b(lv));
+    return;
+  }
+  for (int c = 0; c < std::max(1, h->opt.cycles); ++c)
+    cycle_rec<T>(e, h, 0, LvVec<T>::x(lv), LvVec<T>::b(lv), c == 0);
+}
+template void record_map_phases<float>(amg_handle*, int, std::vector<Phase>&);
+template void record_map_phases<double>(amg_handle*, int, std::vector<Phase>&);
+
 // z = M^{-1} r: opt.cycles applications of Algorithm 1 from zero.
 template <>
 void precondition_device<double>(amg_handle* h, const double* r, double* z) {
+  if (h->map_from == 0) {
+    map_apply<double, double>(h, r, z);
+    return;
+  }
   if (h->use_full) {
     Level& lv = *h->L[0];
     launch_copy(r, lv.b64, lv.dofs4(), h->stream, h);
@@ -2407,6 +2392,10 @@ void precondition_device<double>(amg_handle* h, const double* r, double* z) {
 
 template <>
 void precondition_device<float>(amg_handle* h, const double* r, double* z) {
+  if (h->map_from == 0) {
+    map_apply<float, double>(h, r, z);
+    return;
+  }
   Level& lv = *h->L[0];
   const int64_t n = lv.dofs4();
   launch_to_float(r, lv.b32, n, h->stream, h);
@@ -2486,7 +2475,9 @@ void autotune_levels(amg_handle* h) {
     return ms;
   };
   const bool f32 = h->opt.precision == AMG_FP32;
-  for (size_t l = 0; l < h->L.size(); ++l) {
+  // levels that run as one stored matrix keep the default lanes per row
+  const size_t nl = h->map_from >= 0 ? std::max(h->map_from, 1) : h->L.size();
+  for (size_t l = 0; l < nl; ++l) {
     Level& lv = *h->L[l];
     lv.gs_cl = 0;
     int best = 0;
@@ -2534,7 +2525,9 @@ void autotune_levels(amg_handle* h) {
       lv.group_pair = best;
       AMG_CUDA(cudaStreamSynchronize(s));
     }
-    if (lv.ncolours == 0 || h->saddle || h->opt.smoother != AMG_SMOOTHER_GS) continue;
+    if (lv.ncolours == 0 || h->saddle || h->opt.smoother != AMG_SMOOTHER_GS ||
+        h->map_from == 0)
+      continue;
     best = 0;
     best_ms = 1e30f;
     for (int G : {4, 8, 16, 32}) {
@@ -2728,6 +2721,11 @@ void autotune_levels(amg_handle* h) {
     if (ferr)
       fail(AMG_ERR_TIMEOUT, "a bounded wait of a one-launch colour sweep (mbarrier or dataflow "
                             "flag) timed out during setup tuning");
+  }
+  if (h->map_from >= 0) {
+    cudaEventDestroy(e0);
+    cudaEventDestroy(e1);
+    return;
   }
   // cluster sub-cycle: the largest cluster that fits (16, else 8 CTAs), then the
   // fastest start level among 1..L (or none)

@@ -264,6 +264,7 @@ void set_level_weights(amg_handle* h, const double* w, int n) {
   AMG_CUDA(cudaMemcpyAsync(h->wts.p, v.data(), v.size() * sizeof(double), cudaMemcpyHostToDevice,
                            h->stream));
   AMG_CUDA(cudaStreamSynchronize(h->stream));
+  map_build(h, v.data());   // the stored coarse cycle holds the weights
 }
 
 void set_weights(amg_handle* h, const double* w3) {
@@ -278,6 +279,7 @@ void set_weights(amg_handle* h, const double* w3) {
   AMG_CUDA(cudaMemcpyAsync(h->wts.p, w.data(), w.size() * sizeof(double), cudaMemcpyHostToDevice,
                            h->stream));
   AMG_CUDA(cudaStreamSynchronize(h->stream));
+  map_build(h, w.data());
 }
 
 void get_weights(const amg_handle* h, double* out) {

@@ -1888,7 +1888,9 @@ void build_hierarchy(amg_handle* h, const amg_matrix* m, const int32_t* tags) {
   factor_coarsest(h);
   if (h->saddle && h->opt.smoother == AMG_SMOOTHER_BS) bs_setup(h);
   if (h->saddle && h->opt.smoother == AMG_SMOOTHER_VANKA) vanka_setup(h);
+  map_plan(h);
   autotune_levels(h);
+  map_build(h, std::vector<double>(4 * h->L.size(), 1.0).data());
   AMG_CUDA(cudaStreamSynchronize(s));
 }
 
