@@ -7,6 +7,7 @@
 #include <cstring>
 #include <memory>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "amgp2.h"
@@ -106,7 +107,6 @@ struct Level {
   int group_gs = 0;     // the same for the colour-subset Gauss-Seidel kernel
   int gs_stream = 0;    // CTAs per SM of the grid-stride colour kernel (0: k_gs_pdl)
   int gs_tma = 0;       // 1: the FP32 colour kernel stages its rows' blocks by TMA (k_gs_tma)
-  int gs_xnc = 0;       // k_gs_pdl gathers x through L1 (1) or L2 only (0), by timing
   int group64 = 0;      // the FP64 operator kernel when the cycle runs in FP32
   // level 0 of an FP32 SPD handle with outer_pair: the kernel-layout values as
   // 9 planes of (hi, lo) float pairs, hi = fl32(a), lo = fl32(a - hi)
@@ -128,9 +128,17 @@ struct Level {
   int flow = 0;
   int flow_nchunks = 0;
   int flow_grid32 = 0, flow_grid64 = 0;
-  // learned weights of this level on the device: [0] relaxation multiplier,
-  // [1] coarse-correction scale, [2] pressure-step multiplier (all 1: plain)
+  // the level's steps on the device, learned weights included (1: the plain method), in
+  // both precisions so that no kernel converts them (an FP64 instruction a warp): [0] ws
+  // (Gauss-Seidel), [1] wc (coarse correction), [2] omega ws (damped block Jacobi),
+  // [3] omega_p wp (sGS pressure step)
   double* wt = nullptr;
+  float* wt32 = nullptr;
+  template <class T>
+  const T* steps() const {
+    if constexpr (std::is_same<T, float>::value) return wt32;
+    else return wt;
+  }
 
   // transfer to level+1 (absent on the coarsest level)
   DBuf<int> state, cid;
@@ -259,7 +267,9 @@ struct amg_handle {
   amgp2::DBuf<double> mb, mx, mr, mz, mp, mq, mro, bred, bscal;
   amgp2::DBuf<float> mpf;           // the directions in pair form (FP32-pair operator)
   amgp2::DBuf<int> bit;
-  amgp2::DBuf<double> wts;          // 4 learned weights per level (see Level::wt)
+  amgp2::DBuf<double> wts;          // 4 learned weights per level: ws, wc, wp, 1
+  amgp2::DBuf<double> steps;        // 4 steps per level (Level::wt)
+  amgp2::DBuf<float> steps32;
   bool bf16_coarse = false;         // AMG_FP32_BF16: levels >= 1 keep BF16 values
   ~amg_handle();
 };
@@ -337,6 +347,8 @@ void check_wait_flag(amg_handle* h, const char* what);
 constexpr double kProbeTol = 1e-8;   // the probe solves run to the stopping tolerance of the workloads
 void compute_features(amg_handle* h, double* out);
 void compute_level_features(amg_handle* h, int l, double* out);
+// copies w (4 a level: ws, wc, wp, 1) and the steps that follow from it to the device
+void upload_weights(amg_handle* h, const std::vector<double>& w);
 void set_weights(amg_handle* h, const double* w3);
 void set_level_weights(amg_handle* h, const double* w, int n);
 void get_weights(const amg_handle* h, double* out);

@@ -46,8 +46,8 @@ __global__ void __launch_bounds__(256) k_rows_m(int nrows, const int* __restrict
                                                 const T* __restrict__ val, int64_t nnzb,
                                                 const T* x, const T* __restrict__ b, T* y,
                                                 const T* __restrict__ dinv, T omega,
-                                                const double* __restrict__ wt) {
-  if (wt) omega = (T)((double)omega * wt[0]);   // learned relaxation multiplier
+                                                const T* __restrict__ wt) {
+  if (wt) omega = wt[MODE == mGS ? 0 : 2];   // the level's step, weights included
   const int g = (blockIdx.x * blockDim.x + threadIdx.x) / (K * S);
   const int q = (threadIdx.x / K) % S;
   const int r = threadIdx.x % K;
@@ -173,8 +173,8 @@ __global__ void k_restrict_m(int nc, const int* __restrict__ rrow, const int* __
 template <typename T>
 __global__ void k_prolong_m(int n, const int* __restrict__ prow, const int* __restrict__ pcol,
                             const T* __restrict__ pval, const T* __restrict__ xc, T* x,
-                            const double* __restrict__ wt) {
-  const T wc = wt ? (T)wt[1] : T(1);   // coarse-correction scale
+                            const T* __restrict__ wt) {
+  const T wc = wt ? wt[1] : T(1);   // coarse-correction scale
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int i = t / K, r = t % K;
   if (i >= n) return;
@@ -448,7 +448,7 @@ __global__ void __launch_bounds__(256) k_gs_m_pdl(int nrows, const int* __restri
                                                   const T* __restrict__ val, int64_t nnzb, T* x,
                                                   const T* __restrict__ b,
                                                   const T* __restrict__ dinv,
-                                                  const double* __restrict__ wt) {
+                                                  const T* __restrict__ wt) {
   // S > 2: the S / 2 warps of a row combine their sums through shared memory
   __shared__ T red[S > 2 ? 256 / 32 : 1][K][3];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -487,7 +487,7 @@ __global__ void __launch_bounds__(256) k_gs_m_pdl(int nrows, const int* __restri
   // (the restriction before a sweep's first colour): read only after the wait
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (S <= 2 && !active) return;   // S > 2: every thread reaches the block barrier below
-  const T om = wt ? (T)wt[0] : T(1);   // learned relaxation multiplier (1: plain)
+  const T om = wt ? wt[0] : T(1);   // learned relaxation multiplier (1: plain)
   if (active && q == 0) ld3(b, i * K + r, b0, b1, b2);
   T s0 = T(0), s1 = T(0), s2 = T(0);
 #pragma unroll
@@ -561,7 +561,7 @@ void launch_gs_m_pdl(int nrows, const int* rows, const int* rowptr, Level& lv, c
   cfg.numAttrs = 1;
   AMG_CUDA(cudaLaunchKernelEx(&cfg, k_gs_m_pdl<T, S, U>, nrows, rows, rowptr,
                               (const int*)lv.k_col(), val, lv.nnzb, x, b, dinv,
-                              (const double*)lv.wt));
+                              lv.template steps<T>()));
 }
 
 // one colour of the batched Gauss-Seidel sweep (x updated in place)
@@ -587,7 +587,7 @@ void gs_colour_m(amg_handle* h, Level& lv, int first, int nrows, const T* val, T
 
 template <typename T, int MODE, int S, int U>
 void launch_rows_m(int nrows, const int* rows, const int* rowptr, Level& lv, const T* val,
-                   const T* x, const T* b, T* y, const T* dinv, T omega, const double* wt,
+                   const T* x, const T* b, T* y, const T* dinv, T omega, const T* wt,
                    cudaStream_t s) {
   const int grid = (int)(((int64_t)nrows * K * S + 255) / 256);
   k_rows_m<T, MODE, S, U><<<grid, 256, 0, s>>>(nrows, rows, rowptr, lv.k_col(), val, lv.nnzb, x,
@@ -597,7 +597,7 @@ void launch_rows_m(int nrows, const int* rows, const int* rowptr, Level& lv, con
 template <typename T, int MODE>
 void launch_tile_m(int tile, int nrows, const int* rows, const int* rowptr, Level& lv,
                    const T* val, const T* x, const T* b, T* y, const T* dinv, T omega,
-                   const double* wt, cudaStream_t s) {
+                   const T* wt, cudaStream_t s) {
   switch (tile) {
     case 1: launch_rows_m<T, MODE, 2, 2>(nrows, rows, rowptr, lv, val, x, b, y, dinv, omega, wt, s); break;
     case 2: launch_rows_m<T, MODE, 1, 4>(nrows, rows, rowptr, lv, val, x, b, y, dinv, omega, wt, s); break;
@@ -641,10 +641,10 @@ void rows_m(amg_handle* h, int mode, Level& lv, int first, int nrows, const T* v
       launch_tile_m<T, mResid>(tile, nrows, rows, rowptr, lv, val, x, b, y, dinv, omega, nullptr, s);
       break;
     case mGS:
-      launch_tile_m<T, mGS>(tile, nrows, rows, rowptr, lv, val, x, b, y, dinv, omega, lv.wt, s);
+      launch_tile_m<T, mGS>(tile, nrows, rows, rowptr, lv, val, x, b, y, dinv, omega, lv.template steps<T>(), s);
       break;
     default:
-      launch_tile_m<T, mJacobi>(tile, nrows, rows, rowptr, lv, val, x, b, y, dinv, omega, lv.wt, s);
+      launch_tile_m<T, mJacobi>(tile, nrows, rows, rowptr, lv, val, x, b, y, dinv, omega, lv.template steps<T>(), s);
       break;
   }
   h->launches++;
@@ -710,7 +710,7 @@ void cycle_m(amg_handle* h, int l, T* x, const T* b, bool x_is_zero) {
     cycle_m<T>(h, l + 1, MV<T>::x(bn), MV<T>::b(bn), k == 0);
   k_prolong_m<T><<<gridk((int64_t)lv.n * K), 256, 0, s>>>(lv.n, lv.p_rowptr, lv.p_col,
                                                           MV<T>::pval(lv), MV<T>::x(bn), x,
-                                                          lv.wt);
+                                                          lv.template steps<T>());
   h->launches++;
   for (int k = 0; k < h->opt.m_post; ++k) smooth_m<T>(h, l, x, b, h->opt.post_order != 1);
 }

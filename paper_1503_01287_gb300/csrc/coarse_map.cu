@@ -191,7 +191,8 @@ __global__ void __launch_bounds__(kColThreads) k_cols_rows(const Phase P, int W)
     for (int w = 0; w < kColN; ++w) r[q].v[w] = normal(r[q].v[w]);
   }
   if (P.mode == kResid) return;
-  const S om = P.wt ? (S)(P.omega * P.wt[0]) : (S)P.omega;
+  const S* wt = (const S*)P.wt;
+  const S om = wt ? wt[P.mode == kGS ? 0 : 2] : (S)P.omega;
   const S* d = (const S*)P.dinv + 12 * (int64_t)i;
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
@@ -214,6 +215,7 @@ __global__ void __launch_bounds__(kColThreads) k_cols_phase(const Phase P, int W
   const T* b = (const T*)P.b + c;
   T* y = (T*)P.y + c;
   const S* val = (const S*)P.val;
+  const S* wt = (const S*)P.wt;
   const int64_t o = (int64_t)i * W, o4 = 4 * (int64_t)i * W;
   auto norm = [](Cell<T> v) {
 #pragma unroll
@@ -230,7 +232,7 @@ __global__ void __launch_bounds__(kColThreads) k_cols_phase(const Phase P, int W
 #pragma unroll
         for (int q = 0; q < 3; ++q) axpy(s[q], val[t], ldc(x + j + q * W));
       }
-      const S wc = P.wt ? (S)P.wt[1] : S(1);
+      const S wc = wt ? wt[1] : S(1);
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
         if (P.type == PH_PROLONG) {
@@ -249,7 +251,7 @@ __global__ void __launch_bounds__(kColThreads) k_cols_phase(const Phase P, int W
         axpy(s, val[t], ldc(x + (int64_t)P.col[t] * W));
       if (P.type == PH_PROLONG1) {
         Cell<T> v = ldc(y + o);
-        axpy(v, P.wt ? (S)P.wt[1] : S(1), norm(s));
+        axpy(v, wt ? wt[1] : S(1), norm(s));
         s = v;
       }
       stc(y + o, s);
@@ -303,7 +305,7 @@ __global__ void __launch_bounds__(kColThreads) k_cols_phase(const Phase P, int W
       } else if (P.mode == 3) {
         axpy(s, S(-1), ldc(b + o));
       } else if (P.mode == 2) {
-        const S om = P.wt ? (S)(P.omega * P.wt[2]) : (S)P.omega;
+        const S om = wt ? wt[3] : (S)P.omega;
         const S d = ((const S*)P.sd)[i];
         axpy(s, S(-1), ldc(b + o));
         s = norm(s);

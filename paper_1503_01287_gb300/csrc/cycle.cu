@@ -90,12 +90,11 @@ __device__ __forceinline__ void rows_body(int nrows, const int* __restrict__ row
                                           const int* __restrict__ col,
                                           const V* __restrict__ val, int64_t nnzb, const T* x,
                                           const T* b, T* y, const T* __restrict__ dinv,
-                                          T omega, const double* __restrict__ wt, int warp,
+                                          T omega, const T* __restrict__ wt, int warp,
                                           int nwarps) {
   constexpr int RPW = 32 / G;
-  // relaxation: omega (Jacobi damping, 1 for Gauss-Seidel) times the level's
-  // learned multiplier (1 for the plain method)
-  if (MODE == kGS || MODE == kJacobi) omega = wt ? (T)((double)omega * wt[0]) : omega;
+  // relaxation: the level's step, weights included (Level::wt), else omega
+  if ((MODE == kGS || MODE == kJacobi) && wt) omega = wt[MODE == kGS ? 0 : 2];
   const int lane = threadIdx.x & 31;
   const int sub = lane / G, gl = lane & (G - 1);
   for (int base = warp * RPW; base < nrows; base += nwarps * RPW) {
@@ -105,12 +104,13 @@ __device__ __forceinline__ void rows_body(int nrows, const int* __restrict__ row
     T s0 = T(0), s1 = T(0), s2 = T(0);
     // operands of the row update that depend only on the row: loaded before the
     // row's blocks so that they are not on the critical path
-    T b0 = T(0), b1 = T(0), b2 = T(0), xi0 = T(0), xi1 = T(0), xi2 = T(0);
+    using End = RowEnd<T, G>;
+    T bi[End::N] = {}, xi[End::N] = {};
     if (active) {
       i = rows ? ldg(rows + g) : g;
-      if (MODE != kApply && gl == 0) {
-        VL<COH>::node(b, i, b0, b1, b2);
-        if (MODE != kResid) VL<COH>::node(x, i, xi0, xi1, xi2);
+      if (MODE != kApply && End::holds(gl)) {
+        End::template load<VL<COH>>(b, i, gl, bi);
+        if (MODE != kResid) End::template load<VL<COH>>(x, i, gl, xi);
       }
       const int a = ldg(rowptr + g), e = ldg(rowptr + g + 1);
       // U blocks per lane per step: all column indices of the step are loaded
@@ -152,31 +152,28 @@ __device__ __forceinline__ void rows_body(int nrows, const int* __restrict__ row
         }
       }
     }
+    T v[End::N];
+    End::sum(s0, s1, s2, gl, v);
+    if (MODE != kApply) {
 #pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) {
-      s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-      s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-      s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+      for (int q = 0; q < End::N; ++q) v[q] = bi[q] - v[q];
     }
-    if (!active || gl != 0) continue;
-    if (MODE == kApply) {
-      st3(y, i, s0, s1, s2);
-      continue;
+    if (MODE == kGS || MODE == kJacobi) {
+      T r0, r1, r2;
+      End::all(v, r0, r1, r2);
+      if (!active) continue;
+      if (End::holds(gl)) {
+#pragma unroll
+        for (int q = 0; q < End::N; ++q) {
+          T d[3];
+          End::load_dinv_row(dinv, i, gl, q, d);
+          v[q] = xi[q] + omega * (d[0] * r0 + d[1] * r1 + d[2] * r2);
+        }
+      }
+      End::template store<MODE != kGS>(y, i, gl, v);
+    } else if (active) {
+      End::template store<true>(y, i, gl, v);
     }
-    const T r0 = b0 - s0, r1 = b1 - s1, r2 = b2 - s2;
-    if (MODE == kResid) {
-      st3(y, i, r0, r1, r2);
-      continue;
-    }
-    const T* d = dinv + 12 * (int64_t)i;
-    T d0, d1, d2;
-    ld3(d, 0, d0, d1, d2);
-    const T c0 = d0 * r0 + d1 * r1 + d2 * r2;
-    ld3(d, 1, d0, d1, d2);
-    const T c1 = d0 * r0 + d1 * r1 + d2 * r2;
-    ld3(d, 2, d0, d1, d2);
-    const T c2 = d0 * r0 + d1 * r1 + d2 * r2;
-    st3(y, i, xi0 + omega * c0, xi1 + omega * c1, xi2 + omega * c2);
   }
 }
 
@@ -206,9 +203,9 @@ template <typename T, bool COH>
 __device__ __forceinline__ void prolong_body(int n, const int* __restrict__ prow,
                                              const int* __restrict__ pcol,
                                              const T* __restrict__ pval, const T* xc, T* x,
-                                             const double* __restrict__ wt, int tid, int nthr) {
+                                             const T* __restrict__ wt, int tid, int nthr) {
   // coarse-grid correction x += w_c P x_c (w_c = 1 for the plain method)
-  const T wc = wt ? (T)wt[1] : T(1);
+  const T wc = wt ? wt[1] : T(1);
   for (int i = tid; i < n; i += nthr) {
     T s0 = T(0), s1 = T(0), s2 = T(0);
     for (int q = prow[i]; q < prow[i + 1]; ++q) {
@@ -243,8 +240,8 @@ template <typename T, bool COH>
 __device__ __forceinline__ void prolong1_body(int n, const int* __restrict__ prow,
                                               const int* __restrict__ pcol,
                                               const T* __restrict__ pval, const T* xc, T* x,
-                                              const double* __restrict__ wt, int tid, int nthr) {
-  const T wc = wt ? (T)wt[1] : T(1);
+                                              const T* __restrict__ wt, int tid, int nthr) {
+  const T wc = wt ? wt[1] : T(1);
   for (int i = tid; i < n; i += nthr) {
     T s = T(0);
     for (int q = prow[i]; q < prow[i + 1]; ++q) s = fma(pval[q], VL<COH>::one(xc + pcol[q]), s);
@@ -317,8 +314,8 @@ __device__ __forceinline__ void prows_body(int np, const int* __restrict__ brow,
                                            const int* __restrict__ ccol,
                                            const T* __restrict__ cval, const T* u, const T* p,
                                            const T* g, T* yp, const T* __restrict__ sd, T omega,
-                                           const double* __restrict__ wt, int tid, int nthr) {
-  if (MODE == 2 && wt) omega = (T)((double)omega * wt[2]);
+                                           const T* __restrict__ wt, int tid, int nthr) {
+  if (MODE == 2 && wt) omega = wt[3];
   constexpr int L = kProwLanes;
   const int gl = tid & (L - 1);
   const unsigned gmask = ((1u << L) - 1u) << (threadIdx.x & 31 & ~(L - 1));
@@ -473,7 +470,7 @@ __device__ void dispatch_rows_v(const Phase& P, int warp, int nwarps) {
   const T* d = (const T*)P.dinv;
   const T om = (T)P.omega;
 #define AMG_ROWS_MODE(GG, MM)                                                                   \
-  rows_body<T, GG, MM, COH, V>(P.n, P.rows, P.rowptr, P.col, val, P.nnz, x, b, y, d, om, P.wt, \
+  rows_body<T, GG, MM, COH, V>(P.n, P.rows, P.rowptr, P.col, val, P.nnz, x, b, y, d, om, (const T*)P.wt, \
                                warp, nwarps)
 #define AMG_ROWS_G(GG)                              \
   switch (P.mode) {                                 \
@@ -515,7 +512,7 @@ __device__ __forceinline__ void exec_phase(const Phase& P, int tid, int nthr) {
                             nthr);
       break;
     case PH_PROLONG:
-      prolong_body<T, COH>(P.n, P.rowptr, P.col, (const T*)P.val, (const T*)P.x, (T*)P.y, P.wt,
+      prolong_body<T, COH>(P.n, P.rowptr, P.col, (const T*)P.val, (const T*)P.x, (T*)P.y, (const T*)P.wt,
                            tid, nthr);
       break;
     case PH_RESTRICT1:
@@ -523,7 +520,7 @@ __device__ __forceinline__ void exec_phase(const Phase& P, int tid, int nthr) {
                              nthr);
       break;
     case PH_PROLONG1:
-      prolong1_body<T, COH>(P.n, P.rowptr, P.col, (const T*)P.val, (const T*)P.x, (T*)P.y, P.wt,
+      prolong1_body<T, COH>(P.n, P.rowptr, P.col, (const T*)P.val, (const T*)P.x, (T*)P.y, (const T*)P.wt,
                             tid, nthr);
       break;
     case PH_COARSE:
@@ -540,7 +537,7 @@ __device__ __forceinline__ void exec_phase(const Phase& P, int tid, int nthr) {
 #define AMG_PROWS(MM)                                                                        \
   prows_body<T, MM, COH>(P.n, P.rowptr, P.col, (const T*)P.val, P.nnz, P.crow, P.ccol,      \
                          (const T*)P.cval, u, p, (const T*)P.b, (T*)P.y, (const T*)P.sd, om, \
-                         P.wt, tid, nthr)
+                         (const T*)P.wt, tid, nthr)
       if (P.mode == 0) AMG_PROWS(0);
       else if (P.mode == 1) AMG_PROWS(1);
       else if (P.mode == 2) AMG_PROWS(2);
@@ -580,18 +577,17 @@ __device__ __forceinline__ void exec_phase(const Phase& P, int tid, int nthr) {
 // writes guaranteed visible (the first colour of a sweep follows the
 // restriction that writes b).
 // One group of G lanes per stored row; each lane prefetches up to U blocks.
-// XNC: x is gathered through the read-only (L1-cached) path instead of L2 only.
 // Within one colour launch nothing that is gathered is written (rows of one
 // colour are not neighbours; a row reads its own x_i before writing it), and the
 // previous kernels' writes are visible after griddepcontrol.wait.
-template <typename T, int G, int U, typename V = T, bool XNC = false>
+template <typename T, int G, int U, typename V = T>
 __global__ void __launch_bounds__(256) k_gs_pdl(int nrows, const int* __restrict__ rows,
                                                 const int* __restrict__ rowptr,
                                                 const int* __restrict__ col,
                                                 const V* __restrict__ val, int64_t nnzb, T* x,
                                                 const T* __restrict__ b,
                                                 const T* __restrict__ dinv,
-                                                const double* __restrict__ wt) {
+                                                const T* __restrict__ wt) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int g = (blockIdx.x * blockDim.x + threadIdx.x) / G;
   const int gl = threadIdx.x & (G - 1);
@@ -624,19 +620,19 @@ __global__ void __launch_bounds__(256) k_gs_pdl(int nrows, const int* __restrict
     }
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const T om = wt ? (T)wt[0] : T(1);   // learned relaxation multiplier (1: plain)
+  const T om = wt ? wt[0] : T(1);   // learned relaxation multiplier (1: plain)
   T s0 = T(0), s1 = T(0), s2 = T(0);
   T xi0 = T(0), xi1 = T(0), xi2 = T(0);
   if (active) {
     if (gl == 0) {
       ld3(b, i, b0, b1, b2);
-      VL<!XNC>::node(x, i, xi0, xi1, xi2);
+      VL<true>::node(x, i, xi0, xi1, xi2);
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       if (j[u] < 0) continue;
       T x0, x1, x2;
-      VL<!XNC>::node(x, j[u], x0, x1, x2);
+      VL<true>::node(x, j[u], x0, x1, x2);
       s0 = fma(v[u][0], x0, s0); s0 = fma(v[u][1], x1, s0); s0 = fma(v[u][2], x2, s0);
       s1 = fma(v[u][3], x0, s1); s1 = fma(v[u][4], x1, s1); s1 = fma(v[u][5], x2, s1);
       s2 = fma(v[u][6], x0, s2); s2 = fma(v[u][7], x1, s2); s2 = fma(v[u][8], x2, s2);
@@ -645,7 +641,7 @@ __global__ void __launch_bounds__(256) k_gs_pdl(int nrows, const int* __restrict
     for (int k = a + gl + U * G; k < e; k += G) {
       const int jj = ldg(col + k);
       T x0, x1, x2;
-      VL<!XNC>::node(x, jj, x0, x1, x2);
+      VL<true>::node(x, jj, x0, x1, x2);
       const V* vv = val + k;
       s0 = fma(ldg_v<T>(vv), x0, s0);
       s0 = fma(ldg_v<T>(vv + nnzb), x1, s0);
@@ -670,27 +666,129 @@ __global__ void __launch_bounds__(256) k_gs_pdl(int nrows, const int* __restrict
       xi1 + om * (d[3] * r0 + d[4] * r1 + d[5] * r2), xi2 + om * (d[6] * r0 + d[7] * r1 + d[8] * r2));
 }
 
-template <typename T, int G, typename V, bool XNC>
-void launch_gs_pdl_x(const Phase& P, cudaStream_t s) {
-  constexpr int U = (sizeof(T) == 8) ? (G >= 16 ? 2 : 3) : (G >= 16 ? 3 : 4);
+// The same in FP64, ending with one component a lane (row_sum3, spread3): each FP64
+// instruction takes a warp about 19 cycles of the SM's FP64 unit, and the reduction and the
+// update then take 12 a row group where one lane's three components take 30 (G = 32).
+template <int G, int U>
+__global__ void __launch_bounds__(256) k_gs_pdl64(int nrows, const int* __restrict__ rows,
+                                                const int* __restrict__ rowptr,
+                                                const int* __restrict__ col,
+                                                const double* __restrict__ val, int64_t nnzb, double* x,
+                                                const double* __restrict__ b,
+                                                const double* __restrict__ dinv,
+                                                const double* __restrict__ wt) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int g = (blockIdx.x * blockDim.x + threadIdx.x) / G;
+  const int gl = threadIdx.x & (G - 1);
+  const bool active = g < nrows;
+  int i = 0, a = 0, e = 0;
+  int j[U];
+  double v[U][9];
+  const bool mine = active && holds_component<G>(gl);
+  const int comp = component_of<G>(gl);
+  double d0 = 0.0, d1 = 0.0, d2 = 0.0;
+#pragma unroll
+  for (int u = 0; u < U; ++u) j[u] = -1;
+  if (active) {
+    i = ldg(rows + g);
+    a = ldg(rowptr + g);
+    e = ldg(rowptr + g + 1);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int k = a + gl + u * G;
+      if (k < e) {
+        j[u] = __ldcs(col + k);
+#pragma unroll
+        for (int q = 0; q < 9; ++q) v[u][q] = __ldcs(val + q * nnzb + k);
+      }
+    }
+    if (mine) ld3(dinv + 12 * (int64_t)i, comp, d0, d1, d2);
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const double om = wt ? wt[0] : 1.0;   // learned relaxation multiplier (1: plain)
+  double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+  double bi = 0.0, xi = 0.0;
+  if (active) {
+    if (mine) {
+      bi = ldg(b + 4 * (int64_t)i + comp);
+      xi = VL<true>::one(x + 4 * (int64_t)i + comp);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (j[u] < 0) continue;
+      double x0, x1, x2;
+      VL<true>::node(x, j[u], x0, x1, x2);
+      s0 = fma(v[u][0], x0, s0); s0 = fma(v[u][1], x1, s0); s0 = fma(v[u][2], x2, s0);
+      s1 = fma(v[u][3], x0, s1); s1 = fma(v[u][4], x1, s1); s1 = fma(v[u][5], x2, s1);
+      s2 = fma(v[u][6], x0, s2); s2 = fma(v[u][7], x1, s2); s2 = fma(v[u][8], x2, s2);
+    }
+    // blocks beyond the prefetched U per lane
+    for (int k = a + gl + U * G; k < e; k += G) {
+      const int jj = ldg(col + k);
+      double x0, x1, x2;
+      VL<true>::node(x, jj, x0, x1, x2);
+      const double* vv = val + k;
+      s0 = fma(ldg(vv), x0, s0);
+      s0 = fma(ldg(vv + nnzb), x1, s0);
+      s0 = fma(ldg(vv + 2 * nnzb), x2, s0);
+      s1 = fma(ldg(vv + 3 * nnzb), x0, s1);
+      s1 = fma(ldg(vv + 4 * nnzb), x1, s1);
+      s1 = fma(ldg(vv + 5 * nnzb), x2, s1);
+      s2 = fma(ldg(vv + 6 * nnzb), x0, s2);
+      s2 = fma(ldg(vv + 7 * nnzb), x1, s2);
+      s2 = fma(ldg(vv + 8 * nnzb), x2, s2);
+    }
+  }
+  double r0, r1, r2;
+  spread3<G>(bi - row_sum3<G>(s0, s1, s2, gl), threadIdx.x & 31, r0, r1, r2);
+  if (mine) x[4 * (int64_t)i + comp] = xi + om * (d0 * r0 + d1 * r1 + d2 * r2);
+}
+
+// Lanes per block row and threads per CTA of the colour kernels, from the mean rows of a
+// colour (sweeps timed on levels of 117 to 274,625 nodes, all G in 4..32 and 32..256 threads).
+// FP32: the widest group whose lanes still fit the chip at once (72 registers: 3 CTAs of 256
+//   an SM, 117k lanes), else 8: 16^3 level 0 (2,567 rows) 28 / 36 / 44 us with 32 / 16 / 8
+//   lanes, 24^3 (7,073 rows) 62 / 51 / 57, 32^3 (19,616 rows) 144 / 100 / 94.
+// FP64: the chip's FP64 issue limits it, so 16 lanes once a colour fills the SMs, and one
+//   warp a CTA, so that the rows of a small colour go to as many SMs as they can: 16^3 level
+//   1 (180 rows) 112 us with CTAs of 32 threads, 144 with 256 (23 CTAs, whose 8 rows share an
+//   SM's FP64 unit), level 0 (2,567 rows) 97 / 108 with 16 / 32 lanes, 24^3 151 / 206.
+inline int gs_lanes(bool f32, double rows) {
+  if (!f32) return rows * 32 <= 36864 ? 32 : 16;
+  return rows * 32 <= 117000 ? 32 : (rows * 16 <= 140000 ? 16 : 8);
+}
+template <typename T, int G>
+constexpr int kGsThreads = sizeof(T) == 8 ? 32 : (G <= 8 ? 128 : 256);
+
+template <typename T, int G, typename V = T>
+void launch_gs_pdl(const Phase& P, cudaStream_t s) {
+  constexpr int threads = kGsThreads<T, G>;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(((int64_t)P.n * G + 255) / 256));
-  cfg.blockDim = dim3(256);
+  cfg.gridDim = dim3((unsigned)(((int64_t)P.n * G + threads - 1) / threads));
+  cfg.blockDim = dim3(threads);
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  AMG_CUDA(cudaLaunchKernelEx(&cfg, k_gs_pdl<T, G, U, V, XNC>, P.n, P.rows, P.rowptr, P.col,
-                              (const V*)P.val, P.nnz, (T*)P.y, (const T*)P.b,
-                              (const T*)P.dinv, P.wt));
+  if constexpr (sizeof(T) == 8)
+    AMG_CUDA(cudaLaunchKernelEx(&cfg, k_gs_pdl64<G, (G >= 16 ? 2 : 3)>, P.n, P.rows, P.rowptr,
+                                P.col, (const double*)P.val, P.nnz, (double*)P.y,
+                                (const double*)P.b, (const double*)P.dinv,
+                                (const double*)P.wt));
+  else
+    AMG_CUDA(cudaLaunchKernelEx(&cfg, k_gs_pdl<T, G, (G >= 16 ? 3 : 4), V>, P.n, P.rows,
+                                P.rowptr, P.col, (const V*)P.val, P.nnz, (T*)P.y,
+                                (const T*)P.b, (const T*)P.dinv, (const T*)P.wt));
 }
 
-template <typename T, int G, typename V = T>
-void launch_gs_pdl(const Phase& P, cudaStream_t s) {
-  if (P.xnc) launch_gs_pdl_x<T, G, V, true>(P, s);
-  else launch_gs_pdl_x<T, G, V, false>(P, s);
+// Threads a CTA of a row kernel with `lanes` lanes in all: 256, or fewer (a power of two,
+// one warp at least) where 256 would leave SMs without a CTA.
+inline int row_threads(int64_t lanes) {
+  int t = 256;
+  while (t > 32 && lanes <= (int64_t)(t / 2) * 152) t /= 2;
+  return t;
 }
 
 // Multicolour Gauss-Seidel sweep of one small level as ONE launch: a single CTA,
@@ -809,7 +907,7 @@ __global__ void __launch_bounds__(kGsClThreads, 1)
                  const int* __restrict__ rows, const int* __restrict__ rowptr,
                  const int* __restrict__ col, const V* __restrict__ val, int64_t nnzb, T* x,
                  const T* __restrict__ b, const T* __restrict__ dinv,
-                 const double* __restrict__ wt, int* __restrict__ err) {
+                 const T* __restrict__ wt, int* __restrict__ err) {
   extern __shared__ __align__(16) unsigned char gs_smem[];
   uint64_t* bars = reinterpret_cast<uint64_t*>(gs_smem);
   T* xs = reinterpret_cast<T*>(gs_smem + kGsClBarBytes);
@@ -824,7 +922,7 @@ __global__ void __launch_bounds__(kGsClThreads, 1)
   const int warp = (rank * (int)blockDim.x + (int)threadIdx.x) >> 5;
   const int nwarps = (cs * (int)blockDim.x) >> 5;
   const int stride = nwarps * RPW;
-  const T om = wt ? (T)wt[0] : T(1);   // learned relaxation multiplier (1: plain)
+  const T om = wt ? wt[0] : T(1);   // learned relaxation multiplier (1: plain)
   auto colour_of = [&](int q) { return post ? ncolours - 1 - q : q; };
   auto colour_bytes = [&](int q) {
     const int c = colour_of(q);
@@ -1054,7 +1152,7 @@ void launch_gs_cluster_g(const Level& lv, int cs, bool post, bool x_zero, const 
   if (cs == 1) {
     k_gs_cluster<T, G, U, V, true><<<1, kGsClThreads, (size_t)gs_cl_smem<T>(lv.n), s>>>(
         lv.n, lv.ncolours, cp, (int)post, (int)x_zero, lv.k_rows(), lv.k_rowptr(), lv.k_col(),
-        val, lv.nnzb, x, b, dinv, (const double*)lv.wt, err);
+        val, lv.nnzb, x, b, dinv, lv.template steps<T>(), err);
     return;
   }
   auto kern = k_gs_cluster<T, G, U, V, false>;
@@ -1072,7 +1170,7 @@ void launch_gs_cluster_g(const Level& lv, int cs, bool post, bool x_zero, const 
   cfg.numAttrs = 1;
   AMG_CUDA(cudaLaunchKernelEx(&cfg, kern, lv.n, lv.ncolours, cp, (int)post, (int)x_zero,
                               lv.k_rows(), lv.k_rowptr(), lv.k_col(), val, lv.nnzb, x, b, dinv,
-                              (const double*)lv.wt, err));
+                              lv.template steps<T>(), err));
 }
 
 template <typename T, typename V>
@@ -1178,18 +1276,12 @@ __global__ void __launch_bounds__(256) k_apply_pair(int nrows, const int* __rest
         }
       }
     }
-#pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) {
-      float T = __shfl_xor_sync(0xffffffffu, S0, o), t = __shfl_xor_sync(0xffffffffu, s0, o);
-      pair_add(S0, s0, T, t);
-      T = __shfl_xor_sync(0xffffffffu, S1, o); t = __shfl_xor_sync(0xffffffffu, s1, o);
-      pair_add(S1, s1, T, t);
-      T = __shfl_xor_sync(0xffffffffu, S2, o); t = __shfl_xor_sync(0xffffffffu, s2, o);
-      pair_add(S2, s2, T, t);
-    }
-    if (!active || gl != 0) continue;
-    const int i = rows ? __ldg(rows + g) : g;
-    st3(y, i, (double)S0 + (double)s0, (double)S1 + (double)s1, (double)S2 + (double)s2);
+    const float2 s = row_sum3_pair<G>(make_float2(S0, s0), make_float2(S1, s1),
+                                      make_float2(S2, s2), gl);
+    if (!active) continue;
+    const int64_t o = 4 * (int64_t)(rows ? __ldg(rows + g) : g);
+    if (holds_component<G>(gl)) y[o + component_of<G>(gl)] = (double)s.x + (double)s.y;
+    else if (gl == G - 1) y[o + 3] = 0.0;
   }
 }
 
@@ -1273,16 +1365,19 @@ __global__ void __launch_bounds__(256) k_rows(const Phase P) {
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
   rows_body<T, G, MODE, false, V>(P.n, P.rows, P.rowptr, P.col, (const V*)P.val, P.nnz,
                                (const T*)P.x, (const T*)P.b, (T*)P.y, (const T*)P.dinv,
-                               (T)P.omega, P.wt, tid >> 5, (gridDim.x * blockDim.x) >> 5);
+                               (T)P.omega, (const T*)P.wt, tid >> 5, (gridDim.x * blockDim.x) >> 5);
 }
 
 template <typename T, int G, typename V>
-void launch_rows_mode(const Phase& P, int grid, cudaStream_t s) {
+void launch_rows_mode(const Phase& P, cudaStream_t s) {
+  // one group of G lanes per row
+  const int t = row_threads((int64_t)P.n * G);
+  const int grid = (int)(((int64_t)P.n * G + t - 1) / t);
   switch (P.mode) {
-    case kApply: k_rows<T, G, kApply, V><<<grid, 256, 0, s>>>(P); break;
-    case kResid: k_rows<T, G, kResid, V><<<grid, 256, 0, s>>>(P); break;
-    case kGS: k_rows<T, G, kGS, V><<<grid, 256, 0, s>>>(P); break;
-    default: k_rows<T, G, kJacobi, V><<<grid, 256, 0, s>>>(P); break;
+    case kApply: k_rows<T, G, kApply, V><<<grid, t, 0, s>>>(P); break;
+    case kResid: k_rows<T, G, kResid, V><<<grid, t, 0, s>>>(P); break;
+    case kGS: k_rows<T, G, kGS, V><<<grid, t, 0, s>>>(P); break;
+    default: k_rows<T, G, kJacobi, V><<<grid, t, 0, s>>>(P); break;
   }
 }
 
@@ -1391,7 +1486,7 @@ __global__ void __launch_bounds__(256) k_gs_stream(int nrows, const int* __restr
                                                    const T* __restrict__ val, int64_t nnzb, T* x,
                                                    const T* __restrict__ b,
                                                    const T* __restrict__ dinv,
-                                                   const double* __restrict__ wt) {
+                                                   const T* __restrict__ wt) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   constexpr int R = 32 / G;
   const int lane = threadIdx.x & 31, sub = lane / G, gl = lane & (G - 1);
@@ -1401,7 +1496,7 @@ __global__ void __launch_bounds__(256) k_gs_stream(int nrows, const int* __restr
   int g = warp * R + sub;
   gs_set_load(A, g, nrows, rows, rowptr, col, val, nnzb, dinv, gl);
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const T om = wt ? (T)wt[0] : T(1);   // learned relaxation multiplier (1: plain)
+  const T om = wt ? wt[0] : T(1);   // learned relaxation multiplier (1: plain)
   // rows of one colour are not neighbours: the x gathers read only earlier
   // colours' values (L2-coherent loads all the same, the kernel writes x)
   for (int base = warp * R; base < nrows; base += 2 * step) {
@@ -1435,7 +1530,7 @@ void launch_gs_stream(const Phase& P, cudaStream_t s) {
   cfg.numAttrs = 1;
   AMG_CUDA(cudaLaunchKernelEx(&cfg, k_gs_stream<T, G, U>, P.n, P.rows, P.rowptr, P.col,
                               (const T*)P.val, P.nnz, (T*)P.y, (const T*)P.b,
-                              (const T*)P.dinv, P.wt));
+                              (const T*)P.dinv, (const T*)P.wt));
 }
 
 // ------------------------------------------------- TMA-staged colour kernel (FP32)
@@ -1483,14 +1578,14 @@ __device__ __forceinline__ bool tma_wait(uint32_t bar) {
   return false;
 }
 
-template <int G, bool XNC>
+template <int G>
 __global__ void __launch_bounds__(256) k_gs_tma(int nrows, const int* __restrict__ rows,
                                                 const int* __restrict__ rowptr,
                                                 const int* __restrict__ col,
                                                 const float* __restrict__ val, int64_t nnzb,
                                                 float* x, const float* __restrict__ b,
                                                 const float* __restrict__ dinv,
-                                                const double* __restrict__ wt,
+                                                const float* __restrict__ wt,
                                                 int* __restrict__ err) {
   extern __shared__ __align__(128) float tma_sm[];
   __shared__ __align__(8) uint64_t tbar;
@@ -1570,7 +1665,7 @@ __global__ void __launch_bounds__(256) k_gs_tma(int nrows, const int* __restrict
   if (active) {
     if (gl == 0) {
       ld3(b, i, b0, b1, b2);
-      VL<!XNC>::node(x, i, xi0, xi1, xi2);
+      VL<true>::node(x, i, xi0, xi1, xi2);
     }
     int off[10];
 #pragma unroll
@@ -1591,7 +1686,7 @@ __global__ void __launch_bounds__(256) k_gs_tma(int nrows, const int* __restrict
         for (int q = 0; q < 9; ++q) v[q] = __ldg(val + q * nnzb + k);
       }
       float x0, x1, x2;
-      VL<!XNC>::node(x, jj, x0, x1, x2);
+      VL<true>::node(x, jj, x0, x1, x2);
       s0 = fmaf(v[0], x0, s0); s0 = fmaf(v[1], x1, s0); s0 = fmaf(v[2], x2, s0);
       s1 = fmaf(v[3], x0, s1); s1 = fmaf(v[4], x1, s1); s1 = fmaf(v[5], x2, s1);
       s2 = fmaf(v[6], x0, s2); s2 = fmaf(v[7], x1, s2); s2 = fmaf(v[8], x2, s2);
@@ -1609,11 +1704,11 @@ __global__ void __launch_bounds__(256) k_gs_tma(int nrows, const int* __restrict
       xi1 + om * (d[3] * r0 + d[4] * r1 + d[5] * r2), xi2 + om * (d[6] * r0 + d[7] * r1 + d[8] * r2));
 }
 
-template <int G, bool XNC>
-void launch_gs_tma_x(const Phase& P, cudaStream_t s) {
+template <int G>
+void launch_gs_tma(const Phase& P, cudaStream_t s) {
   static bool attr = false;
   if (!attr) {
-    AMG_CUDA(cudaFuncSetAttribute(k_gs_tma<G, XNC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    AMG_CUDA(cudaFuncSetAttribute(k_gs_tma<G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   tma_smem<G>()));
     attr = true;
   }
@@ -1627,15 +1722,9 @@ void launch_gs_tma_x(const Phase& P, cudaStream_t s) {
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  AMG_CUDA(cudaLaunchKernelEx(&cfg, k_gs_tma<G, XNC>, P.n, P.rows, P.rowptr, P.col,
+  AMG_CUDA(cudaLaunchKernelEx(&cfg, k_gs_tma<G>, P.n, P.rows, P.rowptr, P.col,
                               (const float*)P.val, P.nnz, (float*)P.y, (const float*)P.b,
-                              (const float*)P.dinv, P.wt, P.err));
-}
-
-template <int G>
-void launch_gs_tma(const Phase& P, cudaStream_t s) {
-  if (P.xnc) launch_gs_tma_x<G, true>(P, s);
-  else launch_gs_tma_x<G, false>(P, s);
+                              (const float*)P.dinv, (const float*)P.wt, P.err));
 }
 
 template <typename T, typename V>
@@ -1668,13 +1757,11 @@ void launch_rows_v(const Phase& P, cudaStream_t s, bool pdl) {
       default: launch_gs_pdl<T, 32, V>(P, s); return;
     }
   }
-  // one group of G lanes per row: nrows * G threads
-  const int grid = (int)(((int64_t)P.n * P.G + 255) / 256);
   switch (P.G) {
-    case 4: launch_rows_mode<T, 4, V>(P, grid, s); break;
-    case 8: launch_rows_mode<T, 8, V>(P, grid, s); break;
-    case 16: launch_rows_mode<T, 16, V>(P, grid, s); break;
-    default: launch_rows_mode<T, 32, V>(P, grid, s); break;
+    case 4: launch_rows_mode<T, 4, V>(P, s); break;
+    case 8: launch_rows_mode<T, 8, V>(P, s); break;
+    case 16: launch_rows_mode<T, 16, V>(P, s); break;
+    default: launch_rows_mode<T, 32, V>(P, s); break;
   }
 }
 
@@ -1866,13 +1953,12 @@ struct Emit {
   void rows(int mode, const Level& lv, int G, int first, int nrows, const T* val, const T* x,
             const T* b, T* y, const T* dinv, T omega) {
     Phase P = blank(PH_ROWS);
-    P.wt = (mode == kGS || mode == kJacobi) ? lv.wt : nullptr;
+    P.wt = (mode == kGS || mode == kJacobi) ? lv.template steps<T>() : nullptr;
     const int* order = lv.k_rows();
     P.mode = mode; P.G = G; P.n = nrows; P.rows = order ? order + first : nullptr;
     P.rowptr = lv.k_rowptr() + first; P.col = lv.k_col();
     P.val = val; P.nnz = lv.nnzb; P.x = x; P.b = b; P.y = y; P.dinv = dinv; P.omega = omega;
     P.sctas = mode == kGS ? lv.gs_stream : 0;
-    P.xnc = mode == kGS ? lv.gs_xnc : 0;
     P.tma = mode == kGS ? lv.gs_tma : 0;
     P.err = h->flag.p;
     if (sizeof(T) == 4 && lv.val16.p && (const void*)val == (const void*)lv.val32.p) {
@@ -1913,7 +1999,7 @@ struct Emit {
     put(P, n);
   }
   void transfer(int type, int n, const int* row, const int* col, const T* val, const T* src,
-                T* dst, const double* wt = nullptr) {
+                T* dst, const T* wt = nullptr) {
     Phase P = blank(type);
     P.n = n; P.rowptr = row; P.col = col; P.val = val; P.x = src; P.y = dst; P.wt = wt;
     put(P, n);
@@ -1973,7 +2059,7 @@ struct Emit {
     P.val = LvVec<T>::bval(lv); P.nnz = lv.b_nnz; P.crow = lv.c_rowptr; P.ccol = lv.c_col;
     P.cval = LvVec<T>::cval(lv); P.x = u; P.p = p; P.b = g; P.y = yp;
     P.sd = LvVec<T>::schur(lv); P.omega = (double)omega;
-    P.wt = mode == 2 ? lv.wt : nullptr;
+    P.wt = mode == 2 ? lv.template steps<T>() : nullptr;
     put(P, lv.np, kProwLanes);
   }
 };
@@ -2125,10 +2211,10 @@ template <typename T>
 void e_prolong(Emit<T>& e, amg_handle* h, int l, const T* xc, T* x) {
   Level& lv = *h->L[l];
   Level& nx = *h->L[l + 1];
-  e.transfer(PH_PROLONG, lv.n, lv.p_rowptr, lv.p_col, LvVec<T>::pval(lv), xc, x, lv.wt);
+  e.transfer(PH_PROLONG, lv.n, lv.p_rowptr, lv.p_col, LvVec<T>::pval(lv), xc, x, lv.template steps<T>());
   if (h->saddle && lv.np > 0)
     e.transfer(PH_PROLONG1, lv.np, lv.h_rowptr, lv.h_col, LvVec<T>::hval(lv), xc + 4 * nx.n,
-               x + 4 * lv.n, lv.wt);
+               x + 4 * lv.n, lv.template steps<T>());
 }
 
 template <typename T>
@@ -2475,6 +2561,8 @@ void autotune_levels(amg_handle* h) {
     return ms;
   };
   const bool f32 = h->opt.precision == AMG_FP32;
+  for (auto& lv : h->L)
+    if (lv->ncolours > 0) lv->group_gs = gs_lanes(f32, (double)lv->n / lv->ncolours);
   // levels that run as one stored matrix keep the default lanes per row
   const size_t nl = h->map_from >= 0 ? std::max(h->map_from, 1) : h->L.size();
   for (size_t l = 0; l < nl; ++l) {
@@ -2528,35 +2616,9 @@ void autotune_levels(amg_handle* h) {
     if (lv.ncolours == 0 || h->saddle || h->opt.smoother != AMG_SMOOTHER_GS ||
         h->map_from == 0)
       continue;
-    best = 0;
-    best_ms = 1e30f;
-    for (int G : {4, 8, 16, 32}) {
-      lv.group_gs = G;
-      for (int r = 0; r < 3; ++r) {
-        if (r == 1) AMG_CUDA(cudaEventRecord(e0, s));
-        if (f32) level_smooth<float>(h, (int)l, lv.x32.p, lv.b32.p, false, false);
-        else level_smooth<double>(h, (int)l, lv.x64.p, lv.b64.p, false, false);
-      }
-      const float ms = elapsed();
-      if (ms < best_ms) { best_ms = ms; best = G; }
-    }
-    lv.group_gs = best;
     lv.gs_stream = 0;
-    // the colour kernel's x gathers through L1 or L2 only: the faster
-    {
-      lv.gs_xnc = 0;
-      float t_l2 = 0.f, t_l1 = 0.f;
-      for (int xnc : {0, 1}) {
-        lv.gs_xnc = xnc;
-        for (int r = 0; r < 7; ++r) {
-          if (r == 2) AMG_CUDA(cudaEventRecord(e0, s));
-          if (f32) level_smooth<float>(h, (int)l, lv.x32.p, lv.b32.p, false, false);
-          else level_smooth<double>(h, (int)l, lv.x64.p, lv.b64.p, false, false);
-        }
-        (xnc ? t_l1 : t_l2) = elapsed();
-      }
-      lv.gs_xnc = t_l1 < t_l2 ? 1 : 0;
-    }
+    if (h->map_from >= 0) continue;   // the other sweep kernels below were slower on every
+                                      // level that the stored matrix leaves to the chain
     auto sweep_ms = [&]() {
       for (int r = 0; r < 7; ++r) {
         if (r == 2) AMG_CUDA(cudaEventRecord(e0, s));

@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(kFlowThreads)
     k_gs_flow(int nchunks, const int* __restrict__ chunk, const int* __restrict__ rows,
               const int* __restrict__ rowptr, const unsigned* __restrict__ fcol,
               const T* __restrict__ val, int64_t nnzb, T* x, const T* __restrict__ b,
-              const T* __restrict__ dinv, const double* __restrict__ wt,
+              const T* __restrict__ dinv, const T* __restrict__ wt,
               unsigned long long* xt, unsigned* state, int reverse, int* err) {
   const int lane = threadIdx.x & 31;
   const int sub = lane / G, gl = lane & (G - 1);
@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(kFlowThreads)
   const int nwarps = (int)((gridDim.x * blockDim.x) >> 5);
   const unsigned ep = flow_ld_relaxed(state) + 1u;
   const unsigned wbit = reverse ? kHigherBit : kLowerBit;
-  const T om = wt ? (T)wt[0] : T(1);   // learned relaxation multiplier (1: plain)
+  const T om = wt ? wt[0] : T(1);   // learned relaxation multiplier (1: plain)
   int spins = 0;
   for (int p = warp; p < nchunks; p += nwarps) {
     const int q = reverse ? nchunks - 1 - p : p;
@@ -407,7 +407,7 @@ void launch_gs_flow(amg_handle* h, Level& lv, T* x, const T* b, const T* val, co
   const int* rows = lv.colour_rows.p;
   const int* rowptr = lv.srowptr.p;
   const unsigned* fcol = lv.fcol.p;
-  const double* wt = lv.wt;
+  const T* wt = lv.template steps<T>();
   const int rev = reverse ? 1 : 0;
   switch (lv.flow) {
 #define AMG_FLOW_LAUNCH(GG)                                                                   \

@@ -256,14 +256,32 @@ void compute_level_features(amg_handle* h, int l, double* out) {
   level_features_from(h, acc, l, out);
 }
 
+void upload_weights(amg_handle* h, const std::vector<double>& w) {
+  std::vector<double> s(w);
+  std::vector<float> f(w.size());
+  for (size_t l = 0; 4 * l < w.size(); ++l) {
+    s[4 * l + 2] = h->opt.omega * w[4 * l];
+    s[4 * l + 3] = h->opt.omega_p * w[4 * l + 2];
+    f[4 * l] = (float)w[4 * l];
+    f[4 * l + 1] = (float)w[4 * l + 1];
+    f[4 * l + 2] = (float)((double)(float)h->opt.omega * w[4 * l]);
+    f[4 * l + 3] = (float)((double)(float)h->opt.omega_p * w[4 * l + 2]);
+  }
+  AMG_CUDA(cudaMemcpyAsync(h->wts.p, w.data(), w.size() * sizeof(double), cudaMemcpyHostToDevice,
+                           h->stream));
+  AMG_CUDA(cudaMemcpyAsync(h->steps.p, s.data(), s.size() * sizeof(double),
+                           cudaMemcpyHostToDevice, h->stream));
+  AMG_CUDA(cudaMemcpyAsync(h->steps32.p, f.data(), f.size() * sizeof(float),
+                           cudaMemcpyHostToDevice, h->stream));
+  AMG_CUDA(cudaStreamSynchronize(h->stream));
+}
+
 void set_level_weights(amg_handle* h, const double* w, int n) {
   const int nl = (int)h->L.size();
   std::vector<double> v(4 * (size_t)nl, 1.0);
   for (int l = 0; l < nl && l < n; ++l)
     for (int e = 0; e < 3; ++e) v[4 * l + e] = w[3 * l + e];
-  AMG_CUDA(cudaMemcpyAsync(h->wts.p, v.data(), v.size() * sizeof(double), cudaMemcpyHostToDevice,
-                           h->stream));
-  AMG_CUDA(cudaStreamSynchronize(h->stream));
+  upload_weights(h, v);
   map_build(h, v.data());   // the stored coarse cycle holds the weights
 }
 
@@ -276,9 +294,7 @@ void set_weights(amg_handle* h, const double* w3) {
     w[4 * l + 2] = w3[2];
     w[4 * l + 3] = 1.0;
   }
-  AMG_CUDA(cudaMemcpyAsync(h->wts.p, w.data(), w.size() * sizeof(double), cudaMemcpyHostToDevice,
-                           h->stream));
-  AMG_CUDA(cudaStreamSynchronize(h->stream));
+  upload_weights(h, w);
   map_build(h, w.data());
 }
 

@@ -39,11 +39,10 @@ struct Phase {
   const double* X;
   int m, n3;
   double omega;
-  const double* wt;       // the level's learned weights (null: plain method)
+  const void* wt;         // the level's steps, weights included (null: omega, 1)
   int vbf;                // PH_ROWS: values stored as BF16 (FP32 arithmetic)
   int sctas;              // PH_ROWS, Gauss-Seidel: CTAs per SM of the streaming colour
                           // kernel (0: one group of lanes per row, k_gs_pdl)
-  int xnc;                // PH_ROWS, Gauss-Seidel (k_gs_pdl): x through the L1 path
   int tma;                // PH_ROWS, Gauss-Seidel, FP32: the TMA-staged colour kernel
   int* err;               // the handle's error word (bounded waits that gave up)
   const long long* off;   // PH_VANKA: offsets of the patch inverses

@@ -1882,15 +1882,22 @@ void build_hierarchy(amg_handle* h, const amg_matrix* m, const int32_t* tags) {
   }
   for (size_t l = 0; l < h->L.size(); ++l) finish_level(h, *h->L[l], l + 1 == h->L.size());
   // learned weights start at the plain method's (all 1)
-  h->wts.alloc(4 * h->L.size());
-  launch_fill(h->wts, 1.0, 4 * (int64_t)h->L.size(), s, h);
-  for (size_t l = 0; l < h->L.size(); ++l) h->L[l]->wt = h->wts.p + 4 * l;
+  const size_t nw = 4 * h->L.size();
+  h->wts.alloc(nw);
+  h->steps.alloc(nw);
+  h->steps32.alloc(nw);
+  const std::vector<double> plain(nw, 1.0);
+  upload_weights(h, plain);
+  for (size_t l = 0; l < h->L.size(); ++l) {
+    h->L[l]->wt = h->steps.p + 4 * l;
+    h->L[l]->wt32 = h->steps32.p + 4 * l;
+  }
   factor_coarsest(h);
   if (h->saddle && h->opt.smoother == AMG_SMOOTHER_BS) bs_setup(h);
   if (h->saddle && h->opt.smoother == AMG_SMOOTHER_VANKA) vanka_setup(h);
   map_plan(h);
   autotune_levels(h);
-  map_build(h, std::vector<double>(4 * h->L.size(), 1.0).data());
+  map_build(h, plain.data());
   AMG_CUDA(cudaStreamSynchronize(s));
 }
 
