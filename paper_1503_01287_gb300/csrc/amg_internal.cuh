@@ -208,6 +208,16 @@ struct BatchLevel {
   int tile_gs = 0;     // tile of the multi-right-hand-side colour kernel
 };
 
+// The cycle from level `from` down (from x = 0) as an m x m matrix, row-major with rows ld
+// apart, in the cycle's precision (from = -1: off).
+struct CoarseMap {
+  int from = -1;
+  int m = 0, ld = 0;
+  DBuf<float> m32;
+  DBuf<double> m64;
+  std::vector<double> w;   // the level weights that it was built with
+};
+
 }  // namespace amgp2
 
 struct amg_handle {
@@ -255,13 +265,10 @@ struct amg_handle {
   amgp2::DBuf<unsigned char> full_ph32, full_ph64;
   int full_n32 = 0, full_n64 = 0;
   amgp2::DBuf<unsigned> grid_bar;
-  // the cycle from level map_from down as one stored matrix (coarse_map.cu; -1: off),
-  // map_m x map_m row-major with rows map_ld apart, in the cycle's precision
-  int map_from = -1;
-  int map_m = 0, map_ld = 0;
-  amgp2::DBuf<float> map32;
-  amgp2::DBuf<double> map64;
-  std::vector<double> map_w;         // the weights that it was built with
+  // the cycle from a level down as one stored matrix (coarse_map.cu), and a smaller one
+  // for batched solves where that one is too large for 16 right-hand sides
+  amgp2::CoarseMap map, bmap;
+  const amgp2::CoarseMap* batch_map = nullptr;   // of the two, for the batched cycle
   // batched (multi-right-hand-side) solves
   std::vector<amgp2::BatchLevel> B;
   amgp2::DBuf<double> mb, mx, mr, mz, mp, mq, mro, bred, bscal;
@@ -317,13 +324,21 @@ void autotune_levels(amg_handle* h);
 void set_subcycle(amg_handle* h, int from);
 
 // coarse_map.cu: the cycle below a level as one stored matrix
-// picks the level and allocates the matrix (before autotune_levels)
+// picks the level of h->map and allocates the matrix (before autotune_levels)
 void map_plan(amg_handle* h);
-// fills the matrix for the level weights w (host, 4 a level); again when they changed
+// the map of the batched solves: h->map, or h->bmap planned here; null: none.  Filled.
+const CoarseMap* map_batch(amg_handle* h);
+// fills the maps for the level weights w (host, 4 a level); again when they changed
 void map_build(amg_handle* h, const double* w);
-// x = (the cycle from level map_from) b, vectors of that level in the padded layout
+// x = (the cycle from level map.from) b, vectors of that level in the padded layout
 template <typename T, typename IO>
 void map_apply(amg_handle* h, const IO* b, IO* x);
+// the same for kRhs vectors at once, FP32, in planes of four vectors: entry k of vector r
+// at ((r / 4) m + k) 4 + r % 4
+void map_apply_m(amg_handle* h, const CoarseMap& M, const float* b, float* x);
+__device__ __forceinline__ int64_t map_plane(int m, int k, int r) {
+  return ((int64_t)(r >> 2) * m + k) * 4 + (r & 3);
+}
 
 // krylov (krylov.cu)
 int solve_device(amg_handle* h, const double* b, double* x, double tol, amg_stats* st);

@@ -149,11 +149,12 @@ __global__ void __launch_bounds__(256) k_apply_pair_m(int nrows, const int* __re
       (double)S2 + (double)s2);
 }
 
-// bc_(I,r) = sum_t w_t v_(i_t, r)
+// bc_(I,r) = sum_t w_t v_(i_t, r); planes > 0: bc in the planes of the stored coarse cycle
+// of that many unknowns (map_plane)
 template <typename T>
 __global__ void k_restrict_m(int nc, const int* __restrict__ rrow, const int* __restrict__ rcol,
                              const T* __restrict__ rval, const T* __restrict__ v,
-                             T* __restrict__ bc) {
+                             T* __restrict__ bc, int planes) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int I = t / K, r = t % K;
   if (I >= nc) return;
@@ -166,6 +167,12 @@ __global__ void k_restrict_m(int nc, const int* __restrict__ rrow, const int* __
     s1 = fma(w, a1, s1);
     s2 = fma(w, a2, s2);
   }
+  if (planes > 0) {
+    bc[map_plane(planes, 3 * I, r)] = s0;
+    bc[map_plane(planes, 3 * I + 1, r)] = s1;
+    bc[map_plane(planes, 3 * I + 2, r)] = s2;
+    return;
+  }
   st3(bc, I * K + r, s0, s1, s2);
 }
 
@@ -173,7 +180,7 @@ __global__ void k_restrict_m(int nc, const int* __restrict__ rrow, const int* __
 template <typename T>
 __global__ void k_prolong_m(int n, const int* __restrict__ prow, const int* __restrict__ pcol,
                             const T* __restrict__ pval, const T* __restrict__ xc, T* x,
-                            const T* __restrict__ wt) {
+                            const T* __restrict__ wt, int planes) {
   const T wc = wt ? wt[1] : T(1);   // coarse-correction scale
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int i = t / K, r = t % K;
@@ -182,7 +189,14 @@ __global__ void k_prolong_m(int n, const int* __restrict__ prow, const int* __re
   for (int q = prow[i]; q < prow[i + 1]; ++q) {
     const T w = pval[q];
     T a0, a1, a2;
-    ld3(xc, pcol[q] * K + r, a0, a1, a2);
+    if (planes > 0) {
+      const int k = 3 * pcol[q];
+      a0 = __ldg(xc + map_plane(planes, k, r));
+      a1 = __ldg(xc + map_plane(planes, k + 1, r));
+      a2 = __ldg(xc + map_plane(planes, k + 2, r));
+    } else {
+      ld3(xc, pcol[q] * K + r, a0, a1, a2);
+    }
     s0 = fma(w, a0, s0);
     s1 = fma(w, a1, s1);
     s2 = fma(w, a2, s2);
@@ -236,6 +250,25 @@ __global__ void k_f2d_m(const float* __restrict__ a, double* __restrict__ b, int
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
        k += (int64_t)gridDim.x * blockDim.x)
     b[k] = (double)a[k];
+}
+
+// [node][K][4] FP64 <-> the planes of the stored cycle of level 0 (padding 0)
+__global__ void k_d2f_planes(const double* __restrict__ a, float* __restrict__ b, int n) {
+  const int64_t tot = (int64_t)n * K * 4;
+  for (int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; f < tot;
+       f += (int64_t)gridDim.x * blockDim.x) {
+    const int c = (int)(f & 3), r = (int)((f >> 2) % K), node = (int)((f >> 2) / K);
+    if (c < 3) b[map_plane(3 * n, 3 * node + c, r)] = (float)a[f];
+  }
+}
+
+__global__ void k_f2d_planes(const float* __restrict__ a, double* __restrict__ b, int n) {
+  const int64_t tot = (int64_t)n * K * 4;
+  for (int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; f < tot;
+       f += (int64_t)gridDim.x * blockDim.x) {
+    const int c = (int)(f & 3), r = (int)((f >> 2) % K), node = (int)((f >> 2) / K);
+    b[f] = c < 3 ? (double)a[map_plane(3 * n, 3 * node + c, r)] : 0.0;
+  }
 }
 
 // user layout (nrhs vectors of 3n, vector r at offset r*3n) <-> [node][K][4]
@@ -701,16 +734,24 @@ void cycle_m(amg_handle* h, int l, T* x, const T* b, bool x_is_zero) {
     k_fill_m<T><<<gridk(nel), 256, 0, s>>>(x, nel);
     h->launches++;
   }
+  // the levels below as one stored matrix
+  const bool mapped = std::is_same<T, float>::value && h->batch_map && h->batch_map->from == l + 1;
+  const int planes = mapped ? h->batch_map->m : 0;
   T* r = MV<T>::r(bl);
   rows_m<T>(h, mResid, lv, 0, lv.n, MV<T>::val(lv), x, b, r, nullptr, T(0), bl.tile);
   k_restrict_m<T><<<gridk((int64_t)nx.n * K), 256, 0, s>>>(nx.n, lv.r_rowptr, lv.r_col,
-                                                          MV<T>::rval(lv), r, MV<T>::b(bn));
+                                                          MV<T>::rval(lv), r, MV<T>::b(bn),
+                                                          planes);
   h->launches++;
-  for (int k = 0; k < std::max(1, (l + 1 == L) ? 1 : h->opt.nu); ++k)
+  if (mapped) {
+    if constexpr (std::is_same<T, float>::value)
+      map_apply_m(h, *h->batch_map, MV<T>::b(bn), MV<T>::x(bn));
+  }
+  for (int k = 0; !mapped && k < std::max(1, (l + 1 == L) ? 1 : h->opt.nu); ++k)
     cycle_m<T>(h, l + 1, MV<T>::x(bn), MV<T>::b(bn), k == 0);
   k_prolong_m<T><<<gridk((int64_t)lv.n * K), 256, 0, s>>>(lv.n, lv.p_rowptr, lv.p_col,
                                                           MV<T>::pval(lv), MV<T>::x(bn), x,
-                                                          lv.template steps<T>());
+                                                          lv.template steps<T>(), planes);
   h->launches++;
   for (int k = 0; k < h->opt.m_post; ++k) smooth_m<T>(h, l, x, b, h->opt.post_order != 1);
 }
@@ -721,7 +762,12 @@ void precond_m(amg_handle* h, const double* r, double* z) {
   BatchLevel& b0 = h->B[0];
   const int64_t nel = 4 * (int64_t)K * l0.n;
   cudaStream_t s = h->stream;
-  if (h->opt.precision == AMG_FP32) {
+  if (h->batch_map && h->batch_map->from == 0) {
+    k_d2f_planes<<<gridk(nel), 256, 0, s>>>(r, b0.b32, l0.n);
+    map_apply_m(h, *h->batch_map, b0.b32, b0.x32);
+    k_f2d_planes<<<gridk(nel), 256, 0, s>>>(b0.x32, z, l0.n);
+    h->launches += 2;
+  } else if (h->opt.precision == AMG_FP32) {
     k_d2f_m<<<gridk(nel), 256, 0, s>>>(r, b0.b32, nel);
     h->launches++;
     for (int c = 0; c < std::max(1, h->opt.cycles); ++c)
@@ -806,8 +852,9 @@ int tune_pair_tile(amg_handle* h) {
 }
 
 void alloc_batch(amg_handle* h) {
-  if (!h->B.empty()) return;
   if (h->saddle) fail(AMG_ERR_UNSUPPORTED, "batched solves are provided for the SPD kinds");
+  h->batch_map = map_batch(h);
+  if (!h->B.empty()) return;
   h->B.resize(h->L.size());
   const bool f32 = h->opt.precision == AMG_FP32;
   auto z64 = [&](DBuf<double>& v, int64_t n) {

@@ -431,11 +431,11 @@ void run_cols(amg_handle* h, const Phase& P, int W) {
 
 // M (the handle's precision S) from the cycle's operations on blocks of T vectors
 template <typename T, typename S>
-void build(amg_handle* h, S* M) {
+void build(amg_handle* h, const CoarseMap& map, S* M) {
   // all columns at once up to kColMax: a launch's CTAs go over the rows of a colour first,
   // so a block of 256 columns keeps its vectors in L2, and the small colours still fill the
   // chip (512 columns a pass at 32^3: 97 ms, all but a few launches waiting on latency)
-  const int from = h->map_from, m = h->map_m;
+  const int from = map.from, m = map.m;
   const int nchunk = div_up(m, kColMax);
   const int W = div_up(div_up(m, nchunk), kColBlock) * kColBlock;
   std::vector<Phase> ph;
@@ -464,7 +464,7 @@ void build(amg_handle* h, S* M) {
     AMG_CUDA(cudaMemsetAsync(b, 0, (size_t)lv.dofs4() * W * sizeof(T), h->stream));
     k_cols_unit<T><<<div_up(W, 256), 256, 0, h->stream>>>(b, first, m, n3, W);
     for (const Phase& P : ph) run_cols<T, S>(h, P, W);
-    k_cols_store<T, S><<<m, 256, 0, h->stream>>>(x, M, first, m, h->map_ld, n3, W);
+    k_cols_store<T, S><<<m, 256, 0, h->stream>>>(x, M, first, m, map.ld, n3, W);
     h->launches += 2;
   }
   AMG_LAUNCH_CHECK();
@@ -553,13 +553,72 @@ __global__ void __launch_bounds__(kMapThreads) k_map_apply(int m, int ld, int n3
   }
 }
 
-template <typename T>
-const T* matrix(const amg_handle* h) {
-  if constexpr (std::is_same<T, float>::value) return h->map32.p;
-  else return h->map64.p;
+// X = M B for kRhs = 16 vectors in planes of four (map_plane).  A CTA takes R rows; its 8
+// warps share the columns (32 a step), so a lane multiplies one column of R rows with the
+// column's 16 entries of B: per step R coalesced 4-byte loads of M and 4 coalesced 16-byte
+// loads of B for 16 R FMAs.  The lanes' sums are reduced by halving exchanges (lane L ends
+// with R / 2 of the 16 R sums), then across the warps in shared memory.  FP32 issue bounds it
+// (16 m^2 FMAs: 2 us at m = 2,048 with the chip to itself).
+template <int R>
+__global__ void __launch_bounds__(256, R == 8 ? 1 : 2) k_map_m(int m, int ld,
+                                                               const float* __restrict__ M,
+                                                               const float* __restrict__ B,
+                                                               float* __restrict__ X) {
+  constexpr int V = R * kRhs;
+  __shared__ float red[8][V];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int row0 = blockIdx.x * R;
+  const float4* b4 = reinterpret_cast<const float4*>(B);
+  float v[V];
+#pragma unroll
+  for (int i = 0; i < V; ++i) v[i] = 0.f;
+#pragma unroll 2
+  for (int k = w * 32 + lane; k < m; k += 256) {
+    float a[R];
+    float4 b[4];
+#pragma unroll
+    for (int r = 0; r < R; ++r) a[r] = __ldg(M + (int64_t)min(row0 + r, m - 1) * ld + k);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) b[q] = __ldg(b4 + (int64_t)q * m + k);
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        float* s = v + r * kRhs + 4 * q;
+        s[0] = fmaf(a[r], b[q].x, s[0]);
+        s[1] = fmaf(a[r], b[q].y, s[1]);
+        s[2] = fmaf(a[r], b[q].z, s[2]);
+        s[3] = fmaf(a[r], b[q].w, s[3]);
+      }
+  }
+  int first = 0;
+#pragma unroll
+  for (int o = 16, n = V / 2; o > 0; o >>= 1, n >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+      const float other = __shfl_xor_sync(0xffffffffu, up ? v[i] : v[i + n], o);
+      v[i] = (up ? v[i + n] : v[i]) + other;
+    }
+    first += up ? n : 0;
+  }
+#pragma unroll
+  for (int i = 0; i < V / 32; ++i) red[w][first + i] = v[i];
+  __syncthreads();
+  const int t = threadIdx.x, row = row0 + t / kRhs, r = t % kRhs;
+  if (t < V && row < m) {
+    float s = 0.f, e = 0.f;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) pair_add(s, e, red[q][t], 0.f);
+    X[map_plane(m, row, r)] = s + e;
+  }
 }
 
-}  // namespace
+template <typename T>
+const T* matrix(const CoarseMap& M) {
+  if constexpr (std::is_same<T, float>::value) return M.m32.p;
+  else return M.m64.p;
+}
 
 // The largest level stored as a matrix.  Below these sizes M b is faster than the chain
 // of launches that it replaces: reading M takes 4 m^2 bytes at about 6 TB/s in FP32 (63 us
@@ -571,52 +630,87 @@ constexpr int kMapMax64 = 6144;
 // and the share of the coarsest solve (FP64) in the construction
 constexpr int64_t kMapCoarseWork = 4000000000ll;
 
-void map_plan(amg_handle* h) {
-  const amg_options& o = h->opt;
-  h->map_from = -1;
-  // a launch variant that the caller forces keeps its levels; the Vanka phases are not recorded
-  if (o.cluster_from != -1 || o.cycle_kernel != 0 || o.gs_cluster != -1 || o.gs_flow != -1 ||
-      o.gs_stream != -1 || o.gs_tma != -1 || o.smoother == AMG_SMOOTHER_VANKA)
-    return;
-  const bool f32 = o.precision == AMG_FP32;
+// Batched solves, FP32: M B takes 16 m^2 FMAs, 8 us of the whole chip at 4,096.  The chain
+// that it replaces leaves most of the chip to the other problems, so no larger map is used.
+constexpr int kMapMaxBatch = 4096;
+
+// the first level of at most `most` unknowns, its matrix allocated and zero
+void plan(amg_handle* h, CoarseMap& M, int most) {
+  const bool f32 = h->opt.precision == AMG_FP32;
   for (int l = 0; l + 1 < (int)h->L.size(); ++l) {
     const int m = h->L[l]->dofs();
-    if (m > (f32 ? kMapMax32 : kMapMax64) ||
-        (int64_t)h->coarse_m * h->coarse_m * m > kMapCoarseWork)
-      continue;
-    h->map_m = m;
-    h->map_ld = (m + 31) / 32 * 32;
-    const size_t count = (size_t)m * h->map_ld;
+    if (m > most || (int64_t)h->coarse_m * h->coarse_m * m > kMapCoarseWork) continue;
+    M.m = m;
+    M.ld = (m + 31) / 32 * 32;
+    const size_t count = (size_t)m * M.ld;
     try {
-      if (f32) h->map32.alloc(count);
-      else h->map64.alloc(count);
+      if (f32) M.m32.alloc(count);
+      else M.m64.alloc(count);
     } catch (const Error& e) {
       if (e.code != AMG_ERR_NOMEM) throw;
       return;   // no room: the cycle runs operation by operation
     }
     // the padding of the rows stays 0
-    if (f32) AMG_CUDA(cudaMemsetAsync(h->map32.p, 0, h->map32.bytes(), h->stream));
-    else AMG_CUDA(cudaMemsetAsync(h->map64.p, 0, h->map64.bytes(), h->stream));
-    h->map_from = l;
+    if (f32) AMG_CUDA(cudaMemsetAsync(M.m32.p, 0, M.m32.bytes(), h->stream));
+    else AMG_CUDA(cudaMemsetAsync(M.m64.p, 0, M.m64.bytes(), h->stream));
+    M.from = l;
     return;
   }
 }
 
-void map_build(amg_handle* h, const double* w) {
-  if (h->map_from < 0) return;
+void fill(amg_handle* h, CoarseMap& M, const double* w) {
+  if (M.from < 0) return;
   // the weights of the levels that M holds (4 a level): nothing to do if they are as built
-  const std::vector<double> now(w + 4 * h->map_from, w + 4 * h->L.size());
-  if (now == h->map_w) return;
-  h->map_w.clear();
-  if (h->map32.p) build<Pair, float>(h, h->map32.p);
-  else build<double, double>(h, h->map64.p);
-  h->map_w = now;
+  const std::vector<double> now(w + 4 * M.from, w + 4 * h->L.size());
+  if (now == M.w) return;
+  M.w.clear();
+  if (M.m32.p) build<Pair, float>(h, M, M.m32.p);
+  else build<double, double>(h, M, M.m64.p);
+  M.w = now;
+}
+
+}  // namespace
+
+void map_plan(amg_handle* h) {
+  const amg_options& o = h->opt;
+  // a launch variant that the caller forces keeps its levels; the Vanka phases are not recorded
+  if (o.cluster_from != -1 || o.cycle_kernel != 0 || o.gs_cluster != -1 || o.gs_flow != -1 ||
+      o.gs_stream != -1 || o.gs_tma != -1 || o.smoother == AMG_SMOOTHER_VANKA)
+    return;
+  plan(h, h->map, o.precision == AMG_FP32 ? kMapMax32 : kMapMax64);
+}
+
+const CoarseMap* map_batch(amg_handle* h) {
+  // the batched cycle reads the FP32 values of every level, also with BF16 storage
+  if (h->map.from < 0 || !h->map.m32.p || h->bf16_coarse || h->opt.batch_tile != -1)
+    return nullptr;
+  if (h->map.m <= kMapMaxBatch) return &h->map;
+  if (h->bmap.from < 0) {
+    plan(h, h->bmap, kMapMaxBatch);
+    if (h->bmap.from < 0) return nullptr;
+    std::vector<double> w(4 * h->L.size());
+    get_weights(h, w.data());
+    fill(h, h->bmap, w.data());
+  }
+  return &h->bmap;
+}
+
+void map_build(amg_handle* h, const double* w) {
+  fill(h, h->map, w);
+  fill(h, h->bmap, w);
+}
+
+void map_apply_m(amg_handle* h, const CoarseMap& M, const float* b, float* x) {
+  // 4 rows a CTA where 8 would leave SMs idle
+  if (M.m < 8 * 152) k_map_m<4><<<div_up(M.m, 4), 256, 0, h->stream>>>(M.m, M.ld, M.m32, b, x);
+  else k_map_m<8><<<div_up(M.m, 8), 256, 0, h->stream>>>(M.m, M.ld, M.m32, b, x);
+  h->launches++;
 }
 
 template <typename T, typename IO>
 void map_apply(amg_handle* h, const IO* b, IO* x) {
-  const int m = h->map_m, ld = h->map_ld, n3 = 3 * h->L[h->map_from]->n;
-  const T* M = matrix<T>(h);
+  const int m = h->map.m, ld = h->map.ld, n3 = 3 * h->L[h->map.from]->n;
+  const T* M = matrix<T>(h->map);
   const int smem = ld * (int)sizeof(T);
   const bool stream = (int64_t)m * ld * sizeof(T) > (64ll << 20);
   const auto k = stream ? k_map_apply<T, IO, true> : k_map_apply<T, IO, false>;

@@ -2229,7 +2229,7 @@ void cycle_rec(Emit<T>& e, amg_handle* h, int l, T* x, const T* b, bool x_is_zer
 template <typename T>
 void coarse_calls(Emit<T>& e, amg_handle* h, int l, T* xc, const T* bc) {
   const int L = (int)h->L.size() - 1;
-  if (!e.rec && h->map_from > 0 && l == h->map_from) {
+  if (!e.rec && h->map.from > 0 && l == h->map.from) {
     map_apply<T, T>(h, bc, xc);
     return;
   }
@@ -2461,7 +2461,7 @@ template void record_map_phases<double>(amg_handle*, int, std::vector<Phase>&);
 // z = M^{-1} r: opt.cycles applications of Algorithm 1 from zero.
 template <>
 void precondition_device<double>(amg_handle* h, const double* r, double* z) {
-  if (h->map_from == 0) {
+  if (h->map.from == 0) {
     map_apply<double, double>(h, r, z);
     return;
   }
@@ -2478,7 +2478,7 @@ void precondition_device<double>(amg_handle* h, const double* r, double* z) {
 
 template <>
 void precondition_device<float>(amg_handle* h, const double* r, double* z) {
-  if (h->map_from == 0) {
+  if (h->map.from == 0) {
     map_apply<float, double>(h, r, z);
     return;
   }
@@ -2564,7 +2564,7 @@ void autotune_levels(amg_handle* h) {
   for (auto& lv : h->L)
     if (lv->ncolours > 0) lv->group_gs = gs_lanes(f32, (double)lv->n / lv->ncolours);
   // levels that run as one stored matrix keep the default lanes per row
-  const size_t nl = h->map_from >= 0 ? std::max(h->map_from, 1) : h->L.size();
+  const size_t nl = h->map.from >= 0 ? std::max(h->map.from, 1) : h->L.size();
   for (size_t l = 0; l < nl; ++l) {
     Level& lv = *h->L[l];
     lv.gs_cl = 0;
@@ -2614,10 +2614,10 @@ void autotune_levels(amg_handle* h) {
       AMG_CUDA(cudaStreamSynchronize(s));
     }
     if (lv.ncolours == 0 || h->saddle || h->opt.smoother != AMG_SMOOTHER_GS ||
-        h->map_from == 0)
+        h->map.from == 0)
       continue;
     lv.gs_stream = 0;
-    if (h->map_from >= 0) continue;   // the other sweep kernels below were slower on every
+    if (h->map.from >= 0) continue;   // the other sweep kernels below were slower on every
                                       // level that the stored matrix leaves to the chain
     auto sweep_ms = [&]() {
       for (int r = 0; r < 7; ++r) {
@@ -2784,7 +2784,7 @@ void autotune_levels(amg_handle* h) {
       fail(AMG_ERR_TIMEOUT, "a bounded wait of a one-launch colour sweep (mbarrier or dataflow "
                             "flag) timed out during setup tuning");
   }
-  if (h->map_from >= 0) {
+  if (h->map.from >= 0) {
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     return;

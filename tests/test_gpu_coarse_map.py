@@ -103,3 +103,28 @@ def test_linear_and_repeatable():
     zu, zv, zs = apply(h, u), apply(h, v), apply(h, 3.0 * u + v)
     assert float((zs - 3.0 * zu - zv).norm() / zs.norm()) <= TOL[0]
     assert torch.equal(apply(h, u), zu)
+
+
+@pytest.mark.parametrize("n_rhs", [1, 16])
+@pytest.mark.parametrize("size", [3, (4, 5, 3), 8, (10, 11, 9), 12])
+def test_batched_stored_cycle(size, n_rhs):
+    """Batched FP32 solves through the stored cycle (level 0, level 1, and a batch-only one
+    below the single solve's) against batched solves without it (batch_tile given): the same
+    iteration counts within one and the same solutions to the solver's tolerance."""
+    prob = fp.elasticity_problem(size, seed=9, nu=0.35)
+    rng = np.random.default_rng(10)
+    b = rng.standard_normal((n_rhs, 3 * prob.n_nodes))
+    b[:, np.repeat((prob.tags & fp.TAG_DIRICHLET) != 0, 3)] = 0.0
+    b = torch.from_numpy(b).cuda()
+    out = []
+    for tile in (-1, 0):
+        h = B().setup_problem(prob, B().default_options(precision=1, batch_tile=tile))
+        for w in ((1.0, 1.0, 1.0), (0.9, 1.1, 1.0)):    # the batch's own matrix follows too
+            h.set_weights(*w)
+            x = torch.zeros_like(b)
+            rc, st = B().solve_batched([h], [b], [x], n_rhs, 1e-9)
+            assert rc == 0
+            out.append((x, st[0].iterations))
+    for k in (0, 1):
+        assert abs(out[k][1] - out[2 + k][1]) <= 1
+        assert float((out[k][0] - out[2 + k][0]).norm() / out[2 + k][0].norm()) <= 1e-7
