@@ -96,6 +96,8 @@ struct Level {
   // a colour sweep reads one contiguous range.  The cycle's row kernels use it.
   bool stored = false;
   DBuf<int> srowptr, scol;
+  DBuf<int> smid, sup;          // the diagonal block of a stored row, the first block after it
+                                // (before it the lower colours, after it the higher ones)
   DBuf<double> sval;            // 9 planes, stored order
   const int* k_rowptr() const { return stored ? srowptr.p : rowptr.p; }
   const int* k_col() const { return stored ? scol.p : col.p; }

@@ -38,10 +38,11 @@ __device__ __forceinline__ T ldg(const T* p) { return __ldg(p); }
 // Tile of the SpMM row kernels: S lane groups of 16 per stored row (lane r of a
 // group = right-hand side r), group q taking the blocks q, q + S, ... of the row
 // (S = 2: one warp a row, partial sums combined by a shuffle); U blocks unrolled.
-// Row data at rowptr[g]..rowptr[g+1] (colour-major storage when rows != null).
+// Row data at rowptr[g]..rowend[g] (colour-major storage when rows != null).
 template <typename T, int MODE, int S, int U>
 __global__ void __launch_bounds__(256) k_rows_m(int nrows, const int* __restrict__ rows,
                                                 const int* __restrict__ rowptr,
+                                                const int* __restrict__ rowend,
                                                 const int* __restrict__ col,
                                                 const T* __restrict__ val, int64_t nnzb,
                                                 const T* x, const T* __restrict__ b, T* y,
@@ -53,7 +54,7 @@ __global__ void __launch_bounds__(256) k_rows_m(int nrows, const int* __restrict
   const int r = threadIdx.x % K;
   if (g >= nrows) return;                       // uniform over the S groups of a row
   const int i = rows ? ldg(rows + g) : g;
-  const int a = ldg(rowptr + g), e = ldg(rowptr + g + 1);
+  const int a = ldg(rowptr + g), e = ldg(rowend + g);
   T s0 = T(0), s1 = T(0), s2 = T(0);
 #pragma unroll U
   for (int k = a + q; k < e; k += S) {
@@ -474,14 +475,15 @@ constexpr int kGsTiles = 8; // colour kernel: tiles 0..3 as above, 4..7: S = 4 <
 // come after the wait, which is where the previous kernel's writes become
 // visible.  Tiles as in k_rows_m, and with S = 4 or 8 lane groups a row (2 or 4 warps,
 // their sums combined in shared memory) for rows whose dependent block chain is long.
-template <typename T, int S, int U>
+template <typename T, int S, int U, bool FIRST>
 __global__ void __launch_bounds__(256) k_gs_m_pdl(int nrows, const int* __restrict__ rows,
                                                   const int* __restrict__ rowptr,
+                                                  const int* __restrict__ rowend,
                                                   const int* __restrict__ col,
                                                   const T* __restrict__ val, int64_t nnzb, T* x,
                                                   const T* __restrict__ b,
                                                   const T* __restrict__ dinv,
-                                                  const T* __restrict__ wt) {
+                                                  const T* __restrict__ wt, T* __restrict__ seed) {
   // S > 2: the S / 2 warps of a row combine their sums through shared memory
   __shared__ T red[S > 2 ? 256 / 32 : 1][K][3];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -499,7 +501,7 @@ __global__ void __launch_bounds__(256) k_gs_m_pdl(int nrows, const int* __restri
   if (active) {
     i = __ldg(rows + g);
     a = __ldg(rowptr + g);
-    e = __ldg(rowptr + g + 1);
+    e = __ldg(rowend + g);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int k = a + q + u * S;
@@ -572,17 +574,19 @@ __global__ void __launch_bounds__(256) k_gs_m_pdl(int nrows, const int* __restri
   }
   if (S >= 2 && q != 0) return;
   const int o = i * K + r;
-  T x0, x1, x2;
-  ld3(x, o, x0, x1, x2);
+  T x0 = T(0), x1 = T(0), x2 = T(0);
+  if (!FIRST) ld3(x, o, x0, x1, x2);
   const T r0 = b0 - s0, r1 = b1 - s1, r2 = b2 - s2;
+  if (FIRST && seed) st3(seed, o, (T(1) - om) * r0, (T(1) - om) * r1, (T(1) - om) * r2);
   st3(x, o, x0 + om * (d[0] * r0 + d[1] * r1 + d[2] * r2),
       x1 + om * (d[3] * r0 + d[4] * r1 + d[5] * r2),
       x2 + om * (d[6] * r0 + d[7] * r1 + d[8] * r2));
 }
 
 template <typename T, int S, int U>
-void launch_gs_m_pdl(int nrows, const int* rows, const int* rowptr, Level& lv, const T* val,
-                     T* x, const T* b, const T* dinv, cudaStream_t s) {
+void launch_gs_m_pdl(int nrows, const int* rows, const int* rowptr, const int* rowend, Level& lv,
+                     const T* val, T* x, const T* b, const T* dinv, bool first, T* seed,
+                     cudaStream_t s) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(((int64_t)nrows * K * S + 255) / 256));
   cfg.blockDim = dim3(256);
@@ -592,50 +596,54 @@ void launch_gs_m_pdl(int nrows, const int* rows, const int* rowptr, Level& lv, c
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  AMG_CUDA(cudaLaunchKernelEx(&cfg, k_gs_m_pdl<T, S, U>, nrows, rows, rowptr,
-                              (const int*)lv.k_col(), val, lv.nnzb, x, b, dinv,
-                              lv.template steps<T>()));
+  const auto k = first ? k_gs_m_pdl<T, S, U, true> : k_gs_m_pdl<T, S, U, false>;
+  AMG_CUDA(cudaLaunchKernelEx(&cfg, k, nrows, rows, rowptr, rowend, (const int*)lv.k_col(), val,
+                              lv.nnzb, x, b, dinv, lv.template steps<T>(), seed));
 }
 
-// one colour of the batched Gauss-Seidel sweep (x updated in place)
+// one colour of the batched Gauss-Seidel sweep (x updated in place; `first`: from x = 0 on the
+// lower-colour blocks, leaving the residual's seed, as kFirst of the single cycle)
 template <typename T>
-void gs_colour_m(amg_handle* h, Level& lv, int first, int nrows, const T* val, T* x,
-                 const T* b, const T* dinv, int tile) {
+void gs_colour_m(amg_handle* h, Level& lv, int at, int nrows, const T* val, T* x, const T* b,
+                 const T* dinv, int tile, bool first, T* seed) {
   if (nrows <= 0) return;
-  const int* rows = lv.k_rows() + first;
-  const int* rowptr = lv.k_rowptr() + first;
+  const int* rows = lv.k_rows() + at;
+  const int* rp = lv.k_rowptr() + at;
+  const int* re = first ? lv.smid.p + at : rp + 1;
   cudaStream_t s = h->stream;
   switch (tile) {
-    case 1: launch_gs_m_pdl<T, 2, 2>(nrows, rows, rowptr, lv, val, x, b, dinv, s); break;
-    case 2: launch_gs_m_pdl<T, 1, 4>(nrows, rows, rowptr, lv, val, x, b, dinv, s); break;
-    case 3: launch_gs_m_pdl<T, 2, 4>(nrows, rows, rowptr, lv, val, x, b, dinv, s); break;
-    case 4: launch_gs_m_pdl<T, 4, 2>(nrows, rows, rowptr, lv, val, x, b, dinv, s); break;
-    case 5: launch_gs_m_pdl<T, 8, 2>(nrows, rows, rowptr, lv, val, x, b, dinv, s); break;
-    case 6: launch_gs_m_pdl<T, 4, 4>(nrows, rows, rowptr, lv, val, x, b, dinv, s); break;
-    case 7: launch_gs_m_pdl<T, 8, 4>(nrows, rows, rowptr, lv, val, x, b, dinv, s); break;
-    default: launch_gs_m_pdl<T, 1, 2>(nrows, rows, rowptr, lv, val, x, b, dinv, s); break;
+    case 1: launch_gs_m_pdl<T, 2, 2>(nrows, rows, rp, re, lv, val, x, b, dinv, first, seed, s); break;
+    case 2: launch_gs_m_pdl<T, 1, 4>(nrows, rows, rp, re, lv, val, x, b, dinv, first, seed, s); break;
+    case 3: launch_gs_m_pdl<T, 2, 4>(nrows, rows, rp, re, lv, val, x, b, dinv, first, seed, s); break;
+    case 4: launch_gs_m_pdl<T, 4, 2>(nrows, rows, rp, re, lv, val, x, b, dinv, first, seed, s); break;
+    case 5: launch_gs_m_pdl<T, 8, 2>(nrows, rows, rp, re, lv, val, x, b, dinv, first, seed, s); break;
+    case 6: launch_gs_m_pdl<T, 4, 4>(nrows, rows, rp, re, lv, val, x, b, dinv, first, seed, s); break;
+    case 7: launch_gs_m_pdl<T, 8, 4>(nrows, rows, rp, re, lv, val, x, b, dinv, first, seed, s); break;
+    default: launch_gs_m_pdl<T, 1, 2>(nrows, rows, rp, re, lv, val, x, b, dinv, first, seed, s); break;
   }
   h->launches++;
 }
 
 template <typename T, int MODE, int S, int U>
-void launch_rows_m(int nrows, const int* rows, const int* rowptr, Level& lv, const T* val,
+void launch_rows_m(int nrows, const int* rows, const int* rowptr, const int* rowend, Level& lv,
+                   const T* val,
                    const T* x, const T* b, T* y, const T* dinv, T omega, const T* wt,
                    cudaStream_t s) {
   const int grid = (int)(((int64_t)nrows * K * S + 255) / 256);
-  k_rows_m<T, MODE, S, U><<<grid, 256, 0, s>>>(nrows, rows, rowptr, lv.k_col(), val, lv.nnzb, x,
-                                               b, y, dinv, omega, wt);
+  k_rows_m<T, MODE, S, U><<<grid, 256, 0, s>>>(nrows, rows, rowptr, rowend, lv.k_col(), val,
+                                               lv.nnzb, x, b, y, dinv, omega, wt);
 }
 
 template <typename T, int MODE>
-void launch_tile_m(int tile, int nrows, const int* rows, const int* rowptr, Level& lv,
+void launch_tile_m(int tile, int nrows, const int* rows, const int* rowptr, const int* rowend,
+                   Level& lv,
                    const T* val, const T* x, const T* b, T* y, const T* dinv, T omega,
                    const T* wt, cudaStream_t s) {
   switch (tile) {
-    case 1: launch_rows_m<T, MODE, 2, 2>(nrows, rows, rowptr, lv, val, x, b, y, dinv, omega, wt, s); break;
-    case 2: launch_rows_m<T, MODE, 1, 4>(nrows, rows, rowptr, lv, val, x, b, y, dinv, omega, wt, s); break;
-    case 3: launch_rows_m<T, MODE, 2, 4>(nrows, rows, rowptr, lv, val, x, b, y, dinv, omega, wt, s); break;
-    default: launch_rows_m<T, MODE, 1, 2>(nrows, rows, rowptr, lv, val, x, b, y, dinv, omega, wt, s); break;
+    case 1: launch_rows_m<T, MODE, 2, 2>(nrows, rows, rowptr, rowend, lv, val, x, b, y, dinv, omega, wt, s); break;
+    case 2: launch_rows_m<T, MODE, 1, 4>(nrows, rows, rowptr, rowend, lv, val, x, b, y, dinv, omega, wt, s); break;
+    case 3: launch_rows_m<T, MODE, 2, 4>(nrows, rows, rowptr, rowend, lv, val, x, b, y, dinv, omega, wt, s); break;
+    default: launch_rows_m<T, MODE, 1, 2>(nrows, rows, rowptr, rowend, lv, val, x, b, y, dinv, omega, wt, s); break;
   }
 }
 
@@ -660,31 +668,33 @@ void apply_pair_m(amg_handle* h, const float* xp, double* y, int tile) {
 
 template <typename T>
 void rows_m(amg_handle* h, int mode, Level& lv, int first, int nrows, const T* val, const T* x,
-            const T* b, T* y, const T* dinv, T omega, int tile) {
+            const T* b, T* y, const T* dinv, T omega, int tile, bool upper = false) {
   if (nrows <= 0) return;
   const int* order = lv.k_rows();
   const int* rows = order ? order + first : nullptr;
-  const int* rowptr = lv.k_rowptr() + first;
+  const int* rowptr = (upper ? lv.sup.p : lv.k_rowptr()) + first;   // upper: higher colours only
+  const int* rowend = lv.k_rowptr() + first + 1;
   cudaStream_t s = h->stream;
   switch (mode) {
     case mApply:
-      launch_tile_m<T, mApply>(tile, nrows, rows, rowptr, lv, val, x, b, y, dinv, omega, nullptr, s);
+      launch_tile_m<T, mApply>(tile, nrows, rows, rowptr, rowend, lv, val, x, b, y, dinv, omega, nullptr, s);
       break;
     case mResid:
-      launch_tile_m<T, mResid>(tile, nrows, rows, rowptr, lv, val, x, b, y, dinv, omega, nullptr, s);
+      launch_tile_m<T, mResid>(tile, nrows, rows, rowptr, rowend, lv, val, x, b, y, dinv, omega, nullptr, s);
       break;
     case mGS:
-      launch_tile_m<T, mGS>(tile, nrows, rows, rowptr, lv, val, x, b, y, dinv, omega, lv.template steps<T>(), s);
+      launch_tile_m<T, mGS>(tile, nrows, rows, rowptr, rowend, lv, val, x, b, y, dinv, omega, lv.template steps<T>(), s);
       break;
     default:
-      launch_tile_m<T, mJacobi>(tile, nrows, rows, rowptr, lv, val, x, b, y, dinv, omega, lv.template steps<T>(), s);
+      launch_tile_m<T, mJacobi>(tile, nrows, rows, rowptr, rowend, lv, val, x, b, y, dinv, omega, lv.template steps<T>(), s);
       break;
   }
   h->launches++;
 }
 
 template <typename T>
-void smooth_m(amg_handle* h, int l, T* x, const T* b, bool post) {
+void smooth_m(amg_handle* h, int l, T* x, const T* b, bool post, bool first = false,
+              T* seed = nullptr) {
   Level& lv = *h->L[l];
   BatchLevel& bl = h->B[l];
   if (h->opt.smoother == AMG_SMOOTHER_JACOBI) {
@@ -699,7 +709,8 @@ void smooth_m(amg_handle* h, int l, T* x, const T* b, bool post) {
     const int c = post ? lv.ncolours - 1 - q : q;
     const int a = lv.colour_ptr[c], e = lv.colour_ptr[c + 1];
     if (h->use_pdl && lv.k_rows())
-      gs_colour_m<T>(h, lv, a, e - a, MV<T>::val(lv), x, b, MV<T>::dinv(lv), bl.tile_gs);
+      gs_colour_m<T>(h, lv, a, e - a, MV<T>::val(lv), x, b, MV<T>::dinv(lv), bl.tile_gs,
+                     first, seed);
     else
       rows_m<T>(h, mGS, lv, a, e - a, MV<T>::val(lv), x, b, x, MV<T>::dinv(lv), T(1), bl.tile);
   }
@@ -722,12 +733,17 @@ void cycle_m(amg_handle* h, int l, T* x, const T* b, bool x_is_zero) {
   BatchLevel& bn = h->B[l + 1];
   const int64_t nel = 4 * (int64_t)K * lv.n;
   bool zero = x_is_zero;
+  // a first Gauss-Seidel sweep from x = 0 and the residual after it on half of A each
+  T* seed = nullptr;
+  const bool first = zero && h->opt.m_pre > 0 && h->opt.smoother == AMG_SMOOTHER_GS &&
+                     h->use_pdl && lv.stored;
   for (int k = 0; k < h->opt.m_pre; ++k) {
-    if (zero) {
+    if (zero && !first) {
       k_fill_m<T><<<gridk(nel), 256, 0, s>>>(x, nel);
       h->launches++;
     }
-    smooth_m<T>(h, l, x, b, false);
+    if (k == 0 && first && h->opt.m_pre == 1) seed = MV<T>::t(bl);
+    smooth_m<T>(h, l, x, b, false, k == 0 && first, seed);
     zero = false;
   }
   if (zero) {
@@ -738,7 +754,8 @@ void cycle_m(amg_handle* h, int l, T* x, const T* b, bool x_is_zero) {
   const bool mapped = std::is_same<T, float>::value && h->batch_map && h->batch_map->from == l + 1;
   const int planes = mapped ? h->batch_map->m : 0;
   T* r = MV<T>::r(bl);
-  rows_m<T>(h, mResid, lv, 0, lv.n, MV<T>::val(lv), x, b, r, nullptr, T(0), bl.tile);
+  rows_m<T>(h, mResid, lv, 0, lv.n, MV<T>::val(lv), x, seed ? seed : b, r, nullptr, T(0), bl.tile,
+            seed != nullptr);
   k_restrict_m<T><<<gridk((int64_t)nx.n * K), 256, 0, s>>>(nx.n, lv.r_rowptr, lv.r_col,
                                                           MV<T>::rval(lv), r, MV<T>::b(bn),
                                                           planes);

@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(kColThreads) k_cols_rows(const Phase P, int W)
   const T* x = (const T*)P.x + c;
   const V* val = (const V*)P.val;
   const int i = P.rows ? __ldg(P.rows + g) : g;
-  const int a = __ldg(P.rowptr + g), e = __ldg(P.rowptr + g + 1);
+  const int a = __ldg(P.rowptr + g), e = __ldg(P.rowend + g);
   // the row's columns and values staged in shared memory, kStage blocks at a time; A sums
   // of every A-th block each, whose loads are in flight together
   constexpr int A = 4, kStage = 64;
@@ -192,13 +192,19 @@ __global__ void __launch_bounds__(kColThreads) k_cols_rows(const Phase P, int W)
   }
   if (P.mode == kResid) return;
   const S* wt = (const S*)P.wt;
-  const S om = wt ? wt[P.mode == kGS ? 0 : 2] : (S)P.omega;
+  const S om = wt ? wt[P.mode == kJacobi ? 2 : 0] : (S)P.omega;
   const S* d = (const S*)P.dinv + 12 * (int64_t)i;
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
-    Cell<T> t = zero<T>(), xi = ldc(x + o + q * W);
+    Cell<T> t = zero<T>(), xi = zero<T>();
+    if (P.mode != kFirst) xi = ldc(x + o + q * W);
 #pragma unroll
     for (int p = 0; p < 3; ++p) axpy(t, __ldg(d + 4 * q + p), r[p]);
+    if (P.mode == kFirst && P.p) {
+      Cell<T> u = zero<T>();
+      axpy(u, S(1) - om, r[q]);
+      stc((T*)P.p + c + o + q * W, u);
+    }
 #pragma unroll
     for (int w = 0; w < kColN; ++w) t.v[w] = normal(t.v[w]);
     axpy(xi, om, t);

@@ -87,14 +87,16 @@ struct VL<true> {
 template <typename T, int G, int MODE, bool COH, typename V = T>
 __device__ __forceinline__ void rows_body(int nrows, const int* __restrict__ rows,
                                           const int* __restrict__ rowptr,
+                                          const int* __restrict__ rowend,
                                           const int* __restrict__ col,
                                           const V* __restrict__ val, int64_t nnzb, const T* x,
                                           const T* b, T* y, const T* __restrict__ dinv,
-                                          T omega, const T* __restrict__ wt, int warp,
+                                          T omega, const T* __restrict__ wt, T* seed, int warp,
                                           int nwarps) {
   constexpr int RPW = 32 / G;
   // relaxation: the level's step, weights included (Level::wt), else omega
-  if ((MODE == kGS || MODE == kJacobi) && wt) omega = wt[MODE == kGS ? 0 : 2];
+  if ((MODE == kGS || MODE == kJacobi || MODE == kFirst) && wt)
+    omega = wt[MODE == kJacobi ? 2 : 0];
   const int lane = threadIdx.x & 31;
   const int sub = lane / G, gl = lane & (G - 1);
   for (int base = warp * RPW; base < nrows; base += nwarps * RPW) {
@@ -110,9 +112,9 @@ __device__ __forceinline__ void rows_body(int nrows, const int* __restrict__ row
       i = rows ? ldg(rows + g) : g;
       if (MODE != kApply && End::holds(gl)) {
         End::template load<VL<COH>>(b, i, gl, bi);
-        if (MODE != kResid) End::template load<VL<COH>>(x, i, gl, xi);
+        if (MODE != kResid && MODE != kFirst) End::template load<VL<COH>>(x, i, gl, xi);
       }
-      const int a = ldg(rowptr + g), e = ldg(rowptr + g + 1);
+      const int a = ldg(rowptr + g), e = ldg(rowend + g);
       // U blocks per lane per step: all column indices of the step are loaded
       // before the gathers that depend on them
       // FP64 keeps fewer blocks in flight per lane (register budget)
@@ -158,10 +160,16 @@ __device__ __forceinline__ void rows_body(int nrows, const int* __restrict__ row
 #pragma unroll
       for (int q = 0; q < End::N; ++q) v[q] = bi[q] - v[q];
     }
-    if (MODE == kGS || MODE == kJacobi) {
+    if (MODE == kGS || MODE == kJacobi || MODE == kFirst) {
       T r0, r1, r2;
       End::all(v, r0, r1, r2);
       if (!active) continue;
+      if (MODE == kFirst && seed) {
+        T o[End::N];
+#pragma unroll
+        for (int q = 0; q < End::N; ++q) o[q] = (T(1) - omega) * v[q];
+        End::template store<true>(seed, i, gl, o);
+      }
       if (End::holds(gl)) {
 #pragma unroll
         for (int q = 0; q < End::N; ++q) {
@@ -470,13 +478,14 @@ __device__ void dispatch_rows_v(const Phase& P, int warp, int nwarps) {
   const T* d = (const T*)P.dinv;
   const T om = (T)P.omega;
 #define AMG_ROWS_MODE(GG, MM)                                                                   \
-  rows_body<T, GG, MM, COH, V>(P.n, P.rows, P.rowptr, P.col, val, P.nnz, x, b, y, d, om, (const T*)P.wt, \
-                               warp, nwarps)
+  rows_body<T, GG, MM, COH, V>(P.n, P.rows, P.rowptr, P.rowend, P.col, val, P.nnz, x, b, y, d, \
+                               om, (const T*)P.wt, (T*)P.p, warp, nwarps)
 #define AMG_ROWS_G(GG)                              \
   switch (P.mode) {                                 \
     case kApply: AMG_ROWS_MODE(GG, kApply); break;  \
     case kResid: AMG_ROWS_MODE(GG, kResid); break;  \
     case kGS: AMG_ROWS_MODE(GG, kGS); break;        \
+    case kFirst: AMG_ROWS_MODE(GG, kFirst); break;  \
     default: AMG_ROWS_MODE(GG, kJacobi); break;     \
   }
   switch (P.G) {
@@ -580,14 +589,15 @@ __device__ __forceinline__ void exec_phase(const Phase& P, int tid, int nthr) {
 // Within one colour launch nothing that is gathered is written (rows of one
 // colour are not neighbours; a row reads its own x_i before writing it), and the
 // previous kernels' writes are visible after griddepcontrol.wait.
-template <typename T, int G, int U, typename V = T>
+template <typename T, int G, int U, bool FIRST, typename V = T>
 __global__ void __launch_bounds__(256) k_gs_pdl(int nrows, const int* __restrict__ rows,
                                                 const int* __restrict__ rowptr,
+                                                const int* __restrict__ rowend,
                                                 const int* __restrict__ col,
                                                 const V* __restrict__ val, int64_t nnzb, T* x,
                                                 const T* __restrict__ b,
                                                 const T* __restrict__ dinv,
-                                                const T* __restrict__ wt) {
+                                                const T* __restrict__ wt, T* __restrict__ seed) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int g = (blockIdx.x * blockDim.x + threadIdx.x) / G;
   const int gl = threadIdx.x & (G - 1);
@@ -602,7 +612,7 @@ __global__ void __launch_bounds__(256) k_gs_pdl(int nrows, const int* __restrict
   if (active) {
     i = ldg(rows + g);
     a = ldg(rowptr + g);
-    e = ldg(rowptr + g + 1);
+    e = ldg(rowend + g);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int k = a + gl + u * G;
@@ -626,7 +636,7 @@ __global__ void __launch_bounds__(256) k_gs_pdl(int nrows, const int* __restrict
   if (active) {
     if (gl == 0) {
       ld3(b, i, b0, b1, b2);
-      VL<true>::node(x, i, xi0, xi1, xi2);
+      if (!FIRST) VL<true>::node(x, i, xi0, xi1, xi2);
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -662,6 +672,7 @@ __global__ void __launch_bounds__(256) k_gs_pdl(int nrows, const int* __restrict
   }
   if (!active || gl != 0) return;
   const T r0 = b0 - s0, r1 = b1 - s1, r2 = b2 - s2;
+  if (FIRST && seed) st3(seed, i, (T(1) - om) * r0, (T(1) - om) * r1, (T(1) - om) * r2);
   st3(x, i, xi0 + om * (d[0] * r0 + d[1] * r1 + d[2] * r2),
       xi1 + om * (d[3] * r0 + d[4] * r1 + d[5] * r2), xi2 + om * (d[6] * r0 + d[7] * r1 + d[8] * r2));
 }
@@ -669,14 +680,16 @@ __global__ void __launch_bounds__(256) k_gs_pdl(int nrows, const int* __restrict
 // The same in FP64, ending with one component a lane (row_sum3, spread3): each FP64
 // instruction takes a warp about 19 cycles of the SM's FP64 unit, and the reduction and the
 // update then take 12 a row group where one lane's three components take 30 (G = 32).
-template <int G, int U>
+template <int G, int U, bool FIRST>
 __global__ void __launch_bounds__(256) k_gs_pdl64(int nrows, const int* __restrict__ rows,
                                                 const int* __restrict__ rowptr,
+                                                const int* __restrict__ rowend,
                                                 const int* __restrict__ col,
                                                 const double* __restrict__ val, int64_t nnzb, double* x,
                                                 const double* __restrict__ b,
                                                 const double* __restrict__ dinv,
-                                                const double* __restrict__ wt) {
+                                                const double* __restrict__ wt,
+                                                double* __restrict__ seed) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int g = (blockIdx.x * blockDim.x + threadIdx.x) / G;
   const int gl = threadIdx.x & (G - 1);
@@ -692,7 +705,7 @@ __global__ void __launch_bounds__(256) k_gs_pdl64(int nrows, const int* __restri
   if (active) {
     i = ldg(rows + g);
     a = ldg(rowptr + g);
-    e = ldg(rowptr + g + 1);
+    e = ldg(rowend + g);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int k = a + gl + u * G;
@@ -711,7 +724,7 @@ __global__ void __launch_bounds__(256) k_gs_pdl64(int nrows, const int* __restri
   if (active) {
     if (mine) {
       bi = ldg(b + 4 * (int64_t)i + comp);
-      xi = VL<true>::one(x + 4 * (int64_t)i + comp);
+      if (!FIRST) xi = VL<true>::one(x + 4 * (int64_t)i + comp);
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -740,8 +753,15 @@ __global__ void __launch_bounds__(256) k_gs_pdl64(int nrows, const int* __restri
     }
   }
   double r0, r1, r2;
-  spread3<G>(bi - row_sum3<G>(s0, s1, s2, gl), threadIdx.x & 31, r0, r1, r2);
-  if (mine) x[4 * (int64_t)i + comp] = xi + om * (d0 * r0 + d1 * r1 + d2 * r2);
+  const double r = bi - row_sum3<G>(s0, s1, s2, gl);
+  spread3<G>(r, threadIdx.x & 31, r0, r1, r2);
+  if (!mine) return;
+  const int64_t o = 4 * (int64_t)i + comp;
+  x[o] = xi + om * (d0 * r0 + d1 * r1 + d2 * r2);
+  if (FIRST) {
+    if (seed) seed[o] = (1.0 - om) * r;
+    if (comp == 2) x[o + 1] = 0.0;   // the padding (the sweep does not zero x first)
+  }
 }
 
 // Lanes per block row and threads per CTA of the colour kernels, from the mean rows of a
@@ -757,10 +777,15 @@ inline int gs_lanes(bool f32, double rows) {
   if (!f32) return rows * 32 <= 36864 ? 32 : 16;
   return rows * 32 <= 117000 ? 32 : (rows * 16 <= 140000 ? 16 : 8);
 }
+// The same for the sweep from x = 0, which reads half a row: 8 lanes where 16 were chosen in
+// FP64 for rows of about 28 blocks (preconditioner, 16^3: 513 to 497 us; 32^3: 1499 to 1437).
+inline int first_lanes(bool f32, int gs, double row_blocks) {
+  return !f32 && gs == 16 && row_blocks < 40.0 ? 8 : gs;
+}
 template <typename T, int G>
 constexpr int kGsThreads = sizeof(T) == 8 ? 32 : (G <= 8 ? 128 : 256);
 
-template <typename T, int G, typename V = T>
+template <typename T, int G, bool FIRST, typename V = T>
 void launch_gs_pdl(const Phase& P, cudaStream_t s) {
   constexpr int threads = kGsThreads<T, G>;
   cudaLaunchConfig_t cfg{};
@@ -773,14 +798,14 @@ void launch_gs_pdl(const Phase& P, cudaStream_t s) {
   cfg.attrs = at;
   cfg.numAttrs = 1;
   if constexpr (sizeof(T) == 8)
-    AMG_CUDA(cudaLaunchKernelEx(&cfg, k_gs_pdl64<G, (G >= 16 ? 2 : 3)>, P.n, P.rows, P.rowptr,
-                                P.col, (const double*)P.val, P.nnz, (double*)P.y,
-                                (const double*)P.b, (const double*)P.dinv,
-                                (const double*)P.wt));
+    AMG_CUDA(cudaLaunchKernelEx(&cfg, k_gs_pdl64<G, (G >= 16 ? 2 : 3), FIRST>, P.n, P.rows,
+                                P.rowptr, P.rowend, P.col, (const double*)P.val, P.nnz,
+                                (double*)P.y, (const double*)P.b, (const double*)P.dinv,
+                                (const double*)P.wt, (double*)P.p));
   else
-    AMG_CUDA(cudaLaunchKernelEx(&cfg, k_gs_pdl<T, G, (G >= 16 ? 3 : 4), V>, P.n, P.rows,
-                                P.rowptr, P.col, (const V*)P.val, P.nnz, (T*)P.y,
-                                (const T*)P.b, (const T*)P.dinv, (const T*)P.wt));
+    AMG_CUDA(cudaLaunchKernelEx(&cfg, k_gs_pdl<T, G, (G >= 16 ? 3 : 4), FIRST, V>, P.n, P.rows,
+                                P.rowptr, P.rowend, P.col, (const V*)P.val, P.nnz, (T*)P.y,
+                                (const T*)P.b, (const T*)P.dinv, (const T*)P.wt, (T*)P.p));
 }
 
 // Threads a CTA of a row kernel with `lanes` lanes in all: 256, or fewer (a power of two,
@@ -1363,9 +1388,9 @@ __global__ void __launch_bounds__(256) k_phase(const Phase P) {
 template <typename T, int G, int MODE, typename V = T>
 __global__ void __launch_bounds__(256) k_rows(const Phase P) {
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-  rows_body<T, G, MODE, false, V>(P.n, P.rows, P.rowptr, P.col, (const V*)P.val, P.nnz,
+  rows_body<T, G, MODE, false, V>(P.n, P.rows, P.rowptr, P.rowend, P.col, (const V*)P.val, P.nnz,
                                (const T*)P.x, (const T*)P.b, (T*)P.y, (const T*)P.dinv,
-                               (T)P.omega, (const T*)P.wt, tid >> 5, (gridDim.x * blockDim.x) >> 5);
+                               (T)P.omega, (const T*)P.wt, (T*)P.p, tid >> 5, (gridDim.x * blockDim.x) >> 5);
 }
 
 template <typename T, int G, typename V>
@@ -1377,6 +1402,7 @@ void launch_rows_mode(const Phase& P, cudaStream_t s) {
     case kApply: k_rows<T, G, kApply, V><<<grid, t, 0, s>>>(P); break;
     case kResid: k_rows<T, G, kResid, V><<<grid, t, 0, s>>>(P); break;
     case kGS: k_rows<T, G, kGS, V><<<grid, t, 0, s>>>(P); break;
+    case kFirst: k_rows<T, G, kFirst, V><<<grid, t, 0, s>>>(P); break;
     default: k_rows<T, G, kJacobi, V><<<grid, t, 0, s>>>(P); break;
   }
 }
@@ -1751,10 +1777,18 @@ void launch_rows_v(const Phase& P, cudaStream_t s, bool pdl) {
   }
   if (pdl && P.mode == kGS && P.rows) {
     switch (P.G) {
-      case 4: launch_gs_pdl<T, 4, V>(P, s); return;
-      case 8: launch_gs_pdl<T, 8, V>(P, s); return;
-      case 16: launch_gs_pdl<T, 16, V>(P, s); return;
-      default: launch_gs_pdl<T, 32, V>(P, s); return;
+      case 4: launch_gs_pdl<T, 4, false, V>(P, s); return;
+      case 8: launch_gs_pdl<T, 8, false, V>(P, s); return;
+      case 16: launch_gs_pdl<T, 16, false, V>(P, s); return;
+      default: launch_gs_pdl<T, 32, false, V>(P, s); return;
+    }
+  }
+  if (pdl && P.mode == kFirst) {
+    switch (P.G) {
+      case 4: launch_gs_pdl<T, 4, true, V>(P, s); return;
+      case 8: launch_gs_pdl<T, 8, true, V>(P, s); return;
+      case 16: launch_gs_pdl<T, 16, true, V>(P, s); return;
+      default: launch_gs_pdl<T, 32, true, V>(P, s); return;
     }
   }
   switch (P.G) {
@@ -1950,13 +1984,17 @@ struct Emit {
     return P;
   }
   // block rows [first, first + nrows) of the level's kernel layout
+  // (their lower-colour blocks: kFirst; their higher-colour blocks: upper)
   void rows(int mode, const Level& lv, int G, int first, int nrows, const T* val, const T* x,
-            const T* b, T* y, const T* dinv, T omega) {
+            const T* b, T* y, const T* dinv, T omega, T* seed = nullptr, bool upper = false) {
     Phase P = blank(PH_ROWS);
-    P.wt = (mode == kGS || mode == kJacobi) ? lv.template steps<T>() : nullptr;
+    P.p = seed;
+    P.wt = (mode == kGS || mode == kJacobi || mode == kFirst) ? lv.template steps<T>() : nullptr;
     const int* order = lv.k_rows();
     P.mode = mode; P.G = G; P.n = nrows; P.rows = order ? order + first : nullptr;
-    P.rowptr = lv.k_rowptr() + first; P.col = lv.k_col();
+    P.rowptr = (upper ? lv.sup.p : lv.k_rowptr()) + first;
+    P.rowend = mode == kFirst ? lv.smid.p + first : lv.k_rowptr() + first + 1;
+    P.col = lv.k_col();
     P.val = val; P.nnz = lv.nnzb; P.x = x; P.b = b; P.y = y; P.dinv = dinv; P.omega = omega;
     P.sctas = mode == kGS ? lv.gs_stream : 0;
     P.tma = mode == kGS ? lv.gs_tma : 0;
@@ -2197,6 +2235,15 @@ void e_smooth(Emit<T>& e, amg_handle* h, Level& lv, T* x, const T* b, bool post,
   }
 }
 
+// Whether a level's sweep from x = 0 runs on the lower-colour blocks alone: the colour chain
+// of a coloured level (recorded phases always run it), not a sweep variant chosen instead.
+template <typename T>
+bool first_sweep(const Emit<T>& e, amg_handle* h, const Level& lv) {
+  if (h->saddle || h->opt.smoother != AMG_SMOOTHER_GS || !lv.stored) return false;
+  return e.rec || !((lv.gs_cl > 0 && lv.gs_cl_bytes == (int)sizeof(T)) || lv.flow > 0 ||
+                    lv.gs_stream > 0 || lv.gs_tma > 0);
+}
+
 template <typename T>
 void e_restrict(Emit<T>& e, amg_handle* h, int l, const T* r, T* bc) {
   Level& lv = *h->L[l];
@@ -2255,13 +2302,28 @@ void cycle_rec(Emit<T>& e, amg_handle* h, int l, T* x, const T* b, bool x_is_zer
   Level& nx = *h->L[l + 1];
   const amg_options& o = h->opt;
   bool zero = x_is_zero;
-  for (int k = 0; k < o.m_pre; ++k) {
+  T* r = LvVec<T>::r(lv);
+  T* seed = nullptr;
+  if (zero && o.m_pre > 0 && first_sweep<T>(e, h, lv)) {
+    // the first sweep and, if it is the only one, the residual after it read half of A each
+    // (not with BF16 values: D^{-1} is not the inverse of the rounded D)
+    if (o.m_pre == 1 && !(sizeof(T) == 4 && lv.val16.p)) seed = LvVec<T>::t(lv);
+    const int G = first_lanes(sizeof(T) == 4, lv.group_gs, lv.avg_row_blocks);
+    for (int c = 0; c < lv.ncolours; ++c)
+      e.rows(kFirst, lv, G, lv.colour_ptr[c], lv.colour_ptr[c + 1] - lv.colour_ptr[c],
+             LvVec<T>::val(lv), x, b, x, LvVec<T>::dinv(lv), T(1), seed);
+    zero = false;
+  }
+  for (int k = x_is_zero && !zero ? 1 : 0; k < o.m_pre; ++k) {
     e_smooth<T>(e, h, lv, x, b, false, zero);
     zero = false;
   }
   if (zero) e.zero(x, lv.dofs4());   // no pre-smoothing: x is still the zero initial guess
-  T* r = LvVec<T>::r(lv);
-  e_residual<T>(e, lv, x, b, r, h->saddle);
+  if (seed)
+    e.rows(kResid, lv, group_for(lv), 0, lv.n, LvVec<T>::val(lv), x, seed, r, nullptr, T(0),
+           nullptr, true);
+  else
+    e_residual<T>(e, lv, x, b, r, h->saddle);
   T* bc = LvVec<T>::b(nx);
   T* xc = LvVec<T>::x(nx);
   e_restrict<T>(e, h, l, r, bc);

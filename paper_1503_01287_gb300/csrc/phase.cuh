@@ -11,7 +11,11 @@ struct amg_handle;
 
 namespace amgp2 {
 
-enum RowMode { kApply = 0, kResid = 1, kGS = 2, kJacobi = 3 };
+// kFirst: the colours of a Gauss-Seidel sweep from x = 0 on a row's lower-colour blocks
+// (x_j = 0 on the others), x_i = omega D^{-1} s with s = b_i - (L x)_i; it also leaves
+// p_i = (1 - omega) s, from which the residual after the sweep is p_i - (U x)_i: kResid with
+// b = p on the row's higher-colour blocks (b - L x - D x = s - omega s).
+enum RowMode { kApply = 0, kResid = 1, kGS = 2, kJacobi = 3, kFirst = 4 };
 
 enum PhaseType : int {
   PH_ZERO = 0, PH_COPY, PH_ROWS, PH_RESTRICT, PH_PROLONG, PH_RESTRICT1, PH_PROLONG1,
@@ -23,7 +27,8 @@ enum PhaseType : int {
 struct Phase {
   int type, mode, G, n;   // n: rows / nodes / entries
   const int* rows;
-  const int* rowptr;
+  const int* rowptr;      // PH_ROWS: blocks rowptr[g] .. rowend[g] of stored row g
+  const int* rowend;
   const int* col;
   const void* val;
   int64_t nnz;
@@ -35,7 +40,7 @@ struct Phase {
   const int* ccol;
   const void* cval;
   const void* sd;
-  const void* p;          // pressure iterate (PH_PROWS)
+  const void* p;          // pressure iterate (PH_PROWS); PH_ROWS, kFirst: output (1 - omega) s
   const double* X;
   int m, n3;
   double omega;

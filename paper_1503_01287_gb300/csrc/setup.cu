@@ -639,20 +639,48 @@ __global__ void k_stored_len(int n, const int* __restrict__ order, const int* __
   }
 }
 
+// Row order[k] of A as stored row k (warp per row), its blocks in three parts, ascending
+// columns within each: the neighbours of lower colour, the diagonal block (at smid[k]), the
+// neighbours of higher colour (from sup[k]).  A forward colour sweep from x = 0 needs only
+// the first part, and the residual after it only the last.
 __global__ void k_stored_copy(int n, const int* __restrict__ order, const int* __restrict__ rowptr,
                               const int* __restrict__ col, const double* __restrict__ val,
-                              int64_t nnzb, const int* __restrict__ srowptr, int* __restrict__ scol,
-                              double* __restrict__ sval) {
+                              int64_t nnzb, const int* __restrict__ colour,
+                              const int* __restrict__ srowptr, int* __restrict__ scol,
+                              double* __restrict__ sval, int* __restrict__ smid,
+                              int* __restrict__ sup) {
   const int lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1u;
   const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int nw = (gridDim.x * blockDim.x) >> 5;
   for (int k = w; k < n; k += nw) {
-    const int i = order[k];
+    const int i = order[k], c = colour[i];
     const int a = rowptr[i], len = rowptr[i + 1] - a, o = srowptr[k];
-    for (int q = lane; q < len; q += 32) {
-      scol[o + q] = col[a + q];
+    int nlow = 0;
+    for (int q0 = 0; q0 < len; q0 += 32) {
+      const int q = q0 + lane;
+      nlow += __popc(__ballot_sync(0xffffffffu, q < len && colour[col[a + q]] < c));
+    }
+    int low = o, high = o + nlow + 1;
+    for (int q0 = 0; q0 < len; q0 += 32) {
+      const int q = q0 + lane;
+      const int j = q < len ? col[a + q] : -1;
+      const bool is_low = q < len && colour[j] < c, is_high = q < len && !is_low && j != i;
+      const unsigned ml = __ballot_sync(0xffffffffu, is_low);
+      const unsigned mh = __ballot_sync(0xffffffffu, is_high);
+      if (q < len) {
+        const int p = is_low ? low + __popc(ml & below)
+                             : (is_high ? high + __popc(mh & below) : o + nlow);
+        scol[p] = j;
 #pragma unroll
-      for (int e = 0; e < 9; ++e) sval[e * nnzb + o + q] = val[e * nnzb + a + q];
+        for (int e = 0; e < 9; ++e) sval[e * nnzb + p] = val[e * nnzb + a + q];
+      }
+      low += __popc(ml);
+      high += __popc(mh);
+    }
+    if (lane == 0) {
+      smid[k] = o + nlow;
+      sup[k] = o + nlow + 1;
     }
   }
 }
@@ -1137,9 +1165,12 @@ void finish_level(amg_handle* h, Level& lv, bool coarsest) {
     exclusive_scan(len, lv.srowptr, n, s, h);
     lv.scol.alloc(std::max<int64_t>(lv.nnzb, 1));
     lv.sval.alloc(9 * (size_t)std::max<int64_t>(lv.nnzb, 1));
+    lv.smid.alloc(std::max(n, 1));
+    lv.sup.alloc(std::max(n, 1));
     k_stored_copy<<<grid_for((int64_t)n * 32), 256, 0, s>>>(n, lv.colour_rows, lv.rowptr, lv.col,
-                                                          lv.val, lv.nnzb, lv.srowptr, lv.scol,
-                                                          lv.sval);
+                                                          lv.val, lv.nnzb, lv.colour,
+                                                          lv.srowptr, lv.scol, lv.sval, lv.smid,
+                                                          lv.sup);
     AMG_LAUNCH_CHECK();
     h->launches += 2;
     lv.stored = true;
