@@ -228,6 +228,10 @@ struct amg_handle {
   bool saddle = false;
   cudaStream_t stream = nullptr;
   cudaStream_t own_stream = nullptr;
+  // a second stream for FP64 work beside the pair operator (FGMRES), forked from and joined
+  // to `stream` by the events
+  cudaStream_t side = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
   std::vector<std::unique_ptr<amgp2::Level>> L;
   int coarse_m = 0;
   int coarse_rank = 0;
@@ -244,7 +248,7 @@ struct amg_handle {
   double pmass_sum = 0.0;
   double* host_scal = nullptr;     // pinned
   int* host_int = nullptr;         // pinned
-  amgp2::DBuf<int> it_dev;         // device iteration counter of the graph loop
+  amgp2::DBuf<int> it_dev;         // device: iteration counter of the graph loop, ticket
   cudaGraphExec_t cg_loop_pcg = nullptr, cg_loop_fcg = nullptr;   // whole-solve loops
   int64_t cg_loop_pcg_launches = 0, cg_loop_fcg_launches = 0;
   bool cg_loop_failed = false;
@@ -313,6 +317,13 @@ void precondition_device(amg_handle* h, const double* r, double* z);
 // planes, x as 8 floats a node: hi x,y,z,0 then lo x,y,z,0); y padded FP64
 void apply_pair(amg_handle* h, const float* xp, double* y);
 void apply_K_pair(amg_handle* h, const double* x, float* xp, double* y);
+// The same in parts for a float x (padded): the velocity block as pairs, yp = A x; and on
+// stream s B^T p as pairs (4 n entries, t: two floats an entry) and B u - C p (FP64, y at
+// 4 n) of the padded FP64 vector z
+void apply_pair_f32(amg_handle* h, const float* x, float2* yp);
+void apply_B_parts(amg_handle* h, const double* z, float* t, double* y, cudaStream_t s);
+// x32 = M^{-1} b32 on the level-0 vectors of an FP32 handle
+void precondition_f32(amg_handle* h);
 // the 8-floats-a-node pair form of a padded FP64 vector of n4 = 4 n entries
 void launch_split_pair(const double* x, float* xp, int64_t n4, cudaStream_t s, amg_handle* h);
 // restriction (restrict = true) or prolongation between level and level+1 on

@@ -68,6 +68,9 @@ amg_handle::~amg_handle() {
   if (cg_loop_fcg) cudaGraphExecDestroy(cg_loop_fcg);
   L.clear();
   coarse_inv.release();
+  if (fork) cudaEventDestroy(fork);
+  if (join) cudaEventDestroy(join);
+  if (side) cudaStreamDestroy(side);
   if (own_stream) cudaStreamDestroy(own_stream);
 }
 

@@ -138,6 +138,14 @@ __global__ void __launch_bounds__(kColThreads) k_cols_rows(const Phase P, int W)
   for (int u = 0; u < A; ++u)
 #pragma unroll
     for (int q = 0; q < 3; ++q) s[u][q] = zero<T>();
+  if (P.crow) {   // saddle levels: with B^T p
+    const S* bv = (const S*)P.cval;
+    for (int t = P.crow[i]; t < P.crow[i + 1]; ++t) {
+      const Cell<T> p = ldc((const T*)P.sd + c + (int64_t)P.ccol[t] * W);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) axpy(s[1][q], __ldg(bv + (int64_t)q * P.n3 + t), p);
+    }
+  }
   for (int k0 = a; k0 < e; k0 += kStage) {
     const int n = min(kStage, e - k0);
     __syncthreads();
@@ -192,7 +200,7 @@ __global__ void __launch_bounds__(kColThreads) k_cols_rows(const Phase P, int W)
   }
   if (P.mode == kResid) return;
   const S* wt = (const S*)P.wt;
-  const S om = wt ? wt[P.mode == kJacobi ? 2 : 0] : (S)P.omega;
+  const S om = wt ? wt[0] : (S)P.omega;
   const S* d = (const S*)P.dinv + 12 * (int64_t)i;
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
@@ -232,6 +240,20 @@ __global__ void __launch_bounds__(kColThreads) k_cols_phase(const Phase P, int W
     case PH_COPY: stc(y + o, ldc(x + o)); break;
     case PH_RESTRICT:
     case PH_PROLONG: {
+      if (i >= P.n) {   // the pressure rows of a saddle level's transfer
+        const int k = i - P.n;
+        const int64_t d = (4 * (int64_t)P.n + k) * W;
+        Cell<T> s = zero<T>();
+        for (int t = P.crow[k]; t < P.crow[k + 1]; ++t)
+          axpy(s, ((const S*)P.cval)[t], ldc(x + (4 * (int64_t)P.n3 + P.ccol[t]) * W));
+        if (P.type == PH_PROLONG) {
+          Cell<T> v = ldc(b + d);
+          axpy(v, wt ? wt[1] : S(1), norm(s));
+          s = v;
+        }
+        stc(y + d, s);
+        break;
+      }
       Cell<T> s[3] = {zero<T>(), zero<T>(), zero<T>()};
       for (int t = P.rowptr[i]; t < P.rowptr[i + 1]; ++t) {
         const int64_t j = 4 * (int64_t)P.col[t] * W;
@@ -242,7 +264,7 @@ __global__ void __launch_bounds__(kColThreads) k_cols_phase(const Phase P, int W
 #pragma unroll
       for (int q = 0; q < 3; ++q) {
         if (P.type == PH_PROLONG) {
-          Cell<T> v = ldc(y + o4 + q * W);
+          Cell<T> v = ldc(b + o4 + q * W);
           axpy(v, wc, norm(s[q]));
           s[q] = v;
         }
@@ -300,7 +322,7 @@ __global__ void __launch_bounds__(kColThreads) k_cols_phase(const Phase P, int W
 #pragma unroll
         for (int q = 0; q < 3; ++q) axpy(s, val[q * P.nnz + t], ldc(x + j + q * W));
       }
-      if (P.mode != 3)
+      if (P.mode != 3 && P.mode != 4)
         for (int t = P.crow[i]; t < P.crow[i + 1]; ++t)
           axpy(cp, ((const S*)P.cval)[t], ldc(p + (int64_t)P.ccol[t] * W));
       axpy(s, S(-1), norm(cp));                        // B u - C p
@@ -310,12 +332,12 @@ __global__ void __launch_bounds__(kColThreads) k_cols_phase(const Phase P, int W
         s = g;
       } else if (P.mode == 3) {
         axpy(s, S(-1), ldc(b + o));
-      } else if (P.mode == 2) {
+      } else if (P.mode == 2 || P.mode == 4) {
         const S om = wt ? wt[3] : (S)P.omega;
         const S d = ((const S*)P.sd)[i];
         axpy(s, S(-1), ldc(b + o));
         s = norm(s);
-        Cell<T> v = ldc(p + o);
+        Cell<T> v = P.mode == 2 ? ldc(p + o) : zero<T>();
         if (d != S(0)) {
 #pragma unroll
           for (int q = 0; q < kColN; ++q) add(v.v[q], scaled(om, s.v[q], d));
@@ -421,7 +443,9 @@ void run_cols(amg_handle* h, const Phase& P, int W) {
     if (P.n > 0) AMG_CUDA(cudaMemsetAsync(P.y, 0, (size_t)P.n * W * sizeof(T), s));
     return;
   }
-  const int items = P.type == PH_COARSE ? P.m : P.n;
+  const int items = P.type == PH_COARSE                              ? P.m
+                    : P.type == PH_RESTRICT || P.type == PH_PROLONG ? P.n + P.m
+                                                                     : P.n;
   if (items <= 0) return;
   const dim3 grid(items, W / kColBlock);
   if (P.type != PH_ROWS) {
@@ -455,7 +479,8 @@ void build(amg_handle* h, const CoarseMap& map, S* M) {
   v.use(lb);
   v.use(lx);
   for (const Phase& P : ph)
-    for (const void* q : {P.x, P.b, P.p, (const void*)P.y}) v.use(q);
+    for (const void* q : {P.x, P.b, P.p, (const void*)P.y, P.type == PH_ROWS ? P.sd : nullptr})
+      v.use(q);
   v.mem.alloc((size_t)v.total * W);
   T* b = v.map(lb, W);
   T* x = v.map(lx, W);
@@ -463,6 +488,7 @@ void build(amg_handle* h, const CoarseMap& map, S* M) {
     for (const void** q : {&P.x, &P.b, &P.p})
       if (*q) *q = v.map(*q, W);
     P.y = v.map(P.y, W);
+    if (P.type == PH_ROWS && P.sd) P.sd = v.map(P.sd, W);
   }
   AMG_CUDA(cudaMemsetAsync(v.mem.p, 0, v.mem.bytes(), h->stream));
   const int n3 = 3 * lv.n;

@@ -84,19 +84,27 @@ struct VL<true> {
 //   kJacobi: y_i = x_i + omega D_i^{-1} (b_i - (A x)_i)
 // Stored row g holds the blocks rowptr[g]..rowptr[g+1] of node i = rows[g]
 // (i = g when rows is null).  D^{-1} is stored as 3 padded rows per node.
-template <typename T, int G, int MODE, bool COH, typename V = T>
+//   BT (saddle levels, kApply, kResid, kJacobi): (A x)_i with (B^T p)_i added, the row's
+//   entries of B^T shared by the same lanes
+struct BtRow {
+  const int* row;
+  const int* col;
+  const void* val;   // 3 planes of nnz
+  int64_t nnz;
+  const void* p;
+};
+template <typename T, int G, int MODE, bool COH, bool BT, typename V = T>
 __device__ __forceinline__ void rows_body(int nrows, const int* __restrict__ rows,
                                           const int* __restrict__ rowptr,
                                           const int* __restrict__ rowend,
                                           const int* __restrict__ col,
                                           const V* __restrict__ val, int64_t nnzb, const T* x,
                                           const T* b, T* y, const T* __restrict__ dinv,
-                                          T omega, const T* __restrict__ wt, T* seed, int warp,
-                                          int nwarps) {
+                                          T omega, const T* __restrict__ wt, T* seed, BtRow bt,
+                                          int warp, int nwarps) {
   constexpr int RPW = 32 / G;
   // relaxation: the level's step, weights included (Level::wt), else omega
-  if ((MODE == kGS || MODE == kJacobi || MODE == kFirst) && wt)
-    omega = wt[MODE == kJacobi ? 2 : 0];
+  if ((MODE == kGS || MODE == kJacobi || MODE == kFirst) && wt) omega = wt[0];
   const int lane = threadIdx.x & 31;
   const int sub = lane / G, gl = lane & (G - 1);
   for (int base = warp * RPW; base < nrows; base += nwarps * RPW) {
@@ -106,13 +114,15 @@ __device__ __forceinline__ void rows_body(int nrows, const int* __restrict__ row
     T s0 = T(0), s1 = T(0), s2 = T(0);
     // operands of the row update that depend only on the row: loaded before the
     // row's blocks so that they are not on the critical path
-    using End = RowEnd<T, G>;
-    T bi[End::N] = {}, xi[End::N] = {};
+    // (kJacobi: D^{-1} too, one row a lane, so that a row ends without another load)
+    using End = RowEnd<T, G, MODE == kJacobi>;
+    T bi[End::N] = {}, xi[End::N] = {}, dj[3] = {};
     if (active) {
       i = rows ? ldg(rows + g) : g;
       if (MODE != kApply && End::holds(gl)) {
         End::template load<VL<COH>>(b, i, gl, bi);
         if (MODE != kResid && MODE != kFirst) End::template load<VL<COH>>(x, i, gl, xi);
+        if (MODE == kJacobi) End::load_dinv_row(dinv, i, gl, 0, dj);
       }
       const int a = ldg(rowptr + g), e = ldg(rowend + g);
       // U blocks per lane per step: all column indices of the step are loaded
@@ -154,6 +164,15 @@ __device__ __forceinline__ void rows_body(int nrows, const int* __restrict__ row
         }
       }
     }
+    if (BT && active && bt.row) {
+      const T* bv = (const T*)bt.val;
+      for (int q = ldg(bt.row + i) + gl, qe = ldg(bt.row + i + 1); q < qe; q += G) {
+        const T pk = VL<COH>::one((const T*)bt.p + ldg(bt.col + q));
+        s0 = fma(ldg(bv + q), pk, s0);
+        s1 = fma(ldg(bv + bt.nnz + q), pk, s1);
+        s2 = fma(ldg(bv + 2 * bt.nnz + q), pk, s2);
+      }
+    }
     T v[End::N];
     End::sum(s0, s1, s2, gl, v);
     if (MODE != kApply) {
@@ -173,8 +192,8 @@ __device__ __forceinline__ void rows_body(int nrows, const int* __restrict__ row
       if (End::holds(gl)) {
 #pragma unroll
         for (int q = 0; q < End::N; ++q) {
-          T d[3];
-          End::load_dinv_row(dinv, i, gl, q, d);
+          T d[3] = {dj[0], dj[1], dj[2]};
+          if (MODE != kJacobi) End::load_dinv_row(dinv, i, gl, q, d);
           v[q] = xi[q] + omega * (d[0] * r0 + d[1] * r1 + d[2] * r2);
         }
       }
@@ -185,13 +204,31 @@ __device__ __forceinline__ void rows_body(int nrows, const int* __restrict__ row
   }
 }
 
-// R = P^T gather: bc_I = sum_t w_t r_{i_t} (3 components, same weight)
+// The pressure part of a transfer between saddle levels, done by the same launch: rows 0..n
+// of H^T (restriction) or H (prolongation), vectors at the given offsets
+struct PRows {
+  int n;
+  const int* row;
+  const int* col;
+  const void* val;
+};
+
+// R = P^T gather: bc_I = sum_t w_t r_{i_t} (3 components, same weight); then the pressure
+// rows (r_p at r + 4 nf, result at bc + 4 nc)
 template <typename T, bool COH>
-__device__ __forceinline__ void restrict_body(int nc, const int* __restrict__ rrow,
+__device__ __forceinline__ void restrict_body(int nc, int nf, const int* __restrict__ rrow,
                                               const int* __restrict__ rcol,
                                               const T* __restrict__ rval, const T* r, T* bc,
-                                              int tid, int nthr) {
-  for (int I = tid; I < nc; I += nthr) {
+                                              PRows h, int tid, int nthr) {
+  for (int I = tid; I < nc + h.n; I += nthr) {
+    if (I >= nc) {
+      const int k = I - nc;
+      T s = T(0);
+      for (int t = h.row[k]; t < h.row[k + 1]; ++t)
+        s = fma(((const T*)h.val)[t], VL<COH>::one(r + 4 * (int64_t)nf + h.col[t]), s);
+      bc[4 * (int64_t)nc + k] = s;
+      continue;
+    }
     T s0 = T(0), s1 = T(0), s2 = T(0);
     for (int t = rrow[I]; t < rrow[I + 1]; ++t) {
       const int i = rcol[t];
@@ -206,15 +243,26 @@ __device__ __forceinline__ void restrict_body(int nc, const int* __restrict__ rr
   }
 }
 
-// x_i += sum_q P_iq xc_q
+// y_i = x_i + w_c sum_q P_iq xc_q (y may be x), then the pressure rows (xc_p at xc + 4 nc,
+// the others at 4 n)
 template <typename T, bool COH>
-__device__ __forceinline__ void prolong_body(int n, const int* __restrict__ prow,
+__device__ __forceinline__ void prolong_body(int n, int nc, const int* __restrict__ prow,
                                              const int* __restrict__ pcol,
-                                             const T* __restrict__ pval, const T* xc, T* x,
-                                             const T* __restrict__ wt, int tid, int nthr) {
+                                             const T* __restrict__ pval, const T* xc, const T* x,
+                                             T* y, const T* __restrict__ wt, PRows h, int tid,
+                                             int nthr) {
   // coarse-grid correction x += w_c P x_c (w_c = 1 for the plain method)
   const T wc = wt ? wt[1] : T(1);
-  for (int i = tid; i < n; i += nthr) {
+  for (int i = tid; i < n + h.n; i += nthr) {
+    if (i >= n) {
+      const int k = i - n;
+      const int64_t o = 4 * (int64_t)n + k;
+      T s = T(0);
+      for (int q = h.row[k]; q < h.row[k + 1]; ++q)
+        s = fma(((const T*)h.val)[q], VL<COH>::one(xc + 4 * (int64_t)nc + h.col[q]), s);
+      y[o] = VL<COH>::one(x + o) + wc * s;
+      continue;
+    }
     T s0 = T(0), s1 = T(0), s2 = T(0);
     for (int q = prow[i]; q < prow[i + 1]; ++q) {
       const int J = pcol[q];
@@ -227,7 +275,7 @@ __device__ __forceinline__ void prolong_body(int n, const int* __restrict__ prow
     }
     T x0, x1, x2;
     VL<COH>::node(x, i, x0, x1, x2);
-    st3(x, i, x0 + wc * s0, x1 + wc * s1, x2 + wc * s2);
+    st3(y, i, x0 + wc * s0, x1 + wc * s1, x2 + wc * s2);
   }
 }
 
@@ -310,6 +358,7 @@ __device__ __forceinline__ void bt_add_body(int n, const int* __restrict__ row,
 // MODE 0: yp = B u - C p;  MODE 1: yp = g - B u + C p (residual);
 // MODE 2: yp = p + omega (B u - C p - g) / S_D (sGS pressure step);
 // MODE 3: yp = B u - g (Braess-Sarazin: g holds the pressure residual)
+// MODE 4: yp = omega (B u - g) / S_D (the sGS pressure step from p = 0)
 // The pressure rows: kProwLanes consecutive lanes share a row (its B entries and then
 // its C entries taken in strides of kProwLanes, the lane sums combined by shuffles),
 // so a row's dependent gather chain is about 1/kProwLanes of its length.
@@ -323,7 +372,7 @@ __device__ __forceinline__ void prows_body(int np, const int* __restrict__ brow,
                                            const T* __restrict__ cval, const T* u, const T* p,
                                            const T* g, T* yp, const T* __restrict__ sd, T omega,
                                            const T* __restrict__ wt, int tid, int nthr) {
-  if (MODE == 2 && wt) omega = wt[3];
+  if ((MODE == 2 || MODE == 4) && wt) omega = wt[3];
   constexpr int L = kProwLanes;
   const int gl = tid & (L - 1);
   const unsigned gmask = ((1u << L) - 1u) << (threadIdx.x & 31 & ~(L - 1));
@@ -338,7 +387,7 @@ __device__ __forceinline__ void prows_body(int np, const int* __restrict__ brow,
       s = fma(bval[2 * bnnz + q], u2, s);
     }
     T cp = T(0);
-    if (MODE != 3)
+    if (MODE != 3 && MODE != 4)
       for (int q = crow[k] + gl; q < crow[k + 1]; q += L)
         cp = fma(cval[q], VL<COH>::one(p + ccol[q]), cp);
 #pragma unroll
@@ -356,7 +405,7 @@ __device__ __forceinline__ void prows_body(int np, const int* __restrict__ brow,
     } else {
       const T d = sd[k];
       const T r = s - cp - VL<COH>::one(g + k);
-      yp[k] = VL<COH>::one(p + k) + (d != T(0) ? omega * r / d : T(0));
+      yp[k] = (MODE == 4 ? T(0) : VL<COH>::one(p + k)) + (d != T(0) ? omega * r / d : T(0));
     }
   }
 }
@@ -477,9 +526,10 @@ __device__ void dispatch_rows_v(const Phase& P, int warp, int nwarps) {
   T* y = (T*)P.y;
   const T* d = (const T*)P.dinv;
   const T om = (T)P.omega;
+  const BtRow bt{P.crow, P.ccol, P.cval, P.n3, P.sd};
 #define AMG_ROWS_MODE(GG, MM)                                                                   \
-  rows_body<T, GG, MM, COH, V>(P.n, P.rows, P.rowptr, P.rowend, P.col, val, P.nnz, x, b, y, d, \
-                               om, (const T*)P.wt, (T*)P.p, warp, nwarps)
+  rows_body<T, GG, MM, COH, true, V>(P.n, P.rows, P.rowptr, P.rowend, P.col, val, P.nnz, x, b,  \
+                                     y, d, om, (const T*)P.wt, (T*)P.p, bt, warp, nwarps)
 #define AMG_ROWS_G(GG)                              \
   switch (P.mode) {                                 \
     case kApply: AMG_ROWS_MODE(GG, kApply); break;  \
@@ -509,20 +559,22 @@ __device__ void dispatch_rows(const Phase& P, int warp, int nwarps) {
   dispatch_rows_v<T, COH, T>(P, warp, nwarps);
 }
 
-template <typename T, bool COH>
+// TYPE: the phase's type where the caller knows it (its own kernel then), else -1
+template <typename T, bool COH, int TYPE = -1>
 __device__ __forceinline__ void exec_phase(const Phase& P, int tid, int nthr) {
   const int warp = tid >> 5, nwarps = nthr >> 5;
-  switch (P.type) {
+  const PRows hp{P.m, P.crow, P.ccol, P.cval};
+  switch (TYPE >= 0 ? TYPE : P.type) {
     case PH_ZERO: zero_body<T>((T*)P.y, P.n, tid, nthr); break;
     case PH_COPY: copy_body<T, COH>((const T*)P.x, (T*)P.y, P.n, tid, nthr); break;
     case PH_ROWS: dispatch_rows<T, COH>(P, warp, nwarps); break;
     case PH_RESTRICT:
-      restrict_body<T, COH>(P.n, P.rowptr, P.col, (const T*)P.val, (const T*)P.x, (T*)P.y, tid,
-                            nthr);
+      restrict_body<T, COH>(P.n, P.n3, P.rowptr, P.col, (const T*)P.val, (const T*)P.x, (T*)P.y,
+                            hp, tid, nthr);
       break;
     case PH_PROLONG:
-      prolong_body<T, COH>(P.n, P.rowptr, P.col, (const T*)P.val, (const T*)P.x, (T*)P.y, (const T*)P.wt,
-                           tid, nthr);
+      prolong_body<T, COH>(P.n, P.n3, P.rowptr, P.col, (const T*)P.val, (const T*)P.x,
+                           (const T*)P.b, (T*)P.y, (const T*)P.wt, hp, tid, nthr);
       break;
     case PH_RESTRICT1:
       restrict1_body<T, COH>(P.n, P.rowptr, P.col, (const T*)P.val, (const T*)P.x, (T*)P.y, tid,
@@ -550,7 +602,8 @@ __device__ __forceinline__ void exec_phase(const Phase& P, int tid, int nthr) {
       if (P.mode == 0) AMG_PROWS(0);
       else if (P.mode == 1) AMG_PROWS(1);
       else if (P.mode == 2) AMG_PROWS(2);
-      else AMG_PROWS(3);
+      else if (P.mode == 3) AMG_PROWS(3);
+      else AMG_PROWS(4);
 #undef AMG_PROWS
       break;
     }
@@ -1254,13 +1307,14 @@ int gs_cluster_fits_level(const Level& lv, int cs, int G) {
 // One group of G lanes per block row (rows in the level's kernel layout, as the
 // FP64 operator kernel); each lane takes U blocks per step; x gathers are two
 // 16-byte loads (hi and lo of the node).
-template <int G, int U>
-__global__ void __launch_bounds__(256) k_apply_pair(int nrows, const int* __restrict__ rows,
-                                                    const int* __restrict__ rowptr,
-                                                    const int* __restrict__ col,
-                                                    const float2* __restrict__ val, int64_t nnzb,
-                                                    const float* __restrict__ xp,
-                                                    double* __restrict__ y) {
+// F32X: x is a padded float vector (no low parts), and y is left in pairs: the FGMRES
+// operator on the FP32 cycle's result.
+template <int G, int U, bool F32X>
+__global__ void __launch_bounds__(256) k_apply_pair(
+    int nrows, const int* __restrict__ rows, const int* __restrict__ rowptr,
+    const int* __restrict__ col, const float2* __restrict__ val, int64_t nnzb,
+    const float* __restrict__ xp,
+    std::conditional_t<F32X, float2, double>* __restrict__ y) {
   constexpr int RPW = 32 / G;
   const int lane = threadIdx.x & 31, sub = lane / G, gl = lane & (G - 1);
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -1287,17 +1341,30 @@ __global__ void __launch_bounds__(256) k_apply_pair(int nrows, const int* __rest
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           if (k0 + u * G >= e) continue;
-          const float4 hi = __ldg(xv + 2 * (int64_t)j[u]);
-          const float4 lo = __ldg(xv + 2 * (int64_t)j[u] + 1);
-          pair_fma(S0, s0, v[u][0], hi.x, lo.x);
-          pair_fma(S0, s0, v[u][1], hi.y, lo.y);
-          pair_fma(S0, s0, v[u][2], hi.z, lo.z);
-          pair_fma(S1, s1, v[u][3], hi.x, lo.x);
-          pair_fma(S1, s1, v[u][4], hi.y, lo.y);
-          pair_fma(S1, s1, v[u][5], hi.z, lo.z);
-          pair_fma(S2, s2, v[u][6], hi.x, lo.x);
-          pair_fma(S2, s2, v[u][7], hi.y, lo.y);
-          pair_fma(S2, s2, v[u][8], hi.z, lo.z);
+          if constexpr (F32X) {
+            const float4 hi = __ldg(xv + j[u]);
+            pair_fma(S0, s0, v[u][0], hi.x);
+            pair_fma(S0, s0, v[u][1], hi.y);
+            pair_fma(S0, s0, v[u][2], hi.z);
+            pair_fma(S1, s1, v[u][3], hi.x);
+            pair_fma(S1, s1, v[u][4], hi.y);
+            pair_fma(S1, s1, v[u][5], hi.z);
+            pair_fma(S2, s2, v[u][6], hi.x);
+            pair_fma(S2, s2, v[u][7], hi.y);
+            pair_fma(S2, s2, v[u][8], hi.z);
+          } else {
+            const float4 hi = __ldg(xv + 2 * (int64_t)j[u]);
+            const float4 lo = __ldg(xv + 2 * (int64_t)j[u] + 1);
+            pair_fma(S0, s0, v[u][0], hi.x, lo.x);
+            pair_fma(S0, s0, v[u][1], hi.y, lo.y);
+            pair_fma(S0, s0, v[u][2], hi.z, lo.z);
+            pair_fma(S1, s1, v[u][3], hi.x, lo.x);
+            pair_fma(S1, s1, v[u][4], hi.y, lo.y);
+            pair_fma(S1, s1, v[u][5], hi.z, lo.z);
+            pair_fma(S2, s2, v[u][6], hi.x, lo.x);
+            pair_fma(S2, s2, v[u][7], hi.y, lo.y);
+            pair_fma(S2, s2, v[u][8], hi.z, lo.z);
+          }
         }
       }
     }
@@ -1305,17 +1372,49 @@ __global__ void __launch_bounds__(256) k_apply_pair(int nrows, const int* __rest
                                       make_float2(S2, s2), gl);
     if (!active) continue;
     const int64_t o = 4 * (int64_t)(rows ? __ldg(rows + g) : g);
-    if (holds_component<G>(gl)) y[o + component_of<G>(gl)] = (double)s.x + (double)s.y;
-    else if (gl == G - 1) y[o + 3] = 0.0;
+    if constexpr (F32X) {
+      if (holds_component<G>(gl)) y[o + component_of<G>(gl)] = norm_pair(s.x, s.y);
+      else if (gl == G - 1) y[o + 3] = make_float2(0.f, 0.f);
+    } else {
+      if (holds_component<G>(gl)) y[o + component_of<G>(gl)] = from_pair(s);
+      else if (gl == G - 1) y[o + 3] = 0.0;
+    }
   }
 }
 
-template <int G>
-void launch_apply_pair(const Level& lv, const float* xp, double* y, cudaStream_t s) {
+template <int G, bool F32X, typename Y>
+void launch_apply_pair(const Level& lv, const float* xp, Y* y, cudaStream_t s) {
   constexpr int U = G >= 16 ? 1 : 2;
   const int grid = (int)std::max<int64_t>(1, ((int64_t)lv.n * G + 255) / 256);
-  k_apply_pair<G, U><<<grid, 256, 0, s>>>(lv.n, lv.k_rows(), lv.k_rowptr(), lv.k_col(),
-                                          lv.val2.p, lv.nnzb, xp, y);
+  k_apply_pair<G, U, F32X><<<grid, 256, 0, s>>>(lv.n, lv.k_rows(), lv.k_rowptr(), lv.k_col(),
+                                                lv.val2.p, lv.nnzb, xp, y);
+}
+template <bool F32X, typename Y>
+void launch_apply_pair(const Level& lv, const float* xp, Y* y, cudaStream_t s) {
+  switch (lv.group_pair) {
+    case 4: launch_apply_pair<4, F32X>(lv, xp, y, s); break;
+    case 8: launch_apply_pair<8, F32X>(lv, xp, y, s); break;
+    case 32: launch_apply_pair<32, F32X>(lv, xp, y, s); break;
+    default: launch_apply_pair<16, F32X>(lv, xp, y, s); break;
+  }
+}
+
+// (B^T p)_i as pairs (summed in FP64), thread per velocity node
+__global__ void k_bt_pair(int n, const int* __restrict__ row, const int* __restrict__ col,
+                          const double* __restrict__ val, int64_t nnz,
+                          const double* __restrict__ p, float4* __restrict__ t) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+    for (int q = row[i]; q < row[i + 1]; ++q) {
+      const double pk = __ldg(p + col[q]);
+      s0 = fma(val[q], pk, s0);
+      s1 = fma(val[nnz + q], pk, s1);
+      s2 = fma(val[2 * nnz + q], pk, s2);
+    }
+    const float2 a = to_pair(s0), b = to_pair(s1), c = to_pair(s2);
+    t[2 * (int64_t)i] = make_float4(a.x, a.y, b.x, b.y);
+    t[2 * (int64_t)i + 1] = make_float4(c.x, c.y, 0.f, 0.f);
+  }
 }
 
 // Residual r = b - K x restricted to the unknowns of one Vanka colour: the velocity
@@ -1378,19 +1477,39 @@ __global__ void __launch_bounds__(256) k_vk_resid(
   }
 }
 
-// one operation as its own kernel
-template <typename T>
+// one operation as its own kernel (one kernel a type: with all of them in one body the
+// transfers and pressure rows ran at the registers of the widest row operation)
+template <typename T, int TYPE>
 __global__ void __launch_bounds__(256) k_phase(const Phase P) {
-  exec_phase<T, false>(P, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+  exec_phase<T, false, TYPE>(P, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+}
+
+template <typename T>
+void launch_phase(const Phase& P, int grid, cudaStream_t s) {
+  switch (P.type) {
+    case PH_ZERO: k_phase<T, PH_ZERO><<<grid, 256, 0, s>>>(P); break;
+    case PH_COPY: k_phase<T, PH_COPY><<<grid, 256, 0, s>>>(P); break;
+    case PH_RESTRICT: k_phase<T, PH_RESTRICT><<<grid, 256, 0, s>>>(P); break;
+    case PH_PROLONG: k_phase<T, PH_PROLONG><<<grid, 256, 0, s>>>(P); break;
+    case PH_RESTRICT1: k_phase<T, PH_RESTRICT1><<<grid, 256, 0, s>>>(P); break;
+    case PH_PROLONG1: k_phase<T, PH_PROLONG1><<<grid, 256, 0, s>>>(P); break;
+    case PH_COARSE: k_phase<T, PH_COARSE><<<grid, 256, 0, s>>>(P); break;
+    case PH_BT_ADD: k_phase<T, PH_BT_ADD><<<grid, 256, 0, s>>>(P); break;
+    case PH_PROWS: k_phase<T, PH_PROWS><<<grid, 256, 0, s>>>(P); break;
+    case PH_SROWS: k_phase<T, PH_SROWS><<<grid, 256, 0, s>>>(P); break;
+    default: k_phase<T, PH_VEC><<<grid, 256, 0, s>>>(P); break;
+  }
 }
 
 // the block-row operations as their own specialised kernels (the hot path)
-template <typename T, int G, int MODE, typename V = T>
+template <typename T, int G, int MODE, bool BT, typename V = T>
 __global__ void __launch_bounds__(256) k_rows(const Phase P) {
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-  rows_body<T, G, MODE, false, V>(P.n, P.rows, P.rowptr, P.rowend, P.col, (const V*)P.val, P.nnz,
-                               (const T*)P.x, (const T*)P.b, (T*)P.y, (const T*)P.dinv,
-                               (T)P.omega, (const T*)P.wt, (T*)P.p, tid >> 5, (gridDim.x * blockDim.x) >> 5);
+  const BtRow bt{P.crow, P.ccol, P.cval, P.n3, P.sd};
+  rows_body<T, G, MODE, false, BT, V>(P.n, P.rows, P.rowptr, P.rowend, P.col, (const V*)P.val,
+                                      P.nnz, (const T*)P.x, (const T*)P.b, (T*)P.y,
+                                      (const T*)P.dinv, (T)P.omega, (const T*)P.wt, (T*)P.p, bt,
+                                      tid >> 5, (gridDim.x * blockDim.x) >> 5);
 }
 
 template <typename T, int G, typename V>
@@ -1398,12 +1517,20 @@ void launch_rows_mode(const Phase& P, cudaStream_t s) {
   // one group of G lanes per row
   const int t = row_threads((int64_t)P.n * G);
   const int grid = (int)(((int64_t)P.n * G + t - 1) / t);
+  if (P.crow) {
+    switch (P.mode) {
+      case kApply: k_rows<T, G, kApply, true, V><<<grid, t, 0, s>>>(P); break;
+      case kResid: k_rows<T, G, kResid, true, V><<<grid, t, 0, s>>>(P); break;
+      default: k_rows<T, G, kJacobi, true, V><<<grid, t, 0, s>>>(P); break;
+    }
+    return;
+  }
   switch (P.mode) {
-    case kApply: k_rows<T, G, kApply, V><<<grid, t, 0, s>>>(P); break;
-    case kResid: k_rows<T, G, kResid, V><<<grid, t, 0, s>>>(P); break;
-    case kGS: k_rows<T, G, kGS, V><<<grid, t, 0, s>>>(P); break;
-    case kFirst: k_rows<T, G, kFirst, V><<<grid, t, 0, s>>>(P); break;
-    default: k_rows<T, G, kJacobi, V><<<grid, t, 0, s>>>(P); break;
+    case kApply: k_rows<T, G, kApply, false, V><<<grid, t, 0, s>>>(P); break;
+    case kResid: k_rows<T, G, kResid, false, V><<<grid, t, 0, s>>>(P); break;
+    case kGS: k_rows<T, G, kGS, false, V><<<grid, t, 0, s>>>(P); break;
+    case kFirst: k_rows<T, G, kFirst, false, V><<<grid, t, 0, s>>>(P); break;
+    default: k_rows<T, G, kJacobi, false, V><<<grid, t, 0, s>>>(P); break;
   }
 }
 
@@ -1783,7 +1910,7 @@ void launch_rows_v(const Phase& P, cudaStream_t s, bool pdl) {
       default: launch_gs_pdl<T, 32, false, V>(P, s); return;
     }
   }
-  if (pdl && P.mode == kFirst) {
+  if (pdl && P.mode == kFirst && P.rows) {
     switch (P.G) {
       case 4: launch_gs_pdl<T, 4, true, V>(P, s); return;
       case 8: launch_gs_pdl<T, 8, true, V>(P, s); return;
@@ -1974,7 +2101,7 @@ struct Emit {
       k_vanka<T><<<(unsigned)std::min<int64_t>(work, 152 * 8), 256, 0, h->stream>>>(
           P.n, P.rows, P.rowptr, P.col, (const T*)P.val, P.nnz, P.off, (const T*)P.dinv,
           (const T*)P.cval, (const T*)P.sd, (const T*)P.x, (T*)P.y, P.n3, (T)P.omega);
-    else k_phase<T><<<gridn(work * threads_per_item), 256, 0, h->stream>>>(P);
+    else launch_phase<T>(P, gridn(work * threads_per_item), h->stream);
     h->launches++;
   }
   static Phase blank(int type) {
@@ -1986,10 +2113,17 @@ struct Emit {
   // block rows [first, first + nrows) of the level's kernel layout
   // (their lower-colour blocks: kFirst; their higher-colour blocks: upper)
   void rows(int mode, const Level& lv, int G, int first, int nrows, const T* val, const T* x,
-            const T* b, T* y, const T* dinv, T omega, T* seed = nullptr, bool upper = false) {
+            const T* b, T* y, const T* dinv, T omega, T* seed = nullptr, bool upper = false,
+            const T* bt_p = nullptr) {
     Phase P = blank(PH_ROWS);
     P.p = seed;
-    P.wt = (mode == kGS || mode == kJacobi || mode == kFirst) ? lv.template steps<T>() : nullptr;
+    P.wt = (mode == kGS || mode == kFirst) ? lv.template steps<T>()
+           : mode == kJacobi               ? lv.template steps<T>() + 2
+                                           : nullptr;
+    if (bt_p) {   // with B^T p
+      P.crow = lv.bt_rowptr; P.ccol = lv.bt_col; P.cval = LvVec<T>::btval(const_cast<Level&>(lv));
+      P.n3 = (int)lv.b_nnz; P.sd = bt_p;
+    }
     const int* order = lv.k_rows();
     P.mode = mode; P.G = G; P.n = nrows; P.rows = order ? order + first : nullptr;
     P.rowptr = (upper ? lv.sup.p : lv.k_rowptr()) + first;
@@ -2004,6 +2138,15 @@ struct Emit {
       P.vbf = 1;
     }
     put(P, nrows, G);
+  }
+  // x = omega D^{-1} b on every node: a damped block Jacobi step from x = 0
+  void jacobi_zero(const Level& lv, const T* val, const T* b, T* x, const T* dinv) {
+    Phase P = blank(PH_ROWS);
+    P.mode = kFirst; P.G = 4; P.n = lv.n; P.rowptr = P.rowend = lv.rowptr; P.col = lv.k_col();
+    P.val = val; P.nnz = lv.nnzb; P.x = x; P.b = b; P.y = x; P.dinv = dinv; P.omega = 1.0;
+    P.wt = lv.template steps<T>() + 2;
+    P.err = h->flag.p;
+    put(P, lv.n, P.G);
   }
   // a level's whole colour sweep as one cluster launch (never recorded)
   void gs_cluster(Level& lv, T* x, const T* b, bool post, bool x_zero) {
@@ -2041,6 +2184,28 @@ struct Emit {
     Phase P = blank(type);
     P.n = n; P.rowptr = row; P.col = col; P.val = val; P.x = src; P.y = dst; P.wt = wt;
     put(P, n);
+  }
+  // restriction and prolongation (y = x + w_c P xc) of a level's vectors, the pressure's with
+  // them on saddle levels
+  void restrict_all(const Level& lv, const Level& nx, const T* r, T* bc) {
+    Phase P = blank(PH_RESTRICT);
+    P.n = nx.n; P.n3 = lv.n; P.rowptr = lv.r_rowptr; P.col = lv.r_col; P.x = r; P.y = bc;
+    P.val = LvVec<T>::rval(const_cast<Level&>(lv));
+    if (h->saddle && nx.np > 0) {
+      P.m = nx.np; P.crow = lv.ht_rowptr; P.ccol = lv.ht_col;
+      P.cval = LvVec<T>::htval(const_cast<Level&>(lv));
+    }
+    put(P, nx.n + P.m);
+  }
+  void prolong_all(const Level& lv, const Level& nx, const T* xc, const T* x, T* y) {
+    Phase P = blank(PH_PROLONG);
+    P.n = lv.n; P.n3 = nx.n; P.rowptr = lv.p_rowptr; P.col = lv.p_col; P.x = xc; P.b = x;
+    P.y = y; P.val = LvVec<T>::pval(const_cast<Level&>(lv)); P.wt = lv.template steps<T>();
+    if (h->saddle && lv.np > 0) {
+      P.m = lv.np; P.crow = lv.h_rowptr; P.ccol = lv.h_col;
+      P.cval = LvVec<T>::hval(const_cast<Level&>(lv));
+    }
+    put(P, lv.n + P.m);
   }
   void coarse(const T* b, T* x) {
     Phase P = blank(PH_COARSE);
@@ -2097,7 +2262,7 @@ struct Emit {
     P.val = LvVec<T>::bval(lv); P.nnz = lv.b_nnz; P.crow = lv.c_rowptr; P.ccol = lv.c_col;
     P.cval = LvVec<T>::cval(lv); P.x = u; P.p = p; P.b = g; P.y = yp;
     P.sd = LvVec<T>::schur(lv); P.omega = (double)omega;
-    P.wt = mode == 2 ? lv.template steps<T>() : nullptr;
+    P.wt = mode == 2 || mode == 4 ? lv.template steps<T>() : nullptr;
     put(P, lv.np, kProwLanes);
   }
 };
@@ -2107,22 +2272,37 @@ struct Emit {
 template <typename T>
 void e_apply(Emit<T>& e, Level& lv, const T* x, T* y, bool saddle) {
   const int G = (sizeof(T) == 8 && lv.group64) ? lv.group64 : group_for(lv);
-  e.rows(kApply, lv, G, 0, lv.n, LvVec<T>::val(lv), x, nullptr, y, nullptr, T(0));
-  if (saddle && lv.np > 0) {
-    const T* p = x + 4 * lv.n;
-    e.bt_add(lv, p, T(1), y);
-    e.prows(0, lv, x, p, nullptr, y + 4 * lv.n, T(0));
-  }
+  const T* p = saddle && lv.np > 0 ? x + 4 * (int64_t)lv.n : nullptr;
+  e.rows(kApply, lv, G, 0, lv.n, LvVec<T>::val(lv), x, nullptr, y, nullptr, T(0), nullptr, false,
+         p);
+  if (p) e.prows(0, lv, x, p, nullptr, y + 4 * lv.n, T(0));
 }
 
 template <typename T>
 void e_residual(Emit<T>& e, Level& lv, const T* x, const T* b, T* r, bool saddle) {
-  e.rows(kResid, lv, group_for(lv), 0, lv.n, LvVec<T>::val(lv), x, b, r, nullptr, T(0));
-  if (saddle && lv.np > 0) {
-    const T* p = x + 4 * lv.n;
-    e.bt_add(lv, p, T(-1), r);
-    e.prows(1, lv, x, p, b + 4 * lv.n, r + 4 * lv.n, T(0));
+  const T* p = saddle && lv.np > 0 ? x + 4 * (int64_t)lv.n : nullptr;
+  e.rows(kResid, lv, group_for(lv), 0, lv.n, LvVec<T>::val(lv), x, b, r, nullptr, T(0), nullptr,
+         false, p);
+  if (p) e.prows(1, lv, x, p, b + 4 * lv.n, r + 4 * lv.n, T(0));
+}
+
+// One segregated Gauss-Seidel sweep, Eq. (uzsm), from x to y (other vectors):
+// u <- u + omega D^{-1} (f - B^T p - A u) (M_A: damped block Jacobi),
+// p <- p + omega_p S_D^{-1} (B u_new - C p - g).  From x = 0 the first is omega D^{-1} f, no
+// pass over A, and y may be x.
+template <typename T>
+void e_sgs(Emit<T>& e, amg_handle* h, Level& lv, const T* x, const T* b, T* y, bool zero) {
+  const int64_t n4 = 4 * (int64_t)lv.n;
+  const T* val = LvVec<T>::val(lv);
+  const T* dinv = LvVec<T>::dinv(lv);
+  if (zero) {
+    e.jacobi_zero(lv, val, b, y, dinv);
+    e.prows(4, lv, y, nullptr, b + n4, y + n4, (T)h->opt.omega_p);
+    return;
   }
+  e.rows(kJacobi, lv, group_for(lv), 0, lv.n, val, x, b, y, dinv, (T)h->opt.omega, nullptr, false,
+         x + n4);
+  e.prows(2, lv, y, x + n4, b + n4, y + n4, (T)h->opt.omega_p);
 }
 
 // One V(1,1)-cycle on the S hierarchy of level l from a zero initial guess
@@ -2151,13 +2331,14 @@ void e_scycle(Emit<T>& e, amg_handle* h, int l, int k, const T* rhs) {
 // One Braess-Sarazin step, Eq. (bssm) with K^ of Eq. (bssmpre):
 // r = b - K x; w = A^{-1} r_u; dp = S^{-1}(B w - r_p); x_u += w - A^{-1} B^T dp; p += dp.
 template <typename T>
-void e_smooth_bs(Emit<T>& e, amg_handle* h, int l, T* x, const T* b) {
+void e_smooth_bs(Emit<T>& e, amg_handle* h, int l, T* x, const T* b, bool zero) {
   Level& lv = *h->L[l];
   const int64_t n4 = 4 * (int64_t)lv.n;
   T* r = LvVec<T>::r(lv);
   T* t = LvVec<T>::t(lv);
   const T* ah = SVec<T>::ahinv(lv);
-  e_residual<T>(e, lv, x, b, r, true);
+  if (zero) e.copy(b, r, lv.dofs4());                      // x = 0
+  else e_residual<T>(e, lv, x, b, r, true);
   e.vec(0, n4, ah, r, nullptr, T(1), t);                   // t_u = w
   e.prows(3, lv, t, nullptr, r + n4, t + n4, T(0));         // t_p = B w - r_p
   e_scycle<T>(e, h, l, 0, t + n4);
@@ -2181,7 +2362,10 @@ void e_smooth(Emit<T>& e, amg_handle* h, Level& lv, T* x, const T* b, bool post,
     e.gs_cluster(lv, x, b, post, x_is_zero);
     return;
   }
-  if (x_is_zero) e.zero(x, dofs);
+  // the damped block Jacobi steps (also sGS's) from x = 0 write x without reading it
+  const bool writes = h->saddle ? h->opt.smoother == AMG_SMOOTHER_SGS
+                                : h->opt.smoother == AMG_SMOOTHER_JACOBI;
+  if (x_is_zero && !writes) e.zero(x, dofs);
   if (!e.rec && lv.flow > 0 && !h->saddle && h->opt.smoother == AMG_SMOOTHER_GS &&
       !(sizeof(T) == 4 && lv.val16.p)) {
     e.gs_flow(lv, x, b, post);
@@ -2193,7 +2377,7 @@ void e_smooth(Emit<T>& e, amg_handle* h, Level& lv, T* x, const T* b, bool post,
   if (h->saddle && h->opt.smoother == AMG_SMOOTHER_BS) {
     int l = 0;
     while (h->L[l].get() != &lv) ++l;
-    e_smooth_bs<T>(e, h, l, x, b);
+    e_smooth_bs<T>(e, h, l, x, b, x_is_zero);
     return;
   }
   if (h->saddle && h->opt.smoother == AMG_SMOOTHER_VANKA) {
@@ -2208,20 +2392,20 @@ void e_smooth(Emit<T>& e, amg_handle* h, Level& lv, T* x, const T* b, bool post,
     return;
   }
   if (h->saddle) {
+    if (x_is_zero) {
+      e_sgs<T>(e, h, lv, x, b, x, true);
+      return;
+    }
     T* t = LvVec<T>::t(lv);
-    T* r = LvVec<T>::r(lv);
-    const T* p = x + 4 * lv.n;
-    // u <- u + omega D^{-1} (f - B^T p - A u)    (M_A = damped block Jacobi)
-    e.copy(b, r, 4 * (int64_t)lv.n);
-    e.bt_add(lv, p, T(-1), r);
-    e.rows(kJacobi, lv, G, 0, lv.n, val, x, r, t, dinv, (T)h->opt.omega);
-    e.copy(t, x, 4 * (int64_t)lv.n);
-    // p <- p + omega_p S_D^{-1} (B u_new - C p - g)
-    e.prows(2, lv, x, x + 4 * lv.n, b + 4 * lv.n, t + 4 * lv.n, (T)h->opt.omega_p);
-    e.copy(t + 4 * lv.n, x + 4 * lv.n, lv.np);
+    e_sgs<T>(e, h, lv, x, b, t, false);
+    e.copy(t, x, dofs);
     return;
   }
   if (h->opt.smoother == AMG_SMOOTHER_JACOBI) {
+    if (x_is_zero) {
+      e.jacobi_zero(lv, val, b, x, dinv);
+      return;
+    }
     T* t = LvVec<T>::t(lv);
     e.rows(kJacobi, lv, G, 0, lv.n, val, x, b, t, dinv, (T)h->opt.omega);
     e.copy(t, x, dofs);
@@ -2246,22 +2430,12 @@ bool first_sweep(const Emit<T>& e, amg_handle* h, const Level& lv) {
 
 template <typename T>
 void e_restrict(Emit<T>& e, amg_handle* h, int l, const T* r, T* bc) {
-  Level& lv = *h->L[l];
-  Level& nx = *h->L[l + 1];
-  e.transfer(PH_RESTRICT, nx.n, lv.r_rowptr, lv.r_col, LvVec<T>::rval(lv), r, bc);
-  if (h->saddle && nx.np > 0)
-    e.transfer(PH_RESTRICT1, nx.np, lv.ht_rowptr, lv.ht_col, LvVec<T>::htval(lv), r + 4 * lv.n,
-               bc + 4 * nx.n);
+  e.restrict_all(*h->L[l], *h->L[l + 1], r, bc);
 }
 
 template <typename T>
 void e_prolong(Emit<T>& e, amg_handle* h, int l, const T* xc, T* x) {
-  Level& lv = *h->L[l];
-  Level& nx = *h->L[l + 1];
-  e.transfer(PH_PROLONG, lv.n, lv.p_rowptr, lv.p_col, LvVec<T>::pval(lv), xc, x, lv.template steps<T>());
-  if (h->saddle && lv.np > 0)
-    e.transfer(PH_PROLONG1, lv.np, lv.h_rowptr, lv.h_col, LvVec<T>::hval(lv), xc + 4 * nx.n,
-               x + 4 * lv.n, lv.template steps<T>());
+  e.prolong_all(*h->L[l], *h->L[l + 1], xc, x, x);
 }
 
 template <typename T>
@@ -2303,6 +2477,37 @@ void cycle_rec(Emit<T>& e, amg_handle* h, int l, T* x, const T* b, bool x_is_zer
   const amg_options& o = h->opt;
   bool zero = x_is_zero;
   T* r = LvVec<T>::r(lv);
+  if (h->saddle && o.smoother == AMG_SMOOTHER_SGS) {
+    // the sweeps go from one of x and t to the other, so that the last one ends in x: a first
+    // sweep from zero starts in either, else the prolongation changes sides where it must
+    T* t = LvVec<T>::t(lv);
+    const int sweeps = (zero ? std::max(0, o.m_pre - 1) : o.m_pre) + o.m_post;
+    T* cur = zero && (sweeps & 1) ? t : x;
+    bool flip = !zero && (sweeps & 1);
+    if (zero) {
+      if (o.m_pre > 0) e_sgs<T>(e, h, lv, cur, b, cur, true);
+      else e.zero(cur, lv.dofs4());
+    }
+    for (int k = zero ? 1 : 0; k < o.m_pre; ++k) {
+      T* other = cur == x ? t : x;
+      e_sgs<T>(e, h, lv, cur, b, other, false);
+      cur = other;
+    }
+    e_residual<T>(e, lv, cur, b, r, true);
+    T* bc = LvVec<T>::b(nx);
+    T* xc = LvVec<T>::x(nx);
+    e_restrict<T>(e, h, l, r, bc);
+    coarse_calls<T>(e, h, l + 1, xc, bc);
+    T* other = cur == x ? t : x;
+    e.prolong_all(lv, nx, xc, cur, flip ? other : cur);
+    if (flip) cur = other;
+    for (int k = 0; k < o.m_post; ++k) {
+      other = cur == x ? t : x;
+      e_sgs<T>(e, h, lv, cur, b, other, false);
+      cur = other;
+    }
+    return;
+  }
   T* seed = nullptr;
   if (zero && o.m_pre > 0 && first_sweep<T>(e, h, lv)) {
     // the first sweep and, if it is the only one, the residual after it read half of A each
@@ -2538,6 +2743,19 @@ void precondition_device<double>(amg_handle* h, const double* r, double* z) {
   for (int c = 0; c < std::max(1, h->opt.cycles); ++c) cycle_rec<double>(e, h, 0, z, r, c == 0);
 }
 
+void precondition_f32(amg_handle* h) {
+  Level& lv = *h->L[0];
+  if (h->map.from == 0) {
+    map_apply<float, float>(h, lv.b32.p, lv.x32.p);
+  } else if (h->use_full) {
+    FullCycle<float>::launch(h);
+  } else {
+    Emit<float> e{h};
+    for (int c = 0; c < std::max(1, h->opt.cycles); ++c)
+      cycle_rec<float>(e, h, 0, lv.x32.p, lv.b32.p, c == 0);
+  }
+}
+
 template <>
 void precondition_device<float>(amg_handle* h, const double* r, double* z) {
   if (h->map.from == 0) {
@@ -2547,13 +2765,7 @@ void precondition_device<float>(amg_handle* h, const double* r, double* z) {
   Level& lv = *h->L[0];
   const int64_t n = lv.dofs4();
   launch_to_float(r, lv.b32, n, h->stream, h);
-  if (h->use_full) {
-    FullCycle<float>::launch(h);
-  } else {
-    Emit<float> e{h};
-    for (int c = 0; c < std::max(1, h->opt.cycles); ++c)
-      cycle_rec<float>(e, h, 0, lv.x32.p, lv.b32.p, c == 0);
-  }
+  precondition_f32(h);
   launch_to_double(lv.x32, z, n, h->stream, h);
 }
 
@@ -2561,13 +2773,25 @@ void apply_pair(amg_handle* h, const float* xp, double* y) {
   const Level& lv = *h->L[0];
   if (!lv.val2.p)
     fail(AMG_ERR_INVALID, "the FP32-pair operator needs an FP32 handle with outer_pair");
-  switch (lv.group_pair) {
-    case 4: launch_apply_pair<4>(lv, xp, y, h->stream); break;
-    case 8: launch_apply_pair<8>(lv, xp, y, h->stream); break;
-    case 32: launch_apply_pair<32>(lv, xp, y, h->stream); break;
-    default: launch_apply_pair<16>(lv, xp, y, h->stream); break;
-  }
+  launch_apply_pair<false>(lv, xp, y, h->stream);
   h->launches++;
+}
+
+void apply_pair_f32(amg_handle* h, const float* x, float2* yp) {
+  launch_apply_pair<true>(*h->L[0], x, yp, h->stream);
+  h->launches++;
+}
+
+void apply_B_parts(amg_handle* h, const double* z, float* t, double* y, cudaStream_t s) {
+  Level& lv = *h->L[0];
+  k_bt_pair<<<gridn(lv.n), 256, 0, s>>>(lv.n, lv.bt_rowptr, lv.bt_col, lv.bt_val, lv.b_nnz,
+                                        z + 4 * (int64_t)lv.n, reinterpret_cast<float4*>(t));
+  h->launches++;
+  const cudaStream_t own = h->stream;
+  h->stream = s;
+  Emit<double> e{h};
+  e.prows(0, lv, z, z + 4 * (int64_t)lv.n, nullptr, y + 4 * (int64_t)lv.n, 0.0);
+  h->stream = own;
 }
 
 // y = K_0 x with the velocity block in FP32-pair arithmetic (x split into xp, 8 floats a

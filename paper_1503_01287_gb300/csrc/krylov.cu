@@ -273,18 +273,6 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_mdot2(int64_t n, int64
   }
 }
 
-// FP32 pair of an FP64 value (hi = fl32(d), lo = fl32(d - hi)) and back
-__device__ __forceinline__ float2 to_pair(double d) {
-  const float hi = __double2float_rn(d);
-  return make_float2(hi, __double2float_rn(d - (double)hi));
-}
-__device__ __forceinline__ double from_pair(float2 p) { return (double)p.x + (double)p.y; }
-// a leading sum S and a small error sum s as one normalised pair (FastTwoSum)
-__device__ __forceinline__ float2 norm_pair(float S, float s) {
-  const float hi = __fadd_rn(S, s);
-  return make_float2(hi, __fsub_rn(s, __fsub_rn(hi, S)));
-}
-
 // Coefficients of the update from the sweep's dots (coef: p at [0, kMaxDots), q at
 // [kMaxDots, 2 kMaxDots), u . u at p[m], u . w at q[m]):
 //   s = ||u - V p|| = sqrt(u . u - p . p)   (u - V p is orthogonal to V)
@@ -414,9 +402,13 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_dcgs2_update(int64_t n
   }
 }
 
-// v *= 1 / sqrt(nrm2[0]) (0 if the norm is 0) in pair arithmetic, also written to v2 as
-// FP64 values: normalises the pending vector and stages it as the preconditioner's input
-__global__ void k_scale_norm(int64_t n, float2* __restrict__ v, double* __restrict__ v2,
+// v *= 1 / sqrt(nrm2[0]) (0 if the norm is 0) in pair arithmetic, also written to v2, as FP64
+// values or, for the FP32 cycle, as floats (a normalised pair's high part is its rounding):
+// normalises the pending vector and stages it as the preconditioner's input
+__device__ __forceinline__ void stage(double& o, float2 p) { o = from_pair(p); }
+__device__ __forceinline__ void stage(float& o, float2 p) { o = p.x; }
+template <typename O>
+__global__ void k_scale_norm(int64_t n, float2* __restrict__ v, O* __restrict__ v2,
                              const double* __restrict__ nrm2) {
   const double r = sqrt(fmax(nrm2[0], 0.0));
   const float2 f = to_pair(r > 0.0 ? 1.0 / r : 0.0);
@@ -427,18 +419,19 @@ __global__ void k_scale_norm(int64_t n, float2* __restrict__ v, double* __restri
     pair_fma(P, pl, f, a.x, a.y);
     const float2 t = norm_pair(P, pl);
     v[k] = t;
-    v2[k] = from_pair(t);
+    stage(v2[k], t);
   }
 }
 
-// v = pairs of a * f, v2 = a * f in FP64 (the first basis vector r / ||r||)
+// v = pairs of a * f, v2 = a * f (the first basis vector r / ||r||)
+template <typename O>
 __global__ void k_pair_scaled(int64_t n, const double* __restrict__ a, double f,
-                              float2* __restrict__ v, double* __restrict__ v2) {
+                              float2* __restrict__ v, O* __restrict__ v2) {
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
        k += (int64_t)gridDim.x * blockDim.x) {
     const double t = a[k] * f;
     v[k] = to_pair(t);
-    v2[k] = t;
+    v2[k] = (O)t;
   }
 }
 
@@ -447,6 +440,23 @@ __global__ void k_to_pair(int64_t n, const double* __restrict__ a, float2* __res
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
        k += (int64_t)gridDim.x * blockDim.x)
     b[k] = to_pair(a[k]);
+}
+
+// the parts of w = K z as pairs: velocity entries (k < n4) w_k + t_k, t = B^T p; pressure
+// entries from the FP64 vector d
+__global__ void k_join(int64_t n, int64_t n4, const float2* __restrict__ t,
+                       const double* __restrict__ d, float2* __restrict__ w) {
+  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
+       k += (int64_t)gridDim.x * blockDim.x) {
+    if (k >= n4) {
+      w[k] = to_pair(d[k]);
+      continue;
+    }
+    float2 a = w[k];
+    const float2 b = t[k];
+    pair_add(a.x, a.y, b.x, b.y);
+    w[k] = norm_pair(a.x, a.y);
+  }
 }
 
 // out[d] = sum_blk partial[blk*nd + d] in block order (deterministic)
@@ -528,7 +538,9 @@ __global__ void k_cg_dir_pair(int64_t n, double* __restrict__ p, const double* _
 
 // x += sum_i y[i] Z_i (y staged in shared memory; the basis loads of one index go
 // out eight at a time, the sum keeps the order i = 0, 1, ...)
-__global__ void __launch_bounds__(256) k_basis_add(int64_t n, int m, const double* __restrict__ Z,
+// (Z: the type of the preconditioned vectors, floats with the FP32 cycle)
+template <typename ZT>
+__global__ void __launch_bounds__(256) k_basis_add(int64_t n, int m, const ZT* __restrict__ Z,
                                                    int64_t ldz, const double* __restrict__ y,
                                                    double* __restrict__ x) {
   __shared__ double ys[kMaxDots];
@@ -541,11 +553,11 @@ __global__ void __launch_bounds__(256) k_basis_add(int64_t n, int m, const doubl
     for (; i + 8 <= m; i += 8) {
       double v[8];
 #pragma unroll
-      for (int g = 0; g < 8; ++g) v[g] = Z[(int64_t)(i + g) * ldz + k];
+      for (int g = 0; g < 8; ++g) v[g] = (double)Z[(int64_t)(i + g) * ldz + k];
 #pragma unroll
       for (int g = 0; g < 8; ++g) acc = fma(ys[i + g], v[g], acc);
     }
-    for (; i < m; ++i) acc = fma(ys[i], Z[(int64_t)i * ldz + k], acc);
+    for (; i < m; ++i) acc = fma(ys[i], (double)Z[(int64_t)i * ldz + k], acc);
     x[k] = acc;
   }
 }
@@ -885,8 +897,38 @@ int solve_fgmres(amg_handle* h, Ctx& c, const double* b, double* x, double tol, 
   double* zr = h->kz;
   // the FP32 cycle's operator products in FP32 pairs for the velocity block (the
   // residual at each restart and at exit stays FP64)
-  float* pf = h->L[0]->val2.p ? h->kpf.p : nullptr;
+  // with the FP32 cycle in FP32 throughout: u_j staged as floats in the cycle's right-hand
+  // side, z_j the cycle's float result, which the pair operator reads as it is
+  Level& lv = *h->L[0];
+  const bool fl = h->opt.precision == AMG_FP32 && lv.val2.p;
+  // z_j itself stored as floats (Stokes projects its pressure in FP64)
+  const bool zf = fl && h->kind != AMG_STOKES;
+  float* Zf = reinterpret_cast<float*>(h->gm_Z.p);
+  float* pf = lv.val2.p ? h->kpf.p : nullptr;
   auto step = [&]() {
+    if (fl) {
+      precondition_f32(h);
+      if (lv.np == 0) {
+        apply_pair_f32(h, lv.x32, wp);
+        return;
+      }
+      // w = K z as pairs.  The FP64 work (z widened, projected, B^T p and B u - C p) on a
+      // second stream: it needs the FP64 units and the pair operator the FP32 ones and the
+      // memory (mixed 40^3: 100 us hidden behind 287)
+      AMG_CUDA(cudaEventRecord(h->fork, s));
+      AMG_CUDA(cudaStreamWaitEvent(h->side, h->fork, 0));
+      launch_to_double(lv.x32, zr, n, h->side, h);
+      Ctx cs{h, h->side, n};
+      project_pressure(h, cs, zr);
+      apply_B_parts(h, zr, pf, w, h->side);
+      AMG_CUDA(cudaEventRecord(h->join, h->side));
+      apply_pair_f32(h, lv.x32, wp);
+      AMG_CUDA(cudaStreamWaitEvent(s, h->join, 0));
+      k_join<<<gridr(n), 256, 0, s>>>(n, 4 * (int64_t)lv.n, reinterpret_cast<const float2*>(pf),
+                                      w, wp);
+      h->launches++;
+      return;
+    }
     precond(h, ur, zr);
     project_pressure(h, c, zr);
     if (pf) apply_K_pair(h, zr, pf, w);
@@ -941,7 +983,8 @@ int solve_fgmres(amg_handle* h, Ctx& c, const double* b, double* x, double tol, 
     c.dots(w, w, S_T0);
     const double beta = std::sqrt(read_scalar(h, S_T0));
     if (beta == 0.0) { conv = true; rel = 0.0; break; }
-    k_pair_scaled<<<gridr(n), 256, 0, s>>>(n, w, 1.0 / beta, V, ur);
+    if (fl) k_pair_scaled<float><<<gridr(n), 256, 0, s>>>(n, w, 1.0 / beta, V, lv.b32.p);
+    else k_pair_scaled<double><<<gridr(n), 256, 0, s>>>(n, w, 1.0 / beta, V, ur);
     h->launches++;
     std::fill(Hc.begin(), Hc.end(), 0.0);
     std::fill(g.begin(), g.end(), 0.0);
@@ -951,9 +994,15 @@ int solve_fgmres(amg_handle* h, Ctx& c, const double* b, double* x, double tol, 
       float2* uj = V + (int64_t)j * ld;
       double* zj = Z + (int64_t)j * ld;
       run_step();
-      launch_copy(zr, zj, n, s, h);
-      k_to_pair<<<gridr(n), 256, 0, s>>>(n, w, wp);
-      h->launches++;
+      if (zf)
+        AMG_CUDA(cudaMemcpyAsync(Zf + (int64_t)j * ld, lv.x32.p, n * sizeof(float),
+                                 cudaMemcpyDeviceToDevice, s));
+      else
+        launch_copy(zr, zj, n, s, h);
+      if (!fl) {
+        k_to_pair<<<gridr(n), 256, 0, s>>>(n, w, wp);
+        h->launches++;
+      }
       // one sweep: dots of rows 0..j with u_j and w, then the update of u_j to v_j and of
       // w to the next pending vector u_{j+1} (row j + 1), normalised on the device
       {
@@ -963,7 +1012,8 @@ int solve_fgmres(amg_handle* h, Ctx& c, const double* b, double* x, double tol, 
         k_dcgs2_update<<<ublocks, kThreads, kStreamSmem, s>>>(n, ld, j, V, uj, wp, un, coef.p,
                                                            h->red, h->flag.p);
         k_final<<<1, 256, 0, s>>>(h->red, ublocks, 1, coef.p + kS + 3);
-        k_scale_norm<<<gridr(n), 256, 0, s>>>(n, un, ur, coef.p + kS + 3);
+        if (fl) k_scale_norm<float><<<gridr(n), 256, 0, s>>>(n, un, lv.b32.p, coef.p + kS + 3);
+        else k_scale_norm<double><<<gridr(n), 256, 0, s>>>(n, un, ur, coef.p + kS + 3);
         h->launches += 4;
       }
       read_coef(kS + 8);
@@ -1027,7 +1077,8 @@ int solve_fgmres(amg_handle* h, Ctx& c, const double* b, double* x, double tol, 
       y[i] = t / col(i)[i];
     }
     AMG_CUDA(cudaMemcpyAsync(ydev.p, y.data(), jused * sizeof(double), cudaMemcpyHostToDevice, s));
-    k_basis_add<<<gridr(n), 256, 0, s>>>(n, jused, Z, ld, ydev.p, x);
+    if (zf) k_basis_add<float><<<gridr(n), 256, 0, s>>>(n, jused, Zf, ld, ydev.p, x);
+    else k_basis_add<double><<<gridr(n), 256, 0, s>>>(n, jused, Z, ld, ydev.p, x);
     h->launches++;
     AMG_CUDA(cudaStreamSynchronize(s));
   }
@@ -1085,7 +1136,14 @@ int solve_device(amg_handle* h, const double* b_user, double* x_user, double tol
       const int m = std::max(1, std::min(h->opt.gmres_restart, kMaxDots - 2));
       const int64_t ld = (n + 7) / 8 * 8;
       ensure(h->gm_V, (int64_t)(m + 1) * ld);
-      ensure(h->gm_Z, (int64_t)m * ld);
+      // floats with the FP32 cycle (see solve_fgmres)
+      const bool zf = h->opt.precision == AMG_FP32 && lv.val2.p && h->kind != AMG_STOKES;
+      ensure(h->gm_Z, zf ? ((int64_t)m * ld + 1) / 2 : (int64_t)m * ld);
+      if (!h->side) {
+        AMG_CUDA(cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking));
+        AMG_CUDA(cudaEventCreateWithFlags(&h->fork, cudaEventDisableTiming));
+        AMG_CUDA(cudaEventCreateWithFlags(&h->join, cudaEventDisableTiming));
+      }
       ensure(h->gm_wp, ld);
       rc = solve_fgmres(h, c, b, x, tol, st);
       break;

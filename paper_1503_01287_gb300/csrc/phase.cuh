@@ -36,7 +36,9 @@ struct Phase {
   const void* x;
   const void* b;
   void* y;
-  const int* crow;
+  const int* crow;        // PH_PROWS: C; PH_ROWS: B^T (null: none), its nnz in n3, its p in
+                          // sd; PH_RESTRICT, PH_PROLONG: m rows of H^T or H, the other
+                          // level's nodes in n3
   const int* ccol;
   const void* cval;
   const void* sd;

@@ -62,6 +62,18 @@ __device__ __forceinline__ void pair_fma(float& S, float& s, float2 a, float xh,
   s = __fadd_rn(s, __fadd_rn(err, e));
 }
 
+// the same for x that is a float (its low part 0)
+__device__ __forceinline__ void pair_fma(float& S, float& s, float2 a, float x) {
+  const float p = __fmul_rn(a.x, x);
+  float e = fmaf(a.x, x, -p);
+  e = fmaf(a.y, x, e);
+  const float t = __fadd_rn(S, p);
+  const float bp = __fsub_rn(t, S);
+  const float err = __fadd_rn(__fsub_rn(S, __fsub_rn(t, bp)), __fsub_rn(p, bp));
+  S = t;
+  s = __fadd_rn(s, __fadd_rn(err, e));
+}
+
 // (S, s) += (T, t) for the reduction across the lanes of a row
 __device__ __forceinline__ void pair_add(float& S, float& s, float T, float t) {
   const float u = __fadd_rn(S, T);
@@ -69,6 +81,18 @@ __device__ __forceinline__ void pair_add(float& S, float& s, float T, float t) {
   const float err = __fadd_rn(__fsub_rn(S, __fsub_rn(u, bp)), __fsub_rn(T, bp));
   S = u;
   s = __fadd_rn(s, __fadd_rn(err, t));
+}
+
+// FP32 pair of an FP64 value (hi = fl32(d), lo = fl32(d - hi)) and back
+__device__ __forceinline__ float2 to_pair(double d) {
+  const float hi = __double2float_rn(d);
+  return make_float2(hi, __double2float_rn(d - (double)hi));
+}
+__device__ __forceinline__ double from_pair(float2 p) { return (double)p.x + (double)p.y; }
+// a leading sum S and a small error sum s as one normalised pair (FastTwoSum)
+__device__ __forceinline__ float2 norm_pair(float S, float s) {
+  const float hi = __fadd_rn(S, s);
+  return make_float2(hi, __fsub_rn(s, __fsub_rn(hi, S)));
 }
 
 // Sums of (s0, s1, s2) over the G lanes of a row, left one component a lane: lane 0 of the
@@ -127,10 +151,10 @@ __device__ __forceinline__ void spread3(T v, int lane, T& v0, T& v1, T& v2) {
 // The end of a block row's update, whose lanes hold the partial sums (s0, s1, s2) of A x:
 // FP64 one component a lane as above; FP32 all three on the group's first lane (the spread
 // costs a shuffle more than the saved instructions give: 32^3 level-0 sweep 103.7 against
-// 98.9 us).  N: components of a lane that `holds` the row's operands.
-template <typename T, int G>
+// 98.9 us) unless SPLIT asks for it.  N: components of a lane that `holds` operands.
+template <typename T, int G, bool SPLIT = false>
 struct RowEnd {
-  static constexpr bool kSplit = sizeof(T) == 8;
+  static constexpr bool kSplit = sizeof(T) == 8 || SPLIT;
   static constexpr int N = kSplit ? 1 : 3;
   static __device__ __forceinline__ bool holds(int gl) {
     return kSplit ? holds_component<G>(gl) : gl == 0;
