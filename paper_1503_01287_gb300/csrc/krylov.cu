@@ -472,69 +472,150 @@ __global__ void k_final(const double* __restrict__ partial, int nblk, int nd,
   }
 }
 
-// CG step: alpha = rz / pq; x += alpha p; (ro = r); r -= alpha q; partial ||r||^2
-__global__ void k_cg_update(int64_t n, double* __restrict__ x, double* __restrict__ r,
-                            const double* __restrict__ p, const double* __restrict__ q,
-                            double* __restrict__ ro, const double* __restrict__ s,
-                            double* __restrict__ partial) {
+// ---------------------------------------------------------------- the CG iteration's vectors
+//
+// Four launches an iteration beside the preconditioner and the operator, each reducing to its
+// scalar by itself: every CTA leaves a partial sum, and the CTA that takes the last ticket
+// adds them in CTA order (the same bits whichever CTA that is) and does the scalar step that
+// follows.  As separate launches (conversions, dots, final sums, beta, check) they were
+// eleven of about 2.3 us each, 25 of the 54 us of an iteration on the 4^3 Laplacian.  A
+// thread takes whole nodes: the fourth entry of the padded layout is 0 and costs no FP64 work.
+
+// The CTA's sums v[0..N) to partial[blockIdx.x * N ..]; true in the last CTA to arrive, then
+// with the totals over all CTAs in v (thread 0).
+template <int N>
+__device__ __forceinline__ bool grid_sum(double (&v)[N], double* partial, unsigned* ticket,
+                                         double* sh) {
+  __shared__ bool last;
+#pragma unroll
+  for (int d = 0; d < N; ++d) {
+    const double t = block_sum(v[d], sh);
+    if (threadIdx.x == 0) partial[blockIdx.x * N + d] = t;
+  }
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+#pragma unroll
+  for (int d = 0; d < N; ++d) {
+    double s = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x)
+      s += __ldcg(partial + b * N + d);
+    v[d] = block_sum(s, sh);
+  }
+  if (threadIdx.x == 0) *ticket = 0;   // for the next launch
+  return true;
+}
+
+// <r, z> and (flexible) <z, r_old>, then beta = (<r, z> - <z, r_old>) / rz or <r, z> / rz and
+// rz <- <r, z>.  z32: the FP32 cycle's result, widened into z here.
+__global__ void __launch_bounds__(256) k_cg_dots(int nn, const double* __restrict__ r,
+                                                 const double* __restrict__ ro, double* z,
+                                                 const float* __restrict__ z32, double* s,
+                                                 double* partial, unsigned* ticket) {
+  __shared__ double sh[32];
+  double v[2] = {0.0, 0.0};
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nn; i += gridDim.x * blockDim.x) {
+    double r0, r1, r2, z0, z1, z2;
+    ld3(r, i, r0, r1, r2);
+    if (z32) {
+      float a, b, c;
+      ld3(z32, i, a, b, c);
+      z0 = a; z1 = b; z2 = c;
+      st3(z, i, z0, z1, z2);
+    } else {
+      ld3c(z, i, z0, z1, z2);
+    }
+    v[0] = fma(r0, z0, fma(r1, z1, fma(r2, z2, v[0])));
+    if (ro) {
+      ld3(ro, i, r0, r1, r2);
+      v[1] = fma(r0, z0, fma(r1, z1, fma(r2, z2, v[1])));
+    }
+  }
+  if (!grid_sum(v, partial, ticket, sh) || threadIdx.x != 0) return;
+  s[S_BETA] = (ro ? v[0] - v[1] : v[0]) / s[S_RZ];
+  s[S_RZ] = v[0];
+}
+
+// p = z + beta p; pf: also p in the pair form of the FP32-pair operator (8 floats a node: hi
+// of the 4 padded entries, then lo; lo = fl32(p - hi))
+__global__ void __launch_bounds__(256) k_cg_dir(int nn, double* p, const double* __restrict__ z,
+                                                const double* __restrict__ s,
+                                                float4* __restrict__ pf) {
+  const double beta = s[S_BETA];
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nn; i += gridDim.x * blockDim.x) {
+    double p0, p1, p2, z0, z1, z2;
+    ld3c(p, i, p0, p1, p2);
+    ld3(z, i, z0, z1, z2);
+    p0 = fma(beta, p0, z0);
+    p1 = fma(beta, p1, z1);
+    p2 = fma(beta, p2, z2);
+    st3(p, i, p0, p1, p2);
+    if (pf) {
+      const float2 a = to_pair(p0), b = to_pair(p1), c = to_pair(p2);
+      pf[2 * (int64_t)i] = make_float4(a.x, b.x, c.x, 0.f);
+      pf[2 * (int64_t)i + 1] = make_float4(a.y, b.y, c.y, 0.f);
+    }
+  }
+}
+
+// s[S_PQ] = <p, q>
+__global__ void __launch_bounds__(256) k_cg_pq(int nn, const double* __restrict__ p,
+                                               const double* __restrict__ q, double* s,
+                                               double* partial, unsigned* ticket) {
+  __shared__ double sh[32];
+  double v[1] = {0.0};
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nn; i += gridDim.x * blockDim.x) {
+    double p0, p1, p2, q0, q1, q2;
+    ld3(p, i, p0, p1, p2);
+    ld3(q, i, q0, q1, q2);
+    v[0] = fma(p0, q0, fma(p1, q1, fma(p2, q2, v[0])));
+  }
+  if (grid_sum(v, partial, ticket, sh) && threadIdx.x == 0) s[S_PQ] = v[0];
+}
+
+// alpha = rz / pq; x += alpha p; (ro = r); r -= alpha q; (r32 = r, the FP32 cycle's right-hand
+// side); s[S_RR] = ||r||^2.  loop: the stopping rule on the device, continue while ||r||^2 >
+// tol^2 ||b||^2, the iteration limit is not reached and the residual is finite.
+__global__ void __launch_bounds__(256) k_cg_update(int nn, double* x, double* r,
+                                                   const double* __restrict__ p,
+                                                   const double* __restrict__ q, double* ro,
+                                                   float* __restrict__ r32, double* s,
+                                                   double* partial, unsigned* ticket, bool loop,
+                                                   cudaGraphConditionalHandle cond, int* it,
+                                                   int maxit) {
   __shared__ double sh[32];
   const double alpha = s[S_RZ] / s[S_PQ];
-  double acc = 0.0;
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-       k += (int64_t)gridDim.x * blockDim.x) {
-    x[k] = fma(alpha, p[k], x[k]);
-    const double rk = r[k];
-    if (ro) ro[k] = rk;
-    const double rn = fma(-alpha, q[k], rk);
-    r[k] = rn;
-    acc = fma(rn, rn, acc);
+  double v[1] = {0.0};
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nn; i += gridDim.x * blockDim.x) {
+    double a0, a1, a2, b0, b1, b2;
+    ld3(p, i, a0, a1, a2);
+    ld3c(x, i, b0, b1, b2);
+    st3(x, i, fma(alpha, a0, b0), fma(alpha, a1, b1), fma(alpha, a2, b2));
+    ld3(q, i, a0, a1, a2);
+    ld3c(r, i, b0, b1, b2);
+    if (ro) st3(ro, i, b0, b1, b2);
+    b0 = fma(-alpha, a0, b0);
+    b1 = fma(-alpha, a1, b1);
+    b2 = fma(-alpha, a2, b2);
+    st3(r, i, b0, b1, b2);
+    if (r32) st3(r32, i, (float)b0, (float)b1, (float)b2);
+    v[0] = fma(b0, b0, fma(b1, b1, fma(b2, b2, v[0])));
   }
-  double t = block_sum(acc, sh);
-  if (threadIdx.x == 0) partial[blockIdx.x] = t;
-}
-
-// beta = (rz_new - <z, r_old>) / rz (flexible) or rz_new / rz; rz <- rz_new
-__global__ void k_cg_beta(double* s, int flexible) {
-  const double num = flexible ? s[S_RZN] - s[S_ZRO] : s[S_RZN];
-  s[S_BETA] = num / s[S_RZ];
-  s[S_RZ] = s[S_RZN];
-}
-
-// stopping rule on the device: continue while ||r||^2 > tol^2 ||b||^2, the
-// iteration limit is not reached and the residual is finite
-__global__ void k_cg_check(cudaGraphConditionalHandle cond, const double* __restrict__ s,
-                           int* it, int maxit) {
-  const int k = ++(*it);
-  const double rr = s[S_RR];
-  const bool go = !(rr <= s[S_TOL2] * s[S_BB]) && k < maxit && isfinite(rr);
-  cudaGraphSetConditional(cond, go ? 1u : 0u);
+  if (!grid_sum(v, partial, ticket, sh) || threadIdx.x != 0) return;
+  const double rr = v[0];
+  s[S_RR] = rr;
+  if (loop) {
+    const int k = ++(*it);
+    const bool go = !(rr <= s[S_TOL2] * s[S_BB]) && k < maxit && isfinite(rr);
+    cudaGraphSetConditional(cond, go ? 1u : 0u);
+  }
 }
 
 __global__ void k_set_tol2(double* s, double tol) { s[S_TOL2] = tol * tol; }
-
-__global__ void k_cg_dir(int64_t n, double* __restrict__ p, const double* __restrict__ z,
-                         const double* __restrict__ s) {
-  const double beta = s[S_BETA];
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-       k += (int64_t)gridDim.x * blockDim.x)
-    p[k] = fma(beta, p[k], z[k]);
-}
-
-// the same, also writing p in the pair form of the FP32-pair operator (8 floats
-// a node: hi of the 4 padded entries, then lo; lo = fl32(p - hi))
-__global__ void k_cg_dir_pair(int64_t n, double* __restrict__ p, const double* __restrict__ z,
-                              const double* __restrict__ s, float* __restrict__ pf) {
-  const double beta = s[S_BETA];
-  for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
-       k += (int64_t)gridDim.x * blockDim.x) {
-    const double v = fma(beta, p[k], z[k]);
-    p[k] = v;
-    const float hi = (float)v;
-    const int64_t o = 8 * (k >> 2) + (k & 3);
-    pf[o] = hi;
-    pf[o + 4] = (float)(v - (double)hi);
-  }
-}
 
 // x += sum_i y[i] Z_i (y staged in shared memory; the basis loads of one index go
 // out eight at a time, the sum keeps the order i = 0, 1, ...)
@@ -665,24 +746,32 @@ int solve_cg(amg_handle* h, Ctx& c, const double* b, double* x, double tol, bool
   // FP32 cycle: the operator products in FP32-pair arithmetic (outer_pair)
   float* pf = (h->opt.precision == AMG_FP32 && h->L[0]->val2.p) ? h->kpf.p : nullptr;
 
-  // the body of one iteration after the first: z = M r, beta, p, q = A p, alpha, x, r
-  auto body = [&](bool first) {
+  // FP32 cycle: r is handed over as floats by the update, z widened by the dots
+  const bool f32 = h->opt.precision == AMG_FP32;
+  const int nn = (int)(n / 4);   // the SPD kinds have no pressure part
+  const int blocks = std::max(1, std::min(div_up(nn, 256), kReduceBlocks));
+  float* r32 = f32 ? h->L[0]->b32.p : nullptr;
+  unsigned* ticket = reinterpret_cast<unsigned*>(h->it_dev.p + 1);
+  // the body of one iteration after the first: z = M r, beta, p, q = A p, alpha, x, r; in the
+  // graph loop with the stopping test on `cond`
+  auto body = [&](bool first, const cudaGraphConditionalHandle* cond = nullptr) {
     if (!first) {
-      precond(h, r, z);
-      if (flexible) c.dots(r, z, S_RZN, z, ro);
-      else c.dots(r, z, S_RZN);
-      k_cg_beta<<<1, 1, 0, s>>>(h->scal.p, flexible ? 1 : 0);
-      if (pf) k_cg_dir_pair<<<gridr(n), 256, 0, s>>>(n, p, z, h->scal.p, pf);
-      else k_cg_dir<<<gridr(n), 256, 0, s>>>(n, p, z, h->scal.p);
+      if (f32) precondition_f32(h);
+      else precond(h, r, z);
+      k_cg_dots<<<blocks, 256, 0, s>>>(nn, r, ro, z, f32 ? h->L[0]->x32.p : nullptr, h->scal.p,
+                                       h->red, ticket);
+      k_cg_dir<<<blocks, 256, 0, s>>>(nn, p, z, h->scal.p, reinterpret_cast<float4*>(pf));
       h->launches += 2;
     } else if (pf) {
       launch_split_pair(p, pf, n, s, h);
     }
     if (pf) apply_pair(h, pf, q);
     else apply_K(h, p, q);
-    c.dots(p, q, S_PQ);
-    k_cg_update<<<kReduceBlocks, kReduceThreads, 0, s>>>(n, x, r, p, q, ro, h->scal.p, h->red);
-    k_final<<<1, 256, 0, s>>>(h->red, kReduceBlocks, 1, h->scal.p + S_RR);
+    k_cg_pq<<<blocks, 256, 0, s>>>(nn, p, q, h->scal.p, h->red, ticket);
+    k_cg_update<<<blocks, 256, 0, s>>>(nn, x, r, p, q, ro, r32, h->scal.p, h->red, ticket,
+                                       cond != nullptr,
+                                       cond ? *cond : cudaGraphConditionalHandle{}, h->it_dev.p,
+                                       h->opt.max_iterations);
     h->launches += 2;
   };
 
@@ -690,7 +779,7 @@ int solve_cg(amg_handle* h, Ctx& c, const double* b, double* x, double tol, bool
   ++it;
   rel = std::sqrt(std::max(0.0, read_scalar(h, S_RR))) / bnorm;
   // All further iterations in one graph launch: a conditional WHILE node whose
-  // body is one iteration followed by the stopping test (k_cg_check).
+  // body is one iteration, whose update ends with the stopping test.
   if (h->opt.use_graphs && !(rel <= tol) && it < h->opt.max_iterations && std::isfinite(rel)) {
     cudaGraphExec_t& wexec = flexible ? h->cg_loop_fcg : h->cg_loop_pcg;
     int64_t& per_iter = flexible ? h->cg_loop_fcg_launches : h->cg_loop_pcg_launches;
@@ -713,13 +802,12 @@ int solve_cg(amg_handle* h, Ctx& c, const double* b, double* x, double tol, bool
         AMG_CUDA(cudaStreamBeginCaptureToGraph(s, bodyg, nullptr, nullptr, 0,
                                                cudaStreamCaptureModeThreadLocal));
         capturing = true;
-        body(false);
-        k_cg_check<<<1, 1, 0, s>>>(cond, h->scal.p, h->it_dev.p, h->opt.max_iterations);
+        body(false, &cond);
         AMG_LAUNCH_CHECK();
         capturing = false;
         AMG_CUDA(cudaStreamEndCapture(s, &bodyg));
         AMG_CUDA(cudaGraphInstantiate(&wexec, g, 0));
-        per_iter = h->launches - l0 + 1;
+        per_iter = h->launches - l0;
       } catch (const Error&) {
         if (capturing) {
           cudaGraph_t junk = nullptr;
@@ -1110,7 +1198,10 @@ int solve_device(amg_handle* h, const double* b_user, double* x_user, double tol
   }
   ensure(h->red, (int64_t)kReduceBlocks * kMaxDots);
   ensure(h->scal, 64);
-  if (!h->it_dev.p) h->it_dev.alloc(1);
+  if (!h->it_dev.p) {   // the iteration count and the reductions' ticket (left at 0)
+    h->it_dev.alloc(2);
+    AMG_CUDA(cudaMemsetAsync(h->it_dev.p, 0, h->it_dev.bytes(), h->stream));
+  }
   int krylov = h->opt.krylov;
   if (krylov == AMG_KRYLOV_AUTO)
     krylov = h->saddle ? AMG_KRYLOV_FGMRES
