@@ -601,6 +601,137 @@ void launch_gs_m_pdl(int nrows, const int* rows, const int* rowptr, const int* r
                               lv.nnzb, x, b, dinv, lv.template steps<T>(), seed));
 }
 
+// The same colour kernel, FP32, with the rows' columns and values staged in shared memory
+// before griddepcontrol.wait.  Read block by block from the 9 planes, the values were 10
+// broadcast loads beside the one gather of x_j, and a lane group took its blocks four at a
+// time: the sweep waited on its load instructions and on rounds of gathers (12^3: 10 us a
+// colour).  Here a row's lanes load its columns and planes coalesced, each once, as three
+// 16-byte entries a block with the column in the first; the loop then takes three 16-byte
+// broadcasts from shared memory and one gather a block, eight gathers in flight.
+// S lane groups of 16 a row (lane r of a group: right-hand side r), 16 / S rows a CTA; row
+// slots of `slot` blocks (the level's longest row) in dynamic shared memory.
+template <int S, bool FIRST>
+__global__ void __launch_bounds__(256) k_gs_m_staged(
+    int nrows, int slot, const int* __restrict__ rows, const int* __restrict__ rowptr,
+    const int* __restrict__ rowend, const int* __restrict__ col, const float* __restrict__ val,
+    int64_t nnzb, float* x, const float* __restrict__ b, const float* __restrict__ dinv,
+    const float* __restrict__ wt, float* __restrict__ seed) {
+  extern __shared__ float4 blocks[];                   // [row of the CTA][3][slot]
+  __shared__ float red[S > 2 ? 8 : 1][K][3];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  constexpr int L = K * S;                             // lanes of a row
+  const int t = threadIdx.x % L, q = t / K, r = t % K;
+  const int g = blockIdx.x * (256 / L) + threadIdx.x / L;
+  const bool active = g < nrows;                       // uniform over the lanes of a row
+  float4* p0 = blocks + (size_t)(threadIdx.x / L) * 3 * slot;
+  float4* p1 = p0 + slot;
+  float4* p2 = p1 + slot;
+  int i = 0, n = 0;
+  float d[9];
+  if (active) {
+    i = __ldg(rows + g);
+    const int a = __ldg(rowptr + g);
+    n = __ldg(rowend + g) - a;
+    for (int k = t; k < n; k += L) {
+      const float* v = val + a + k;
+      p0[k] = make_float4(__ldg(v), __ldg(v + nnzb), __ldg(v + 2 * nnzb),
+                          __int_as_float(__ldg(col + a + k)));
+      p1[k] = make_float4(__ldg(v + 3 * nnzb), __ldg(v + 4 * nnzb), __ldg(v + 5 * nnzb), 0.f);
+      p2[k] = make_float4(__ldg(v + 6 * nnzb), __ldg(v + 7 * nnzb), __ldg(v + 8 * nnzb), 0.f);
+    }
+    if (q == 0) {
+      const float* dp = dinv + 12 * (int64_t)i;
+      ld3(dp, 0, d[0], d[1], d[2]);
+      ld3(dp, 1, d[3], d[4], d[5]);
+      ld3(dp, 2, d[6], d[7], d[8]);
+    }
+  }
+  __syncthreads();
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const float om = wt ? wt[0] : 1.f;
+  float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+  const float4* x4 = reinterpret_cast<const float4*>(x) + r;
+  int k = q;
+  for (; k + 7 * S < n; k += 8 * S) {
+    float4 xv[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) xv[u] = __ldg(x4 + (int64_t)__float_as_int(p0[k + u * S].w) * K);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const float4 a = p0[k + u * S], c = p1[k + u * S], e = p2[k + u * S];
+      s0 = fmaf(a.x, xv[u].x, s0); s0 = fmaf(a.y, xv[u].y, s0); s0 = fmaf(a.z, xv[u].z, s0);
+      s1 = fmaf(c.x, xv[u].x, s1); s1 = fmaf(c.y, xv[u].y, s1); s1 = fmaf(c.z, xv[u].z, s1);
+      s2 = fmaf(e.x, xv[u].x, s2); s2 = fmaf(e.y, xv[u].y, s2); s2 = fmaf(e.z, xv[u].z, s2);
+    }
+  }
+#pragma unroll 4
+  for (; k < n; k += S) {
+    const float4 a = p0[k], c = p1[k], e = p2[k];
+    const float4 v = __ldg(x4 + (int64_t)__float_as_int(a.w) * K);
+    s0 = fmaf(a.x, v.x, s0); s0 = fmaf(a.y, v.y, s0); s0 = fmaf(a.z, v.z, s0);
+    s1 = fmaf(c.x, v.x, s1); s1 = fmaf(c.y, v.y, s1); s1 = fmaf(c.z, v.z, s1);
+    s2 = fmaf(e.x, v.x, s2); s2 = fmaf(e.y, v.y, s2); s2 = fmaf(e.z, v.z, s2);
+  }
+  s0 += __shfl_xor_sync(0xffffffffu, s0, 16);          // lane groups q and q + 1 share a warp
+  s1 += __shfl_xor_sync(0xffffffffu, s1, 16);
+  s2 += __shfl_xor_sync(0xffffffffu, s2, 16);
+  if (S > 2) {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (lane < K) {
+      red[w][lane][0] = s0;
+      red[w][lane][1] = s1;
+      red[w][lane][2] = s2;
+    }
+    __syncthreads();
+    if (!active || q != 0) return;
+    s0 = s1 = s2 = 0.f;
+#pragma unroll
+    for (int v = 0; v < S / 2; ++v) {
+      s0 += red[w + v][r][0];
+      s1 += red[w + v][r][1];
+      s2 += red[w + v][r][2];
+    }
+  }
+  if (!active || q != 0) return;
+  const int o = i * K + r;
+  float b0, b1, b2, x0 = 0.f, x1 = 0.f, x2 = 0.f;
+  ld3(b, o, b0, b1, b2);
+  if (!FIRST) ld3c(x, o, x0, x1, x2);
+  const float r0 = b0 - s0, r1 = b1 - s1, r2 = b2 - s2;
+  if (FIRST && seed) st3(seed, o, (1.f - om) * r0, (1.f - om) * r1, (1.f - om) * r2);
+  st3(x, o, x0 + om * (d[0] * r0 + d[1] * r1 + d[2] * r2),
+      x1 + om * (d[3] * r0 + d[4] * r1 + d[5] * r2),
+      x2 + om * (d[6] * r0 + d[7] * r1 + d[8] * r2));
+}
+
+// Shared memory of the staged kernel's rows, 0 where they do not fit (the kernel above then)
+constexpr int kStageSmem = 64 * 1024;
+inline int stage_lanes(const Level& lv) { return lv.avg_row_blocks < 40.0 ? 2 : 4; }
+inline int stage_smem(const Level& lv) {
+  const int64_t bytes = (int64_t)(K / stage_lanes(lv)) * 3 * lv.max_row_blocks * 16;
+  return bytes <= kStageSmem ? (int)bytes : 0;
+}
+
+template <int S, bool FIRST>
+void launch_gs_m_staged(int nrows, const int* rows, const int* rowptr, const int* rowend,
+                        Level& lv, float* x, const float* b, float* seed, cudaStream_t s) {
+  max_dynamic_smem((const void*)k_gs_m_staged<S, FIRST>, kStageSmem);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(((int64_t)nrows * K * S + 255) / 256));
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = stage_smem(lv);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  AMG_CUDA(cudaLaunchKernelEx(&cfg, k_gs_m_staged<S, FIRST>, nrows, lv.max_row_blocks, rows,
+                              rowptr, rowend, (const int*)lv.k_col(), (const float*)lv.val32.p,
+                              lv.nnzb, x, b, (const float*)lv.dinv32.p,
+                              (const float*)lv.wt32, seed));
+}
+
 // one colour of the batched Gauss-Seidel sweep (x updated in place; `first`: from x = 0 on the
 // lower-colour blocks, leaving the residual's seed, as kFirst of the single cycle)
 template <typename T>
@@ -611,6 +742,20 @@ void gs_colour_m(amg_handle* h, Level& lv, int at, int nrows, const T* val, T* x
   const int* rp = lv.k_rowptr() + at;
   const int* re = first ? lv.smid.p + at : rp + 1;
   cudaStream_t s = h->stream;
+  if constexpr (std::is_same<T, float>::value) {
+    // a tile that the caller gives keeps the kernel that it names
+    if (h->opt.batch_tile < 0 && stage_smem(lv) > 0) {
+      if (stage_lanes(lv) == 2) {
+        if (first) launch_gs_m_staged<2, true>(nrows, rows, rp, re, lv, x, b, seed, s);
+        else launch_gs_m_staged<2, false>(nrows, rows, rp, re, lv, x, b, seed, s);
+      } else {
+        if (first) launch_gs_m_staged<4, true>(nrows, rows, rp, re, lv, x, b, seed, s);
+        else launch_gs_m_staged<4, false>(nrows, rows, rp, re, lv, x, b, seed, s);
+      }
+      h->launches++;
+      return;
+    }
+  }
   switch (tile) {
     case 1: launch_gs_m_pdl<T, 2, 2>(nrows, rows, rp, re, lv, val, x, b, dinv, first, seed, s); break;
     case 2: launch_gs_m_pdl<T, 1, 4>(nrows, rows, rp, re, lv, val, x, b, dinv, first, seed, s); break;
