@@ -152,9 +152,14 @@ typedef struct amg_options {
   int32_t max_iterations;   /* Krylov iteration limit (default 1000)            */
   int32_t use_graphs;       /* 1: replay each Krylov iteration as a CUDA graph  */
   int32_t cluster_from;     /* coarse levels from this level down run as one
-                               thread-block-cluster launch: -1 chosen by timing
-                               at setup (default), 0 never, k >= 1 from level k */
-  int32_t cycle_kernel;     /* 0: chosen by timing at setup (default); 1: one
+                               thread-block-cluster launch: 0 never, k >= 1 from
+                               level k; -1 (default) with cycle_kernel 0 and the
+                               gs_* options below at -1: the levels from the first
+                               of at most 10,240 unknowns (FP64 6,144; segregated
+                               Gauss-Seidel 4,608) down as one stored matrix, the
+                               cycle's own linear map, built at setup and again
+                               when their weights change; else chosen by timing  */
+  int32_t cycle_kernel;     /* 0: as cluster_from -1 (default); 1: one
                                launch per operation (with the cluster levels);
                                2: the whole cycle as one persistent cooperative
                                launch with grid barriers.  With the Vanka
@@ -163,9 +168,10 @@ typedef struct amg_options {
   double omega;             /* block Jacobi damping (default 0.5)               */
   double omega_p;           /* sGS pressure step omega (default 0.125)          */
   int32_t batch_tile;       /* amg_solve_batched: tile of the SpMM row kernels
-                               and of the colour kernels, -1 chosen per level by
-                               timing the SpMM (default; the colour kernels take
-                               the same tile); t =
+                               and of the colour kernels, -1 (default) the SpMM's
+                               chosen per level by timing, FP32 colours staged in
+                               shared memory and small levels as one stored
+                               matrix, FP64 colours with the SpMM's tile; t =
                                0..7 forces (lane groups per row, blocks
                                unrolled) = (1,2), (2,2), (1,4), (2,4), (4,2),
                                (8,2), (4,4), (8,4) on the colour kernels and
@@ -173,8 +179,9 @@ typedef struct amg_options {
   int32_t gs_cluster;       /* multicolour Gauss-Seidel sweep of a level whose
                                iterate, right-hand side and row offsets fit in
                                shared memory (SPD kinds, up to about 5000 nodes
-                               in FP32, 2800 in FP64): -1
-                               chosen per level by timing at setup (default),
+                               in FP32, 2800 in FP64): -1 (default)
+                               0, or where no stored matrix is in use
+                               (cluster_from) chosen per level by timing;
                                0 one launch per colour, k = 1, 2, 4, 8 or 16:
                                the whole sweep in one cluster of k CTAs         */
   int32_t outer_pair;       /* FP32-cycle Krylov solves (CG for SPD kinds, the
@@ -199,26 +206,22 @@ typedef struct amg_options {
   int32_t gs_flow;          /* multicolour Gauss-Seidel sweep of a coloured level
                                as one cooperative launch in dataflow order (each
                                row waits on per-node flags of the neighbours it
-                               reads new values from): -1 chosen per level by
-                               timing at setup (default), 0 never, 1 on every
+                               reads new values from): -1 (default) as
+                               gs_cluster, 0 never, 1 on every
                                coloured level with the lanes per row of the
                                one-launch-per-colour kernel (bitwise its
                                results)                                       */
   int32_t gs_stream;        /* one-launch-per-colour Gauss-Seidel kernels as
                                grid-stride loops over a grid of k CTAs per SM,
                                each warp loading its next rows' blocks while it
-                               updates the current ones: -1 k and the lanes per
-                               row chosen per level by timing at setup
-                               (default; 0 where one group of lanes per row is
-                               faster), 0 never, k = 1..8 forced (lanes per
-                               row as tuned for the chain)                     */
+                               updates the current ones: -1 (default) as
+                               gs_cluster, 0 never, k = 1..8 forced (lanes per
+                               row as the chain's)                     */
   int32_t gs_tma;           /* FP32 one-launch-per-colour Gauss-Seidel kernel
                                with the block values and columns of a CTA's rows
                                staged in shared memory by bulk (TMA) copies
                                issued before the wait on the previous colour:
-                               -1 with its lanes per row where it beats the
-                               register-prefetch kernel, chosen per level by
-                               timing at setup (default), 0 never, 1 on every
+                               -1 (default) as gs_cluster, 0 never, 1 on every
                                coloured FP32 level with the chain's lanes per
                                row (bitwise its results)                       */
 } amg_options;

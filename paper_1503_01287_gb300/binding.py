@@ -247,6 +247,28 @@ def _ptr(a):
     return a.ctypes.data
 
 
+def _ptrs(stream, *arrays):
+    """Addresses for a call that is ordered on `stream` (None: the legacy default stream).
+
+    Work that the caller queued on its current stream precedes the call by itself when the
+    two are the same stream; otherwise the current stream is synchronised, once."""
+    for a in arrays:
+        if getattr(a, "is_cuda", False):
+            import torch
+            cur = torch.cuda.current_stream(a.device)
+            if cur.cuda_stream != (getattr(stream, "value", stream) or 0):
+                cur.synchronize()
+            break
+    out = []
+    for a in arrays:
+        if hasattr(a, "data_ptr"):
+            assert a.is_contiguous()
+            out.append(a.data_ptr())
+        else:
+            out.append(_ptr(a))
+    return out
+
+
 class Handle:
     """Owns one amg_handle.  Arrays passed in are kept alive only for the call."""
 
@@ -408,26 +430,27 @@ class Handle:
 def mlp_forward(theta, x, y, stream=None):
     """y[i] = net(theta, x[i]) on device tensors (float32; x of shape (n, 16))."""
     n = int(x.shape[0])
-    _check(load_library().amg_mlp_forward(_ptr(theta), _ptr(x), n, _ptr(y), stream))
+    th, xp, yp = _ptrs(stream, theta, x, y)
+    _check(load_library().amg_mlp_forward(th, xp, n, yp, stream))
 
 
 def mlp_gradient(theta, x, t, grad, loss, stream=None):
     """grad, loss of the mean squared error of the net on (x, t), device tensors."""
     n = int(x.shape[0])
-    _check(load_library().amg_mlp_gradient(_ptr(theta), _ptr(x), _ptr(t), n, _ptr(grad),
-                                           _ptr(loss), stream))
+    th, xp, tp, gp, lp = _ptrs(stream, theta, x, t, grad, loss)
+    _check(load_library().amg_mlp_gradient(th, xp, tp, n, gp, lp, stream))
 
 
 def mlp_backward(theta, x, dy, grad, stream=None):
     """grad = sum_i dy[i] d net(x[i]) / d theta on device tensors (float32)."""
     n = int(x.shape[0])
-    _check(load_library().amg_mlp_backward(_ptr(theta), _ptr(x), _ptr(dy), n, _ptr(grad),
-                                           stream))
+    th, xp, dp, gp = _ptrs(stream, theta, x, dy, grad)
+    _check(load_library().amg_mlp_backward(th, xp, dp, n, gp, stream))
 
 
 def mlp_adam(theta, grad, m, v, step: int, lr: float, stream=None):
-    _check(load_library().amg_mlp_adam(_ptr(theta), _ptr(grad), _ptr(m), _ptr(v), step,
-                                       float(lr), stream))
+    th, gp, mp, vp = _ptrs(stream, theta, grad, m, v)
+    _check(load_library().amg_mlp_adam(th, gp, mp, vp, step, float(lr), stream))
 
 
 def setup_problem(prob, options: AmgOptions | None = None, stream=None) -> Handle:

@@ -353,6 +353,9 @@ __device__ __forceinline__ int64_t map_plane(int m, int k, int r) {
   return ((int64_t)(r >> 2) * m + k) * 4 + (r & 3);
 }
 
+// forgets the captured CG loops (they hold the cycle's launches)
+void drop_loops(amg_handle* h);
+
 // krylov (krylov.cu)
 int solve_device(amg_handle* h, const double* b, double* x, double tol, amg_stats* st);
 

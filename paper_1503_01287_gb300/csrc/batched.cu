@@ -5,7 +5,9 @@
 // right-hand sides of one node contiguous), so the block-row kernels are SpMM:
 // one lane per right-hand side, the 9 block values and the column index are
 // the same address for all lanes of a row (broadcast), and the gather of x_j
-// for all right-hand sides is one contiguous 16 x 16-byte (FP32) access.
+// for all right-hand sides is one contiguous 16 x 16-byte (FP32) access.  With the FP32
+// cycle the colours stage their rows in shared memory (k_gs_m_staged) and the small levels
+// run as one stored matrix (coarse_map.cu).
 //
 // Each problem runs flexible CG per right-hand side (Polak-Ribiere beta, the
 // FP64 outer iteration of the FP32 or FP64 cycle; with the FP32 cycle the

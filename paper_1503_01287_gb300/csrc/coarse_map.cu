@@ -38,7 +38,7 @@ namespace {
 constexpr int kColThreads = 128;
 constexpr int kColN = 2;                             // vectors of a thread
 constexpr int kColBlock = kColThreads * kColN;       // vectors of a CTA
-constexpr int kColMax = 16 * kColBlock;              // vectors of one pass
+constexpr int kColMax = 20 * kColBlock;              // vectors of one pass
 
 struct Pair {
   float h, l;
@@ -466,8 +466,7 @@ void build(amg_handle* h, const CoarseMap& map, S* M) {
   // so a block of 256 columns keeps its vectors in L2, and the small colours still fill the
   // chip (512 columns a pass at 32^3: 97 ms, all but a few launches waiting on latency)
   const int from = map.from, m = map.m;
-  const int nchunk = div_up(m, kColMax);
-  const int W = div_up(div_up(m, nchunk), kColBlock) * kColBlock;
+  int W = div_up(div_up(m, div_up(m, kColMax)), kColBlock) * kColBlock;
   std::vector<Phase> ph;
   record_map_phases<S>(h, from, ph);
   ColVectors<T, S> v;
@@ -481,7 +480,15 @@ void build(amg_handle* h, const CoarseMap& map, S* M) {
   for (const Phase& P : ph)
     for (const void* q : {P.x, P.b, P.p, (const void*)P.y, P.type == PH_ROWS ? P.sd : nullptr})
       v.use(q);
-  v.mem.alloc((size_t)v.total * W);
+  for (;;) {   // fewer columns a pass where the device has no room (1.6 GB at m = 8,538)
+    try {
+      v.mem.alloc((size_t)v.total * W);
+      break;
+    } catch (const Error& e) {
+      if (e.code != AMG_ERR_NOMEM || W <= kColBlock) throw;
+      W = std::max(kColBlock, W / 2 / kColBlock * kColBlock);
+    }
+  }
   T* b = v.map(lb, W);
   T* x = v.map(lx, W);
   for (Phase& P : ph) {
@@ -659,6 +666,13 @@ const T* matrix(const CoarseMap& M) {
 // 300 MB) and the time of the construction.
 constexpr int kMapMax32 = 10240;
 constexpr int kMapMax64 = 6144;
+// A segregated Gauss-Seidel level is 7 launches, not 65: Stokes 24^3 in FP64 gains 60 us of
+// 580 a preconditioner by its map of 4,159, built in 16 ms.
+constexpr int kMapMaxSgs = 4608;
+// The largest map that a change of weights builds again: at 4,096 it takes about the 4 ms that
+// it saves in one solve, at 8,538 (32^3) 17 ms for 3 ms.  A larger one gives way to one of at
+// most this size.
+constexpr int kMapMaxRebuild = 4096;
 // and the share of the coarsest solve (FP64) in the construction
 constexpr int64_t kMapCoarseWork = 4000000000ll;
 
@@ -695,9 +709,28 @@ void fill(amg_handle* h, CoarseMap& M, const double* w) {
   // the weights of the levels that M holds (4 a level): nothing to do if they are as built
   const std::vector<double> now(w + 4 * M.from, w + 4 * h->L.size());
   if (now == M.w) return;
+  const bool again = !M.w.empty();
   M.w.clear();
-  if (M.m32.p) build<Pair, float>(h, M, M.m32.p);
-  else build<double, double>(h, M, M.m64.p);
+  if (again && M.m > kMapMaxRebuild) {
+    M.from = -1;
+    M.m32.release();
+    M.m64.release();
+    drop_loops(h);
+    plan(h, M, kMapMaxRebuild);
+    fill(h, M, w);
+    return;
+  }
+  try {
+    if (M.m32.p) build<Pair, float>(h, M, M.m32.p);
+    else build<double, double>(h, M, M.m64.p);
+  } catch (const Error& e) {
+    M.from = -1;   // the cycle runs operation by operation, in newly captured loops
+    M.m32.release();
+    M.m64.release();
+    drop_loops(h);
+    if (e.code != AMG_ERR_NOMEM) throw;
+    return;
+  }
   M.w = now;
 }
 
@@ -709,14 +742,20 @@ void map_plan(amg_handle* h) {
   if (o.cluster_from != -1 || o.cycle_kernel != 0 || o.gs_cluster != -1 || o.gs_flow != -1 ||
       o.gs_stream != -1 || o.gs_tma != -1 || o.smoother == AMG_SMOOTHER_VANKA)
     return;
-  plan(h, h->map, o.precision == AMG_FP32 ? kMapMax32 : kMapMax64);
+  plan(h, h->map,
+       o.smoother == AMG_SMOOTHER_SGS ? kMapMaxSgs
+       : o.precision == AMG_FP32      ? kMapMax32
+                                      : kMapMax64);
 }
 
 const CoarseMap* map_batch(amg_handle* h) {
   // the batched cycle reads the FP32 values of every level, also with BF16 storage
   if (h->map.from < 0 || !h->map.m32.p || h->bf16_coarse || h->opt.batch_tile != -1)
     return nullptr;
-  if (h->map.m <= kMapMaxBatch) return &h->map;
+  if (h->map.m <= kMapMaxBatch) {
+    h->bmap = CoarseMap{};   // of a larger map that gave way
+    return &h->map;
+  }
   if (h->bmap.from < 0) {
     plan(h, h->bmap, kMapMaxBatch);
     if (h->bmap.from < 0) return nullptr;

@@ -5,9 +5,9 @@
 //
 // Every operation has one __device__ body.  The cycle is written once against
 // an emitter that either launches one kernel per operation or records it as a
-// phase.  The recorded phases of the small coarse levels run in one launch of a
-// thread-block cluster, separated by cluster barriers, so both paths perform the
-// same operations in the same order.
+// phase.  Recorded phases build the matrix that the small coarse levels run as
+// (coarse_map.cu) or, where an option asks for it, run in one launch of a thread-block
+// cluster, separated by cluster barriers; all paths perform the same operations.
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 

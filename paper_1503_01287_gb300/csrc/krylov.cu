@@ -1179,6 +1179,12 @@ int solve_fgmres(amg_handle* h, Ctx& c, const double* b, double* x, double tol, 
 
 }  // namespace
 
+void drop_loops(amg_handle* h) {
+  if (h->cg_loop_pcg) cudaGraphExecDestroy(h->cg_loop_pcg);
+  if (h->cg_loop_fcg) cudaGraphExecDestroy(h->cg_loop_fcg);
+  h->cg_loop_pcg = h->cg_loop_fcg = nullptr;
+}
+
 int solve_device(amg_handle* h, const double* b_user, double* x_user, double tol,
                  amg_stats* st) {
   const Level& lv = *h->L[0];

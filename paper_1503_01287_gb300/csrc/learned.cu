@@ -406,6 +406,23 @@ void learn_weights(amg_handle* h, const float* theta_host, amg_learned* out) {
   level_apply<double>(h, 0, ypad.p, bpad.p);
   launch_from_padded(bpad, b, l0.n, l0.np, s, h);
   int itp = 0, itl = 0;
+  // The probes' weights are tried once each: with the cycle run operation by operation, so
+  // that the stored coarse cycle is rebuilt for the kept weights only.
+  struct Unmapped {
+    amg_handle* h;
+    int from;
+    explicit Unmapped(amg_handle* q) : h(q), from(q->map.from) {
+      h->map.from = -1;
+      drop_loops(h);
+    }
+    ~Unmapped() { restore(); }
+    void restore() {   // once: the map may be planned anew after it
+      if (!h) return;
+      drop_loops(h);
+      h->map.from = from;
+      h = nullptr;
+    }
+  } unmapped(h);
   set_level_weights(h, plain.data(), nl);
   out->rho_plain = probe_rate(h, b, x, &itp);
   out->probe_iterations_plain = itp;
@@ -432,6 +449,7 @@ void learn_weights(amg_handle* h, const float* theta_host, amg_learned* out) {
   }
   out->fell_back = keep == &plain ? 1 : 0;
   if (out->fell_back) out->rho_learned = out->rho_learned > 0 ? out->rho_learned : out->rho_plain;
+  unmapped.restore();
   set_level_weights(h, keep->data(), nl);
   for (int l = 0; l < nl && l < AMG_MAX_LEVELS; ++l)
     for (int e = 0; e < 3; ++e) out->level_weights[3 * l + e] = (*keep)[3 * l + e];

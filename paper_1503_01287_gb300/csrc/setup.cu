@@ -589,21 +589,41 @@ __global__ void k_dirichlet_diag(int n, const int* __restrict__ tags, const int*
 
 // One round of first-fit colouring in increasing index order: a node is coloured
 // once all its lower-index neighbours are, with the smallest colour none of them
-// uses.
+// uses.  kColourLanes lanes a node share its neighbours: a thread a node read its 60
+// neighbours one after the other, 17 us a round of the 344 rounds of 12x13x14.
+constexpr int kColourLanes = 8;
 __global__ void k_colour_round(int n, const int* __restrict__ rowptr, const int* __restrict__ col,
                                int* colour, int* remaining) {
+  constexpr int L = kColourLanes;
   volatile int* vc = colour;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    if (vc[i] >= 0) continue;
-    int a = rowptr[i], b = rowptr[i + 1];
-    bool ready = true;
-    for (int k = a; k < b; ++k) {
-      int j = col[k];
+  const int gl = threadIdx.x & (L - 1);
+  const unsigned group = ((1u << L) - 1u) << (threadIdx.x & 31 & ~(L - 1));
+  const int stride = gridDim.x * blockDim.x / L;
+  for (int i = (blockIdx.x * blockDim.x + threadIdx.x) / L; i < n; i += stride) {
+    if (vc[i] >= 0) continue;            // the same value in all lanes: only lane 0 writes it,
+                                         // at the end of this node's turn
+    const int a = rowptr[i], b = rowptr[i + 1];
+    bool wait = false;
+    unsigned low = 0, high = 0;          // colours 0..31 and 32..63 of the lower neighbours
+    for (int k = a + gl; k < b; k += L) {
+      const int j = col[k];
       if (j >= i) break;
-      if (vc[j] < 0) { ready = false; break; }
+      const int c = vc[j];
+      wait |= c < 0;
+      low |= c >= 0 && c < 32 ? 1u << c : 0u;
+      high |= c >= 32 && c < 64 ? 1u << (c - 32) : 0u;
     }
-    if (!ready) { atomicAdd(remaining, 1); continue; }
-    for (int base = 0; base <= b - a; base += 32) {
+#pragma unroll
+    for (int o = L / 2; o > 0; o >>= 1) {
+      low |= __shfl_xor_sync(group, low, o);
+      high |= __shfl_xor_sync(group, high, o);
+    }
+    wait = __any_sync(group, wait);
+    if (gl != 0) continue;
+    if (wait) { atomicAdd(remaining, 1); continue; }
+    if (low != 0xffffffffu) { vc[i] = __ffs(~low) - 1; continue; }
+    if (high != 0xffffffffu) { vc[i] = 32 + __ffs(~high) - 1; continue; }
+    for (int base = 64; base <= b - a; base += 32) {
       unsigned used = 0;
       for (int k = a; k < b; ++k) {
         int j = col[k];
@@ -617,17 +637,6 @@ __global__ void k_colour_round(int n, const int* __restrict__ rowptr, const int*
       }
     }
   }
-}
-
-__global__ void k_colour_flag(int n, const int* __restrict__ colour, int c, int* __restrict__ f) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    f[i] = colour[i] == c ? 1 : 0;
-}
-
-__global__ void k_colour_scatter(int n, const int* __restrict__ colour, int c,
-                                 const int* __restrict__ pos, int offset, int* __restrict__ rows) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    if (colour[i] == c) rows[offset + pos[i]] = i;
 }
 
 // stored-row lengths and block copy into colour order
@@ -1103,7 +1112,8 @@ void colour_graph(amg_handle* h, int n, const DBuf<int>& rowptr, const DBuf<int>
     if (round > n + batch) fail(AMG_ERR_TIMEOUT, "colouring rounds exceeded their bound");
     for (int b = 0; b < batch; ++b) {
       AMG_CUDA(cudaMemsetAsync(rem.p, 0, sizeof(int), s));
-      k_colour_round<<<grid_for(n), 256, 0, s>>>(n, rowptr, col, colour, rem);
+      k_colour_round<<<grid_for((int64_t)n * kColourLanes), 256, 0, s>>>(n, rowptr, col, colour,
+                                                                         rem);
       h->launches++;
     }
     AMG_LAUNCH_CHECK();
@@ -1117,20 +1127,15 @@ void colour_graph(amg_handle* h, int n, const DBuf<int>& rowptr, const DBuf<int>
   for (int c : hc) nc = std::max(nc, c + 1);
   ncolours = nc;
   colour_ptr.assign(nc + 1, 0);
+  // the nodes colour by colour, ascending within one (the colours are on the host; a scan
+  // and a scatter a colour were five launches and a wait each)
+  for (int c : hc) colour_ptr[c + 1]++;
+  for (int c = 0; c < nc; ++c) colour_ptr[c + 1] += colour_ptr[c];
+  std::vector<int> at(colour_ptr.begin(), colour_ptr.end()), order(n);
+  for (int i = 0; i < n; ++i) order[at[hc[i]]++] = i;
   rows.alloc(std::max(n, 1));
-  DBuf<int> fl, pos;
-  fl.alloc(std::max(n, 1));
-  pos.alloc(n + 1);
-  int off = 0;
-  for (int c = 0; c < nc; ++c) {
-    k_colour_flag<<<grid_for(n), 256, 0, s>>>(n, colour, c, fl);
-    int cnt = (int)exclusive_scan(fl, pos, n, s, h);
-    k_colour_scatter<<<grid_for(n), 256, 0, s>>>(n, colour, c, pos, off, rows);
-    h->launches += 2;
-    off += cnt;
-    colour_ptr[c + 1] = off;
-  }
-  AMG_LAUNCH_CHECK();
+  AMG_CUDA(cudaMemcpyAsync(rows.p, order.data(), n * sizeof(int), cudaMemcpyHostToDevice, s));
+  AMG_CUDA(cudaStreamSynchronize(s));
 }
 
 void row_stats(amg_handle* h, Level& lv) {

@@ -95,6 +95,25 @@ def test_weights_reach_the_stored_cycle(name, precision):
     assert torch.equal(apply(h, r), first)
 
 
+@pytest.mark.parametrize("precision", [0, 1])
+def test_weights_replace_a_large_stored_cycle(precision):
+    """A stored level of more than 4,096 unknowns (11^3: 5,202 on level 1) gives way to a
+    smaller one when its weights change, also for the captured CG loop."""
+    prob = fp.elasticity_problem(11, seed=3)
+    h, ops = pair(prob, precision=precision)
+    assert 4096 < 3 * h.level_info(1).n_nodes <= 6144
+    r = residual_like(prob, 6)
+    b = torch.from_numpy(prob.rhs()).cuda()
+    x, y = torch.zeros_like(b), torch.zeros_like(b)
+    for w in ((1.0, 1.0, 1.0), (0.9, 1.1, 1.0), (1.0, 1.0, 1.0)):
+        for q in (h, ops):
+            q.set_weights(*w)
+        z, ref = apply(h, r), apply(ops, r)
+        assert float((z - ref).norm() / ref.norm()) <= TOL[precision]
+        sa, sb = h.solve(b, x, 1e-8, True), ops.solve(b, y, 1e-8, True)
+        assert sa.converged and abs(sa.iterations - sb.iterations) <= 1
+
+
 def test_linear_and_repeatable():
     """M (a u + v) = a M u + M v within rounding, and equal bits on repetition."""
     prob = PROBLEMS["elasticity_9"]()
