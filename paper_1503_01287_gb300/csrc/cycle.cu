@@ -2289,7 +2289,8 @@ void e_residual(Emit<T>& e, Level& lv, const T* x, const T* b, T* r, bool saddle
 // One segregated Gauss-Seidel sweep, Eq. (uzsm), from x to y (other vectors):
 // u <- u + omega D^{-1} (f - B^T p - A u) (M_A: damped block Jacobi),
 // p <- p + omega_p S_D^{-1} (B u_new - C p - g).  From x = 0 the first is omega D^{-1} f, no
-// pass over A, and y may be x.
+// pass over A, and y may be x.  (With a pass over A times zero, separate B^T p and copies the
+// preconditioner of mixed 40^3 took 1195 us in 63 launches, now 815 in 27.)
 template <typename T>
 void e_sgs(Emit<T>& e, amg_handle* h, Level& lv, const T* x, const T* b, T* y, bool zero) {
   const int64_t n4 = 4 * (int64_t)lv.n;
