@@ -229,15 +229,28 @@ __device__ __forceinline__ void restrict_body(int nc, int nf, const int* __restr
       bc[4 * (int64_t)nc + k] = s;
       continue;
     }
+    // four entries at a time: their indices, then their gathers, are in flight together (one
+    // at a time a row of 30 entries was 30 dependent pairs of loads)
     T s0 = T(0), s1 = T(0), s2 = T(0);
-    for (int t = rrow[I]; t < rrow[I + 1]; ++t) {
-      const int i = rcol[t];
-      const T w = rval[t];
-      T r0, r1, r2;
-      VL<COH>::node(r, i, r0, r1, r2);
-      s0 = fma(w, r0, s0);
-      s1 = fma(w, r1, s1);
-      s2 = fma(w, r2, s2);
+    const int e = rrow[I + 1];
+    for (int t = rrow[I]; t < e; t += 4) {
+      int i[4];
+      T w[4], v[4][3];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int q = min(t + u, e - 1);
+        i[u] = rcol[q];
+        w[u] = t + u < e ? rval[q] : T(0);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) VL<COH>::node(r, i[u], v[u][0], v[u][1], v[u][2]);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (t + u >= e) break;
+        s0 = fma(w[u], v[u][0], s0);
+        s1 = fma(w[u], v[u][1], s1);
+        s2 = fma(w[u], v[u][2], s2);
+      }
     }
     st3(bc, I, s0, s1, s2);
   }
