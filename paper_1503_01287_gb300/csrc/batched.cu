@@ -475,7 +475,8 @@ constexpr int kGsTiles = 8; // colour kernel: tiles 0..3 as above, 4..7: S = 4 <
 // no cycle kernel writes) are loaded before griddepcontrol.wait, so this prologue
 // runs under the previous kernel; b, the relaxation multiplier and the x gathers
 // come after the wait, which is where the previous kernel's writes become
-// visible.  Tiles as in k_rows_m, and with S = 4 or 8 lane groups a row (2 or 4 warps,
+// visible.  x is gathered through L2 (ld3g): the colours before may be writing it while
+// this kernel is resident, and their gathers may have left old lines in the SM's L1.  Tiles as in k_rows_m, and with S = 4 or 8 lane groups a row (2 or 4 warps,
 // their sums combined in shared memory) for rows whose dependent block chain is long.
 template <typename T, int S, int U, bool FIRST>
 __global__ void __launch_bounds__(256) k_gs_m_pdl(int nrows, const int* __restrict__ rows,
@@ -531,7 +532,7 @@ __global__ void __launch_bounds__(256) k_gs_m_pdl(int nrows, const int* __restri
   for (int u = 0; u < U; ++u) {
     if (j[u] < 0) continue;
     T x0, x1, x2;
-    ld3(x, j[u] * K + r, x0, x1, x2);
+    ld3g(x, j[u] * K + r, x0, x1, x2);
     s0 = fma(v[u][0], x0, s0); s0 = fma(v[u][1], x1, s0); s0 = fma(v[u][2], x2, s0);
     s1 = fma(v[u][3], x0, s1); s1 = fma(v[u][4], x1, s1); s1 = fma(v[u][5], x2, s1);
     s2 = fma(v[u][6], x0, s2); s2 = fma(v[u][7], x1, s2); s2 = fma(v[u][8], x2, s2);
@@ -539,7 +540,7 @@ __global__ void __launch_bounds__(256) k_gs_m_pdl(int nrows, const int* __restri
   for (int k = a + q + U * S; active && k < e; k += S) {   // blocks beyond the prefetched ones
     const int jj = __ldg(col + k);
     T x0, x1, x2;
-    ld3(x, jj * K + r, x0, x1, x2);
+    ld3g(x, jj * K + r, x0, x1, x2);
     const T* vv = val + k;
     s0 = fma(__ldg(vv), x0, s0);
     s0 = fma(__ldg(vv + nnzb), x1, s0);
@@ -577,7 +578,7 @@ __global__ void __launch_bounds__(256) k_gs_m_pdl(int nrows, const int* __restri
   if (S >= 2 && q != 0) return;
   const int o = i * K + r;
   T x0 = T(0), x1 = T(0), x2 = T(0);
-  if (!FIRST) ld3(x, o, x0, x1, x2);
+  if (!FIRST) ld3g(x, o, x0, x1, x2);
   const T r0 = b0 - s0, r1 = b1 - s1, r2 = b2 - s2;
   if (FIRST && seed) st3(seed, o, (T(1) - om) * r0, (T(1) - om) * r1, (T(1) - om) * r2);
   st3(x, o, x0 + om * (d[0] * r0 + d[1] * r1 + d[2] * r2),
@@ -609,7 +610,9 @@ void launch_gs_m_pdl(int nrows, const int* rows, const int* rowptr, const int* r
 // time: the sweep waited on its load instructions and on rounds of gathers (12^3: 10 us a
 // colour).  Here a row's lanes load its columns and planes coalesced, each once, as three
 // 16-byte entries a block with the column in the first; the loop then takes three 16-byte
-// broadcasts from shared memory and one gather a block, eight gathers in flight.
+// broadcasts from shared memory and one gather a block, eight gathers in flight.  x through
+// L2 as above (10 problems of n in 8..24, 16 right-hand sides: 243 to 264 ms over three
+// draws, 266 with gathers through L1).
 // S lane groups of 16 a row (lane r of a group: right-hand side r), 16 / S rows a CTA; row
 // slots of `slot` blocks (the level's longest row) in dynamic shared memory.
 template <int S, bool FIRST>
@@ -657,7 +660,7 @@ __global__ void __launch_bounds__(256) k_gs_m_staged(
   for (; k + 7 * S < n; k += 8 * S) {
     float4 xv[8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) xv[u] = __ldg(x4 + (int64_t)__float_as_int(p0[k + u * S].w) * K);
+    for (int u = 0; u < 8; ++u) xv[u] = __ldcg(x4 + (int64_t)__float_as_int(p0[k + u * S].w) * K);
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       const float4 a = p0[k + u * S], c = p1[k + u * S], e = p2[k + u * S];
@@ -669,7 +672,7 @@ __global__ void __launch_bounds__(256) k_gs_m_staged(
 #pragma unroll 4
   for (; k < n; k += S) {
     const float4 a = p0[k], c = p1[k], e = p2[k];
-    const float4 v = __ldg(x4 + (int64_t)__float_as_int(a.w) * K);
+    const float4 v = __ldcg(x4 + (int64_t)__float_as_int(a.w) * K);
     s0 = fmaf(a.x, v.x, s0); s0 = fmaf(a.y, v.y, s0); s0 = fmaf(a.z, v.z, s0);
     s1 = fmaf(c.x, v.x, s1); s1 = fmaf(c.y, v.y, s1); s1 = fmaf(c.z, v.z, s1);
     s2 = fmaf(e.x, v.x, s2); s2 = fmaf(e.y, v.y, s2); s2 = fmaf(e.z, v.z, s2);
@@ -698,7 +701,7 @@ __global__ void __launch_bounds__(256) k_gs_m_staged(
   const int o = i * K + r;
   float b0, b1, b2, x0 = 0.f, x1 = 0.f, x2 = 0.f;
   ld3(b, o, b0, b1, b2);
-  if (!FIRST) ld3c(x, o, x0, x1, x2);
+  if (!FIRST) ld3g(x, o, x0, x1, x2);
   const float r0 = b0 - s0, r1 = b1 - s1, r2 = b2 - s2;
   if (FIRST && seed) st3(seed, o, (1.f - om) * r0, (1.f - om) * r1, (1.f - om) * r2);
   st3(x, o, x0 + om * (d[0] * r0 + d[1] * r1 + d[2] * r2),

@@ -56,17 +56,8 @@ struct VL<false> {
 };
 template <>
 struct VL<true> {
-  __device__ static void node(const float* p, int j, float& a, float& b, float& c) {
-    const float4 v = __ldcg(reinterpret_cast<const float4*>(p) + j);
-    a = v.x; b = v.y; c = v.z;
-  }
-  __device__ static void node(const double* p, int j, double& a, double& b, double& c) {
-    double w;
-    asm volatile("ld.global.cg.v4.f64 {%0, %1, %2, %3}, [%4];"
-                 : "=d"(a), "=d"(b), "=d"(c), "=d"(w)
-                 : "l"(p + 4 * (size_t)j)
-                 : "memory");
-  }
+  template <typename T>
+  __device__ static void node(const T* p, int j, T& a, T& b, T& c) { ld3g(p, j, a, b, c); }
   template <typename T>
   __device__ static T one(const T* p) { return __ldcg(p); }
 };

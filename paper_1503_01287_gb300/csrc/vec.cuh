@@ -34,6 +34,23 @@ __device__ __forceinline__ void ld3c(const double* p, int j, double& a, double& 
                : "memory");
 }
 
+// through L2 only.  A kernel under programmatic dependent launch may share an SM with the
+// kernels before it while these still write: what they write it reads like this, after
+// griddepcontrol.wait (an earlier load may have left the old line in L1, and ld.global.nc
+// is defined for data that nothing writes while the kernel runs).
+__device__ __forceinline__ void ld3g(const float* p, int j, float& a, float& b, float& c) {
+  const float4 v = __ldcg(reinterpret_cast<const float4*>(p) + j);
+  a = v.x; b = v.y; c = v.z;
+}
+
+__device__ __forceinline__ void ld3g(const double* p, int j, double& a, double& b, double& c) {
+  double w;
+  asm volatile("ld.global.cg.v4.f64 {%0, %1, %2, %3}, [%4];"
+               : "=d"(a), "=d"(b), "=d"(c), "=d"(w)
+               : "l"(p + 4 * (size_t)j)
+               : "memory");
+}
+
 __device__ __forceinline__ void st3(float* p, int j, float a, float b, float c) {
   reinterpret_cast<float4*>(p)[j] = make_float4(a, b, c, 0.f);
 }
