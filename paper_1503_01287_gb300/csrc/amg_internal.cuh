@@ -88,6 +88,7 @@ struct Level {
                                 // AMG_FP32_BF16 only)
   DBuf<double> dinv;    // 12 * n: per node 3 padded rows (4 values) of the inverse
   DBuf<float> dinv32;
+  float block_cond = 0.f;   // largest condition number of a diagonal block (row-sum norms)
   int ncolours = 0;
   std::vector<int> colour_ptr;  // host: offsets into colour_rows, ncolours+1
   DBuf<int> colour, colour_rows;
@@ -253,7 +254,7 @@ struct amg_handle {
   int64_t cg_loop_pcg_launches = 0, cg_loop_fcg_launches = 0;
   bool cg_loop_failed = false;
   bool iter_graph_failed = false;
-  amgp2::DBuf<int> flag;           // device error word
+  amgp2::DBuf<int> flag;           // device error word; [1]: scratch of the setup
   std::string last_error;
   int64_t launches = 0;
   double setup_ms = 0.0;

@@ -166,7 +166,7 @@ int amg_setup(const amg_matrix* m, const int32_t* node_tags, int32_t kind, const
       AMG_CUDA(cudaStreamCreateWithFlags(&h->own_stream, cudaStreamNonBlocking));
       h->stream = h->own_stream;
     }
-    h->flag.alloc(1);
+    h->flag.alloc(2);
     AMG_CUDA(cudaMallocHost(&h->host_scal, 8 * sizeof(double)));
     AMG_CUDA(cudaMallocHost(&h->host_int, 8 * sizeof(int)));
     auto t0 = std::chrono::steady_clock::now();

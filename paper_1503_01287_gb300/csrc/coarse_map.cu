@@ -677,6 +677,19 @@ constexpr int kMapMaxSgs = 4608;
 // it saves in one solve, at 8,538 (32^3) 17 ms for 3 ms.  A larger one gives way to one of at
 // most this size.
 constexpr int kMapMaxRebuild = 4096;
+// The worst conditioned diagonal block (row-sum norms) with which a cycle is stored.  M b
+// cancels where the operations do not: a block with directions of very different stiffness,
+// not along the axes, mixes them in every entry of M.  Against the cycle in FP64 (elasticity
+// 12x11x13, its blocks D taken to Q S D S Q^T with S = diag(1, t, 1)), FP32:
+//   t = 8    (condition 113)    operations 5.5e-7, stored 5.7e-7
+//   t = 20   (condition 715)               3.4e-6         3.7e-6
+//   t = 100  (condition 1.7e4)             1.1e-4         2.6e-4
+//   t = 1000 (9x8x10)                      1.4e-2         2.1e-1: CG took 45 iterations with
+//            the operations and did not converge with the matrix
+// In FP64, whose M is built without low parts, the two differ by 1e-15, 2e-14 and 1.6e-11 at
+// t = 8, 20 and 100.  Elasticity has 4 (nu = 0.3), 13 (0.45), 61 (0.49); stretched boxes and
+// jumps of the coefficient 5; there M is as close as the operations.
+constexpr float kMapMaxCond = 128.f;
 // and the share of the coarsest solve (FP64) in the construction
 constexpr int64_t kMapCoarseWork = 4000000000ll;
 
@@ -687,6 +700,8 @@ constexpr int kMapMaxBatch = 4096;
 // the first level of at most `most` unknowns, its matrix allocated and zero
 void plan(amg_handle* h, CoarseMap& M, int most) {
   const bool f32 = h->opt.precision == AMG_FP32;
+  for (const auto& lv : h->L)
+    if (!(lv->block_cond <= kMapMaxCond)) return;
   for (int l = 0; l + 1 < (int)h->L.size(); ++l) {
     const int m = h->L[l]->dofs();
     if (m > most || (int64_t)h->coarse_m * h->coarse_m * m > kMapCoarseWork) continue;

@@ -696,9 +696,12 @@ __global__ void k_stored_copy(int n, const int* __restrict__ order, const int* _
 
 // ============================================================================ block inverses
 
+// Inverses of the diagonal blocks (padded rows).  flag[0]: a block is singular; flag[1]: the
+// largest condition number ||D|| ||D^{-1}|| (maximum row sums), as the bits of a float.
 __global__ void k_dinv(int n, const int* __restrict__ rowptr, const int* __restrict__ col,
                        const double* __restrict__ val, int64_t nnzb, double* __restrict__ dinv,
                        int* __restrict__ flag) {
+  float worst = 0.f;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     int lo = rowptr[i], hi = rowptr[i + 1] - 1;
     while (lo < hi) {
@@ -728,7 +731,17 @@ __global__ void k_dinv(int n, const int* __restrict__ rowptr, const int* __restr
     o[9] = (a[1] * a[6] - a[0] * a[7]) * r;
     o[10] = (a[0] * a[4] - a[1] * a[3]) * r;
     o[11] = 0.0;
+    double na = 0.0, no = 0.0;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      na = fmax(na, fabs(a[3 * q]) + fabs(a[3 * q + 1]) + fabs(a[3 * q + 2]));
+      no = fmax(no, fabs(o[4 * q]) + fabs(o[4 * q + 1]) + fabs(o[4 * q + 2]));
+    }
+    worst = fmaxf(worst, (float)(na * no));
   }
+  // positive floats are ordered as their bits
+  worst = __int_as_float(__reduce_max_sync(0xffffffffu, __float_as_int(worst)));
+  if ((threadIdx.x & 31) == 0) atomicMax(flag + 1, __float_as_int(worst));
 }
 
 // sGS pressure scaling S_D[k] = C_kk + omega * sum_j b_kj^T D_j^{-1} b_kj
@@ -1154,12 +1167,15 @@ void finish_level(amg_handle* h, Level& lv, bool coarsest) {
   int n = lv.n;
   row_stats(h, lv);
   lv.dinv.alloc(12 * (size_t)std::max(n, 1));
-  Flag f(h);
-  f.reset();
+  AMG_CUDA(cudaMemsetAsync(h->flag.p, 0, 2 * sizeof(int), s));
   k_dinv<<<grid_for(n), 256, 0, s>>>(n, lv.rowptr, lv.col, lv.val, lv.nnzb, lv.dinv, h->flag);
   AMG_LAUNCH_CHECK();
   h->launches++;
-  if (f.read()) fail(AMG_ERR_BREAKDOWN, "singular or non-finite 3x3 diagonal block");
+  int found[2];
+  AMG_CUDA(cudaMemcpyAsync(found, h->flag.p, sizeof found, cudaMemcpyDeviceToHost, s));
+  AMG_CUDA(cudaStreamSynchronize(s));
+  if (found[0]) fail(AMG_ERR_BREAKDOWN, "singular or non-finite 3x3 diagonal block");
+  std::memcpy(&lv.block_cond, &found[1], sizeof(float));
   if (!coarsest && !h->saddle) {
     colour_level(h, lv);
     // colour-major copy of A for the cycle kernels
