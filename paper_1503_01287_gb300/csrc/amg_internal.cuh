@@ -319,7 +319,7 @@ void precondition_device(amg_handle* h, const double* r, double* z);
 void apply_pair(amg_handle* h, const float* xp, double* y);
 void apply_K_pair(amg_handle* h, const double* x, float* xp, double* y);
 // The same in parts for a float x (padded): the velocity block as pairs, yp = A x; and on
-// stream s B^T p as pairs (4 n entries, t: two floats an entry) and B u - C p (FP64, y at
+// stream s B^T p in three floats an entry (t: 12 floats a node) and B u - C p (FP64, y at
 // 4 n) of the padded FP64 vector z
 void apply_pair_f32(amg_handle* h, const float* x, float2* yp);
 void apply_B_parts(amg_handle* h, const double* z, float* t, double* y, cudaStream_t s);

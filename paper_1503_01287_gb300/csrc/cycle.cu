@@ -1403,10 +1403,18 @@ void launch_apply_pair(const Level& lv, const float* xp, Y* y, cudaStream_t s) {
   }
 }
 
-// (B^T p)_i as pairs (summed in FP64), thread per velocity node
-__global__ void k_bt_pair(int n, const int* __restrict__ row, const int* __restrict__ col,
-                          const double* __restrict__ val, int64_t nnz,
-                          const double* __restrict__ p, float4* __restrict__ t) {
+// (B^T p)_i summed in FP64, each sum left as three floats that add up to it (hi, its error,
+// the last bits: 24 + 24 + 5), so that it joins a pair without FP64 work there.  Thread per
+// velocity node, three float4 a node.
+__device__ __forceinline__ void split3(double v, float& a, float& b, float& c) {
+  a = __double2float_rn(v);
+  const double r = v - (double)a;
+  b = __double2float_rn(r);
+  c = __double2float_rn(r - (double)b);
+}
+__global__ void k_bt_split(int n, const int* __restrict__ row, const int* __restrict__ col,
+                           const double* __restrict__ val, int64_t nnz,
+                           const double* __restrict__ p, float4* __restrict__ t) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     double s0 = 0.0, s1 = 0.0, s2 = 0.0;
     for (int q = row[i]; q < row[i + 1]; ++q) {
@@ -1415,9 +1423,14 @@ __global__ void k_bt_pair(int n, const int* __restrict__ row, const int* __restr
       s1 = fma(val[nnz + q], pk, s1);
       s2 = fma(val[2 * nnz + q], pk, s2);
     }
-    const float2 a = to_pair(s0), b = to_pair(s1), c = to_pair(s2);
-    t[2 * (int64_t)i] = make_float4(a.x, a.y, b.x, b.y);
-    t[2 * (int64_t)i + 1] = make_float4(c.x, c.y, 0.f, 0.f);
+    float4 a, b, c;
+    split3(s0, a.x, b.x, c.x);
+    split3(s1, a.y, b.y, c.y);
+    split3(s2, a.z, b.z, c.z);
+    a.w = b.w = c.w = 0.f;
+    t[3 * (int64_t)i] = a;
+    t[3 * (int64_t)i + 1] = b;
+    t[3 * (int64_t)i + 2] = c;
   }
 }
 
@@ -2789,14 +2802,17 @@ void apply_pair_f32(amg_handle* h, const float* x, float2* yp) {
 
 void apply_B_parts(amg_handle* h, const double* z, float* t, double* y, cudaStream_t s) {
   Level& lv = *h->L[0];
-  k_bt_pair<<<gridn(lv.n), 256, 0, s>>>(lv.n, lv.bt_rowptr, lv.bt_col, lv.bt_val, lv.b_nnz,
-                                        z + 4 * (int64_t)lv.n, reinterpret_cast<float4*>(t));
+  k_bt_split<<<gridn(lv.n), 256, 0, s>>>(lv.n, lv.bt_rowptr, lv.bt_col, lv.bt_val, lv.b_nnz,
+                                         z + 4 * (int64_t)lv.n, reinterpret_cast<float4*>(t));
   h->launches++;
-  const cudaStream_t own = h->stream;
+  struct Stream {   // the handle's stream comes back, also where a launch fails
+    amg_handle* h;
+    cudaStream_t own;
+    ~Stream() { h->stream = own; }
+  } back{h, h->stream};
   h->stream = s;
   Emit<double> e{h};
   e.prows(0, lv, z, z + 4 * (int64_t)lv.n, nullptr, y + 4 * (int64_t)lv.n, 0.0);
-  h->stream = own;
 }
 
 // y = K_0 x with the velocity block in FP32-pair arithmetic (x split into xp, 8 floats a

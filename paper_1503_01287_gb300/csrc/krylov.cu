@@ -442,9 +442,19 @@ __global__ void k_to_pair(int64_t n, const double* __restrict__ a, float2* __res
     b[k] = to_pair(a[k]);
 }
 
-// the parts of w = K z as pairs: velocity entries (k < n4) w_k + t_k, t = B^T p; pressure
-// entries from the FP64 vector d
-__global__ void k_join(int64_t n, int64_t n4, const float2* __restrict__ t,
+// a + b with its rounding error in e (TwoSum, Knuth)
+__device__ __forceinline__ float two_sum(float a, float b, float& e) {
+  const float t = __fadd_rn(a, b);
+  const float q = __fsub_rn(t, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(t, q)), __fsub_rn(b, q));
+  return t;
+}
+
+// the parts of w = K z as pairs: velocity entries (k < n4) w_k + t_k, t = B^T p in three
+// floats (12 a node), to 2^-48 of the sum also where the two cancel, as their sum in FP64
+// was; pressure entries from the FP64 vector d.  Memory bound, 28 bytes an entry (with B^T p
+// rounded to a pair, 24: mixed 40^3 230.1 against 231.7 ms a solve).
+__global__ void k_join(int64_t n, int64_t n4, const float* __restrict__ t,
                        const double* __restrict__ d, float2* __restrict__ w) {
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
        k += (int64_t)gridDim.x * blockDim.x) {
@@ -452,10 +462,14 @@ __global__ void k_join(int64_t n, int64_t n4, const float2* __restrict__ t,
       w[k] = to_pair(d[k]);
       continue;
     }
-    float2 a = w[k];
-    const float2 b = t[k];
-    pair_add(a.x, a.y, b.x, b.y);
-    w[k] = norm_pair(a.x, a.y);
+    const float2 a = w[k];
+    const float* b = t + 12 * (k >> 2) + (k & 3);
+    float e1, e2, e3, e4;
+    const float s = two_sum(a.x, b[0], e1);
+    const float l = two_sum(a.y, b[4], e2);
+    const float m = two_sum(e1, l, e3);
+    const float hi = two_sum(s, m, e4);
+    w[k] = norm_pair(hi, __fadd_rn(e4, __fadd_rn(__fadd_rn(e2, e3), b[8])));
   }
 }
 
@@ -1012,8 +1026,7 @@ int solve_fgmres(amg_handle* h, Ctx& c, const double* b, double* x, double tol, 
       AMG_CUDA(cudaEventRecord(h->join, h->side));
       apply_pair_f32(h, lv.x32, wp);
       AMG_CUDA(cudaStreamWaitEvent(s, h->join, 0));
-      k_join<<<gridr(n), 256, 0, s>>>(n, 4 * (int64_t)lv.n, reinterpret_cast<const float2*>(pf),
-                                      w, wp);
+      k_join<<<gridr(n), 256, 0, s>>>(n, 4 * (int64_t)lv.n, pf, w, wp);
       h->launches++;
       return;
     }
@@ -1198,8 +1211,10 @@ int solve_device(amg_handle* h, const double* b_user, double* x_user, double tol
   };
   ensure(h->kb, n); ensure(h->kx, n);
   ensure(h->kr, n); ensure(h->kz, n); ensure(h->kp, n); ensure(h->kq, n); ensure(h->kw, n);
-  if (lv.val2.p && (int64_t)h->kpf.n < 2 * n) {
-    h->kpf.alloc(2 * n);
+  // a vector in pairs, or B^T p in three floats an entry (saddle kinds)
+  const int64_t npf = (h->saddle ? 3 : 2) * n;
+  if (lv.val2.p && (int64_t)h->kpf.n < npf) {
+    h->kpf.alloc(npf);
     AMG_CUDA(cudaMemsetAsync(h->kpf.p, 0, h->kpf.bytes(), h->stream));
   }
   ensure(h->red, (int64_t)kReduceBlocks * kMaxDots);
