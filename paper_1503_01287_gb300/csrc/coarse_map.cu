@@ -690,6 +690,14 @@ constexpr int kMapMaxRebuild = 4096;
 // t = 8, 20 and 100.  Elasticity has 4 (nu = 0.3), 13 (0.45), 61 (0.49); stretched boxes and
 // jumps of the coefficient 5; there M is as close as the operations.
 constexpr float kMapMaxCond = 128.f;
+// K of Stokes is singular: the constant pressure is in every column of M, and the response to
+// it in every pressure column, and what is left of them after M b cancelled is the rounding of
+// large entries.  Error of the projected result over 16 residuals K x, stored against
+// operations: FP32 1.6 times on the average of 5^3 to 24^3 (9.8 at 5^3); FP64 5 to 9 times from
+// level 0 (5^3), 1.0 to 1.9 from level 1 (6^3 to 9^3), 1.00 from level 2 (12^3 to 24^3).
+// (Mixed elasticity: 0.94 to 1.10 in FP32, 1.0 to 1.4 in FP64; elasticity and the Laplacian at
+// most 1 in FP32, in FP64 2 to 2.8 from level 0, at 5e-16, and 0.8 to 1.3 below.)
+constexpr int kMapStokesFrom = 2;
 // and the share of the coarsest solve (FP64) in the construction
 constexpr int64_t kMapCoarseWork = 4000000000ll;
 
@@ -702,7 +710,9 @@ void plan(amg_handle* h, CoarseMap& M, int most) {
   const bool f32 = h->opt.precision == AMG_FP32;
   for (const auto& lv : h->L)
     if (!(lv->block_cond <= kMapMaxCond)) return;
-  for (int l = 0; l + 1 < (int)h->L.size(); ++l) {
+  const bool stokes = h->kind == AMG_STOKES;
+  if (stokes && f32) return;
+  for (int l = stokes ? kMapStokesFrom : 0; l + 1 < (int)h->L.size(); ++l) {
     const int m = h->L[l]->dofs();
     if (m > most || (int64_t)h->coarse_m * h->coarse_m * m > kMapCoarseWork) continue;
     M.m = m;
