@@ -449,6 +449,7 @@ def run_gpu(args, rank, world):
                    "gs_cluster_ctas": stats[-1]["level_gs_cluster"],
                    "gs_flow_lanes": stats[-1]["level_gs_flow"],
                    "gs_stream_ctas_per_sm": stats[-1]["level_gs_stream"],
+                   "stored_from": stats[-1]["stored_from"],
                    "cluster_from": stats[-1]["cluster_from"],
                    "cycle_kernel": stats[-1]["cycle_kernel"]},
         "plain_fp64": {"value": world * ndof / (ms_plain * 1e-3), "ms_per_step": ms_plain,

@@ -232,7 +232,8 @@ typedef struct amg_stats {
   int32_t iterations;       /* Krylov iterations (operator applications)       */
   int32_t converged;
   int32_t n_levels;
-  int32_t pad0;
+  int32_t stored_from;      /* k >= 1: the cycle from level k - 1 down ran as the
+                               stored matrix (see cluster_from); 0: none        */
   double rel_residual;      /* recursive residual estimate at exit              */
   double true_rel_residual; /* ||b - K x|| / ||b|| recomputed at exit           */
   double setup_ms;
@@ -245,7 +246,8 @@ typedef struct amg_stats {
   int32_t level_group[AMG_MAX_LEVELS];  /* lanes per block row chosen at setup       */
   int32_t cluster_from;     /* cycle variant in use: first level of the cluster
                                sub-cycle (0: none)                              */
-  int32_t cycle_kernel;     /* 1: one launch per operation, 2: persistent cycle */
+  int32_t cycle_kernel;     /* 1: one launch per operation (above the stored
+                               level, if any), 2: persistent cycle             */
   int32_t level_gs_cluster[AMG_MAX_LEVELS];  /* CTAs of the one-cluster sweep
                                (0: one launch per colour)                       */
   int32_t level_gs_flow[AMG_MAX_LEVELS];     /* lanes per row of the one-launch
