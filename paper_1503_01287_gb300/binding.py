@@ -80,7 +80,7 @@ class AmgOptions(C.Structure):
 
 class AmgStats(C.Structure):
     _fields_ = [("iterations", C.c_int32), ("converged", C.c_int32), ("n_levels", C.c_int32),
-                ("pad0", C.c_int32), ("rel_residual", C.c_double),
+                ("stored_from", C.c_int32), ("rel_residual", C.c_double),
                 ("true_rel_residual", C.c_double), ("setup_ms", C.c_double),
                 ("solve_ms", C.c_double), ("kernel_launches", C.c_int64),
                 ("level_nodes", C.c_int32 * AMG_MAX_LEVELS),
@@ -97,7 +97,8 @@ class AmgStats(C.Structure):
     def as_dict(self) -> dict:
         nl = self.n_levels
         return {"iterations": self.iterations, "converged": bool(self.converged),
-                "n_levels": nl, "rel_residual": self.rel_residual,
+                "n_levels": nl, "stored_from": self.stored_from,
+                "rel_residual": self.rel_residual,
                 "true_rel_residual": self.true_rel_residual, "setup_ms": self.setup_ms,
                 "solve_ms": self.solve_ms, "kernel_launches": self.kernel_launches,
                 "level_nodes": list(self.level_nodes[:nl]),

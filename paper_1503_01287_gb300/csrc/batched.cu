@@ -1261,6 +1261,7 @@ int solve_batched(amg_handle* const* hs, int np, int nrhs, const double* const* 
       st.iterations = it;
       st.converged = conv;
       st.n_levels = (int)h->L.size();
+      st.stored_from = h->batch_map ? h->batch_map->from + 1 : 0;
       st.true_rel_residual = worst;
       st.rel_residual = worst;
       st.solve_ms = ms;
