@@ -211,14 +211,19 @@ struct BatchLevel {
   int tile_gs = 0;     // tile of the multi-right-hand-side colour kernel
 };
 
-// The cycle from level `from` down (from x = 0) as an m x m matrix, row-major with rows ld
-// apart, in the cycle's precision (from = -1: off).
+// The cycle from level `level` down (from x = 0) as an m x m matrix, row-major with rows ld
+// apart, in the cycle's precision (level = -1: none).  from: level where the matrix is in use,
+// -1 where the level weights are not those that it was built with.
 struct CoarseMap {
-  int from = -1;
+  int level = -1, from = -1;
   int m = 0, ld = 0;
   DBuf<float> m32;
   DBuf<double> m64;
-  std::vector<double> w;   // the level weights that it was built with
+  std::vector<double> w, seen;   // its levels' weights: as built, and the current ones
+  int64_t waited = 0;            // applications without it since these are the current ones
+  void used(int64_t applications) {
+    if (level >= 0 && from < 0) waited += applications;
+  }
 };
 
 }  // namespace amgp2
@@ -250,8 +255,9 @@ struct amg_handle {
   double* host_scal = nullptr;     // pinned
   int* host_int = nullptr;         // pinned
   amgp2::DBuf<int> it_dev;         // device: iteration counter of the graph loop, ticket
-  cudaGraphExec_t cg_loop_pcg = nullptr, cg_loop_fcg = nullptr;   // whole-solve loops
-  int64_t cg_loop_pcg_launches = 0, cg_loop_fcg_launches = 0;
+  // whole-solve loops, without and with the stored cycle
+  cudaGraphExec_t cg_loop_pcg[2] = {}, cg_loop_fcg[2] = {};
+  int64_t cg_loop_pcg_launches[2] = {}, cg_loop_fcg_launches[2] = {};
   bool cg_loop_failed = false;
   bool iter_graph_failed = false;
   amgp2::DBuf<int> flag;           // device error word; [1]: scratch of the setup
@@ -275,13 +281,14 @@ struct amg_handle {
   // the cycle from a level down as one stored matrix (coarse_map.cu), and a smaller one
   // for batched solves where that one is too large for 16 right-hand sides
   amgp2::CoarseMap map, bmap;
-  const amgp2::CoarseMap* batch_map = nullptr;   // of the two, for the batched cycle
+  amgp2::CoarseMap* batch_map = nullptr;   // of the two, for the batched cycle
   // batched (multi-right-hand-side) solves
   std::vector<amgp2::BatchLevel> B;
   amgp2::DBuf<double> mb, mx, mr, mz, mp, mq, mro, bred, bscal;
   amgp2::DBuf<float> mpf;           // the directions in pair form (FP32-pair operator)
   amgp2::DBuf<int> bit;
   amgp2::DBuf<double> wts;          // 4 learned weights per level: ws, wc, wp, 1
+  std::vector<double> weights;      // the same on the host
   amgp2::DBuf<double> steps;        // 4 steps per level (Level::wt)
   amgp2::DBuf<float> steps32;
   bool bf16_coarse = false;         // AMG_FP32_BF16: levels >= 1 keep BF16 values
@@ -340,10 +347,15 @@ void set_subcycle(amg_handle* h, int from);
 // coarse_map.cu: the cycle below a level as one stored matrix
 // picks the level of h->map and allocates the matrix (before autotune_levels)
 void map_plan(amg_handle* h);
-// the map of the batched solves: h->map, or h->bmap planned here; null: none.  Filled.
-const CoarseMap* map_batch(amg_handle* h);
-// fills the maps for the level weights w (host, 4 a level); again when they changed
-void map_build(amg_handle* h, const double* w);
+// fills h->map for the current level weights
+void map_build(amg_handle* h);
+// the level weights changed: the maps are in use where they were built with them
+void map_follow(amg_handle* h);
+// fills M for the current weights once enough applications ran without it (M.used); for calls
+// that may allocate
+void map_refresh(amg_handle* h, CoarseMap& M);
+// the map of the batched solves: h->map, or h->bmap planned here; null: none
+CoarseMap* map_batch(amg_handle* h);
 // x = (the cycle from level map.from) b, vectors of that level in the padded layout
 template <typename T, typename IO>
 void map_apply(amg_handle* h, const IO* b, IO* x);

@@ -64,8 +64,7 @@ amg_handle::~amg_handle() {
   if (host_scal) cudaFreeHost(host_scal);
   if (host_int) cudaFreeHost(host_int);
   if (cycle_graph) cudaGraphExecDestroy(cycle_graph);
-  if (cg_loop_pcg) cudaGraphExecDestroy(cg_loop_pcg);
-  if (cg_loop_fcg) cudaGraphExecDestroy(cg_loop_fcg);
+  drop_loops(this);
   L.clear();
   coarse_inv.release();
   if (fork) cudaEventDestroy(fork);
@@ -275,6 +274,8 @@ int amg_solve(amg_handle* h, const double* b, double* x, double rel_tol, int32_t
     AMG_CUDA(cudaEventRecord(e0, h->stream));
     nvtxRangePushA(h->opt.precision == AMG_FP32 ? "amg_solve_fp32" : "amg_solve_fp64");
     struct Pop { ~Pop() { nvtxRangePop(); } } pop;
+    map_refresh(h, h->map);
+    st->stored_from = h->map.from + 1;
     int rc;
     if (device_ptrs) {
       rc = solve_device(h, b, x, rel_tol, st);
@@ -291,6 +292,7 @@ int amg_solve(amg_handle* h, const double* b, double* x, double rel_tol, int32_t
     AMG_CUDA(cudaEventRecord(e1, h->stream));
     AMG_CUDA(cudaEventSynchronize(e1));
     check_wait_flag(h, "the solve");
+    h->map.used(st->iterations);
     float ms = 0.f;
     AMG_CUDA(cudaEventElapsedTime(&ms, e0, e1));
     cudaEventDestroy(e0);
@@ -474,6 +476,8 @@ int amg_apply_preconditioner(amg_handle* h, const double* r, double* z) {
     Level& lv = *h->L[0];
     const int64_t n4 = lv.dofs4();
     if ((int64_t)h->kr.n < n4) { h->kr.alloc(n4); h->kz.alloc(n4); }
+    map_refresh(h, h->map);
+    h->map.used(1);
     launch_to_padded(r, h->kr, lv.n, lv.np, h->stream, h);
     if (h->opt.precision == AMG_FP32) precondition_device<float>(h, h->kr, h->kz);
     else precondition_device<double>(h, h->kr, h->kz);

@@ -1254,6 +1254,8 @@ int solve_batched(amg_handle* const* hs, int np, int nrhs, const double* const* 
       if (sc[M_ACT * K + r] != 0.0) conv = false;
     }
     if (!conv) rc = AMG_NOT_CONVERGED;
+    const int stored_from = h->batch_map ? h->batch_map->from + 1 : 0;
+    if (h->batch_map) h->batch_map->used(it);
     h->launches = l0[p] + per_iter[p] * it;
     if (stats) {
       amg_stats& st = stats[p];
@@ -1261,7 +1263,7 @@ int solve_batched(amg_handle* const* hs, int np, int nrhs, const double* const* 
       st.iterations = it;
       st.converged = conv;
       st.n_levels = (int)h->L.size();
-      st.stored_from = h->batch_map ? h->batch_map->from + 1 : 0;
+      st.stored_from = stored_from;
       st.true_rel_residual = worst;
       st.rel_residual = worst;
       st.solve_ms = ms;

@@ -6,9 +6,10 @@
 // of about 2 x 30 colours and 5 other launches a level, each a few microseconds whatever
 // the level's size (elasticity 32^3, FP32: 280 us of the 774 us preconditioner below
 // level 1, for 8,538 unknowns; FP64 24^3: 690 us of 1317 us for 3,144).  M b instead reads
-// m^2 values once.  M is filled at setup, and again when the level weights change, by
-// running the cycle's own recorded operations on blocks of unit vectors, so it is the same
-// operator, weights, smoother and cycle type, in the cycle's precision.
+// m^2 values once.  M is filled at setup by running the cycle's own recorded operations on
+// blocks of unit vectors, so it is the same operator, weights, smoother and cycle type, in the
+// cycle's precision.  Under other level weights the cycle runs operation by operation, until
+// M is filled for them (map_refresh); back under its own weights M is in use again.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -467,7 +468,7 @@ void build(amg_handle* h, const CoarseMap& map, S* M) {
   // all columns at once up to kColMax: a launch's CTAs go over the rows of a colour first,
   // so a block of 256 columns keeps its vectors in L2, and the small colours still fill the
   // chip (512 columns a pass at 32^3: 97 ms, all but a few launches waiting on latency)
-  const int from = map.from, m = map.m;
+  const int from = map.level, m = map.m;
   int W = div_up(div_up(m, div_up(m, kColMax)), kColBlock) * kColBlock;
   std::vector<Phase> ph;
   record_map_phases<S>(h, from, ph);
@@ -673,10 +674,14 @@ constexpr int kMapMax64 = 6144;
 // A segregated Gauss-Seidel level is 7 launches, not 65: Stokes 24^3 in FP64 gains 60 us of
 // 580 a preconditioner by its map of 4,159, built in 16 ms.
 constexpr int kMapMaxSgs = 4608;
-// The largest map that a change of weights builds again: at 4,096 it takes about the 4 ms that
-// it saves in one solve, at 8,538 (32^3) 17 ms for 3 ms.  A larger one gives way to one of at
-// most this size.
-constexpr int kMapMaxRebuild = 4096;
+// Applications operation by operation, under weights that M was not built with, after which
+// it is filled for them: by then what M would have saved is about what filling it costs, so a
+// program that changes weights often loses nothing and one that keeps them waits at most
+// about twice.  Measured filling time over the time that an application saves: FP32 14 at
+// 1,029 unknowns, 16 at 1,263, 35 at 2,793, 37 at 4,159, 90 at 8,538; FP64 15 at 828, 14 at
+// 1,029, 40 at 2,793, 115 at 4,159 (Stokes, whose cycle saves least).
+inline int64_t map_pays(const CoarseMap& M) { return 10 + M.m / (M.m32.p ? 100 : 60); }
+
 // The worst conditioned diagonal block (row-sum norms) with which a cycle is stored.  M b
 // cancels where the operations do not: a block with directions of very different stiffness,
 // not along the axes, mixes them in every entry of M.  Against the cycle in FP64 (elasticity
@@ -728,39 +733,41 @@ void plan(amg_handle* h, CoarseMap& M, int most) {
     // the padding of the rows stays 0
     if (f32) AMG_CUDA(cudaMemsetAsync(M.m32.p, 0, M.m32.bytes(), h->stream));
     else AMG_CUDA(cudaMemsetAsync(M.m64.p, 0, M.m64.bytes(), h->stream));
-    M.from = l;
+    M.level = l;
     return;
   }
 }
 
-void fill(amg_handle* h, CoarseMap& M, const double* w) {
-  if (M.from < 0) return;
-  // the weights of the levels that M holds (4 a level): nothing to do if they are as built
-  const std::vector<double> now(w + 4 * M.from, w + 4 * h->L.size());
-  if (now == M.w) return;
-  const bool again = !M.w.empty();
+// the weights of the levels that M holds (4 a level)
+std::vector<double> own_weights(const amg_handle* h, const CoarseMap& M) {
+  return {h->weights.begin() + 4 * M.level, h->weights.end()};
+}
+
+// M of the handle's current weights
+void fill(amg_handle* h, CoarseMap& M) {
+  if (M.level < 0) return;
+  M.from = -1;
   M.w.clear();
-  if (again && M.m > kMapMaxRebuild) {
-    M.from = -1;
-    M.m32.release();
-    M.m64.release();
-    drop_loops(h);
-    plan(h, M, kMapMaxRebuild);
-    fill(h, M, w);
-    return;
-  }
   try {
     if (M.m32.p) build<Pair, float>(h, M, M.m32.p);
     else build<double, double>(h, M, M.m64.p);
   } catch (const Error& e) {
-    M.from = -1;   // the cycle runs operation by operation, in newly captured loops
-    M.m32.release();
-    M.m64.release();
+    M = CoarseMap{};   // the cycle runs operation by operation
     drop_loops(h);
     if (e.code != AMG_ERR_NOMEM) throw;
     return;
   }
-  M.w = now;
+  M.w = M.seen = own_weights(h, M);
+  M.from = M.level;
+}
+
+// in use where the weights are those that it was built with
+void follow(amg_handle* h, CoarseMap& M) {
+  if (M.level < 0) return;
+  const std::vector<double> now = own_weights(h, M);
+  if (now != M.seen) M.waited = 0;
+  M.seen = now;
+  M.from = now == M.w ? M.level : -1;
 }
 
 }  // namespace
@@ -777,27 +784,29 @@ void map_plan(amg_handle* h) {
                                       : kMapMax64);
 }
 
-const CoarseMap* map_batch(amg_handle* h) {
+CoarseMap* map_batch(amg_handle* h) {
   // the batched cycle reads the FP32 values of every level, also with BF16 storage
-  if (h->map.from < 0 || !h->map.m32.p || h->bf16_coarse || h->opt.batch_tile != -1)
+  if (h->map.level < 0 || !h->map.m32.p || h->bf16_coarse || h->opt.batch_tile != -1)
     return nullptr;
-  if (h->map.m <= kMapMaxBatch) {
-    h->bmap = CoarseMap{};   // of a larger map that gave way
-    return &h->map;
+  CoarseMap& M = h->map.m <= kMapMaxBatch ? h->map : h->bmap;
+  if (M.level < 0) {
+    plan(h, M, kMapMaxBatch);
+    fill(h, M);
+    if (M.level < 0) return nullptr;
   }
-  if (h->bmap.from < 0) {
-    plan(h, h->bmap, kMapMaxBatch);
-    if (h->bmap.from < 0) return nullptr;
-    std::vector<double> w(4 * h->L.size());
-    get_weights(h, w.data());
-    fill(h, h->bmap, w.data());
-  }
-  return &h->bmap;
+  map_refresh(h, M);
+  return &M;
 }
 
-void map_build(amg_handle* h, const double* w) {
-  fill(h, h->map, w);
-  fill(h, h->bmap, w);
+void map_build(amg_handle* h) { fill(h, h->map); }
+
+void map_follow(amg_handle* h) {
+  follow(h, h->map);
+  follow(h, h->bmap);
+}
+
+void map_refresh(amg_handle* h, CoarseMap& M) {
+  if (M.level >= 0 && M.from < 0 && M.waited >= map_pays(M)) fill(h, M);
 }
 
 void map_apply_m(amg_handle* h, const CoarseMap& M, const float* b, float* x) {

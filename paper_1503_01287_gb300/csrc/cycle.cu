@@ -2871,7 +2871,7 @@ void autotune_levels(amg_handle* h) {
   for (auto& lv : h->L)
     if (lv->ncolours > 0) lv->group_gs = gs_lanes(f32, (double)lv->n / lv->ncolours);
   // levels that run as one stored matrix keep the default lanes per row
-  const size_t nl = h->map.from >= 0 ? std::max(h->map.from, 1) : h->L.size();
+  const size_t nl = h->map.level >= 0 ? std::max(h->map.level, 1) : h->L.size();
   for (size_t l = 0; l < nl; ++l) {
     Level& lv = *h->L[l];
     lv.gs_cl = 0;
@@ -2921,10 +2921,10 @@ void autotune_levels(amg_handle* h) {
       AMG_CUDA(cudaStreamSynchronize(s));
     }
     if (lv.ncolours == 0 || h->saddle || h->opt.smoother != AMG_SMOOTHER_GS ||
-        h->map.from == 0)
+        h->map.level == 0)
       continue;
     lv.gs_stream = 0;
-    if (h->map.from >= 0) continue;   // the other sweep kernels below were slower on every
+    if (h->map.level >= 0) continue;   // the other sweep kernels below were slower on every
                                       // level that the stored matrix leaves to the chain
     auto sweep_ms = [&]() {
       for (int r = 0; r < 7; ++r) {
@@ -3091,7 +3091,7 @@ void autotune_levels(amg_handle* h) {
       fail(AMG_ERR_TIMEOUT, "a bounded wait of a one-launch colour sweep (mbarrier or dataflow "
                             "flag) timed out during setup tuning");
   }
-  if (h->map.from >= 0) {
+  if (h->map.level >= 0) {
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     return;

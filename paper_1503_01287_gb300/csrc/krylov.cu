@@ -795,8 +795,9 @@ int solve_cg(amg_handle* h, Ctx& c, const double* b, double* x, double tol, bool
   // All further iterations in one graph launch: a conditional WHILE node whose
   // body is one iteration, whose update ends with the stopping test.
   if (h->opt.use_graphs && !(rel <= tol) && it < h->opt.max_iterations && std::isfinite(rel)) {
-    cudaGraphExec_t& wexec = flexible ? h->cg_loop_fcg : h->cg_loop_pcg;
-    int64_t& per_iter = flexible ? h->cg_loop_fcg_launches : h->cg_loop_pcg_launches;
+    const int stored = h->map.from >= 0;
+    cudaGraphExec_t& wexec = (flexible ? h->cg_loop_fcg : h->cg_loop_pcg)[stored];
+    int64_t& per_iter = (flexible ? h->cg_loop_fcg_launches : h->cg_loop_pcg_launches)[stored];
     if (!wexec && !h->cg_loop_failed) {
       const int64_t l0 = h->launches;
       cudaGraph_t g = nullptr;
@@ -1193,9 +1194,11 @@ int solve_fgmres(amg_handle* h, Ctx& c, const double* b, double* x, double tol, 
 }  // namespace
 
 void drop_loops(amg_handle* h) {
-  if (h->cg_loop_pcg) cudaGraphExecDestroy(h->cg_loop_pcg);
-  if (h->cg_loop_fcg) cudaGraphExecDestroy(h->cg_loop_fcg);
-  h->cg_loop_pcg = h->cg_loop_fcg = nullptr;
+  for (cudaGraphExec_t* loops : {h->cg_loop_pcg, h->cg_loop_fcg})
+    for (int k = 0; k < 2; ++k) {
+      if (loops[k]) cudaGraphExecDestroy(loops[k]);
+      loops[k] = nullptr;
+    }
 }
 
 int solve_device(amg_handle* h, const double* b_user, double* x_user, double tol,

@@ -274,6 +274,8 @@ void upload_weights(amg_handle* h, const std::vector<double>& w) {
   AMG_CUDA(cudaMemcpyAsync(h->steps32.p, f.data(), f.size() * sizeof(float),
                            cudaMemcpyHostToDevice, h->stream));
   AMG_CUDA(cudaStreamSynchronize(h->stream));
+  h->weights = w;
+  map_follow(h);   // the stored coarse cycle holds the weights
 }
 
 void set_level_weights(amg_handle* h, const double* w, int n) {
@@ -282,7 +284,6 @@ void set_level_weights(amg_handle* h, const double* w, int n) {
   for (int l = 0; l < nl && l < n; ++l)
     for (int e = 0; e < 3; ++e) v[4 * l + e] = w[3 * l + e];
   upload_weights(h, v);
-  map_build(h, v.data());   // the stored coarse cycle holds the weights
 }
 
 void set_weights(amg_handle* h, const double* w3) {
@@ -295,7 +296,6 @@ void set_weights(amg_handle* h, const double* w3) {
     w[4 * l + 3] = 1.0;
   }
   upload_weights(h, w);
-  map_build(h, w.data());
 }
 
 void get_weights(const amg_handle* h, double* out) {
@@ -406,23 +406,6 @@ void learn_weights(amg_handle* h, const float* theta_host, amg_learned* out) {
   level_apply<double>(h, 0, ypad.p, bpad.p);
   launch_from_padded(bpad, b, l0.n, l0.np, s, h);
   int itp = 0, itl = 0;
-  // The probes' weights are tried once each: with the cycle run operation by operation, so
-  // that the stored coarse cycle is rebuilt for the kept weights only.
-  struct Unmapped {
-    amg_handle* h;
-    int from;
-    explicit Unmapped(amg_handle* q) : h(q), from(q->map.from) {
-      h->map.from = -1;
-      drop_loops(h);
-    }
-    ~Unmapped() { restore(); }
-    void restore() {   // once: the map may be planned anew after it
-      if (!h) return;
-      drop_loops(h);
-      h->map.from = from;
-      h = nullptr;
-    }
-  } unmapped(h);
   set_level_weights(h, plain.data(), nl);
   out->rho_plain = probe_rate(h, b, x, &itp);
   out->probe_iterations_plain = itp;
@@ -449,7 +432,6 @@ void learn_weights(amg_handle* h, const float* theta_host, amg_learned* out) {
   }
   out->fell_back = keep == &plain ? 1 : 0;
   if (out->fell_back) out->rho_learned = out->rho_learned > 0 ? out->rho_learned : out->rho_plain;
-  unmapped.restore();
   set_level_weights(h, keep->data(), nl);
   for (int l = 0; l < nl && l < AMG_MAX_LEVELS; ++l)
     for (int e = 0; e < 3; ++e) out->level_weights[3 * l + e] = (*keep)[3 * l + e];

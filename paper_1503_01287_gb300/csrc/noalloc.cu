@@ -64,6 +64,7 @@ void apply_preconditioner_noalloc(amg_handle* h, const double* r, double* z) {
   double* sz = s + kNoallocStride;
   // both staging vectors are fully overwritten (the cycle starts from zero), so
   // whatever an earlier call left in the array does not matter
+  h->map.used(1);   // (filling the map for new weights allocates: left to the other calls)
   launch_to_padded(r, sr, lv.n, lv.np, h->stream, h);
   if (h->opt.precision == AMG_FP32) precondition_device<float>(h, sr, sz);
   else precondition_device<double>(h, sr, sz);

@@ -1949,7 +1949,7 @@ void build_hierarchy(amg_handle* h, const amg_matrix* m, const int32_t* tags) {
   if (h->saddle && h->opt.smoother == AMG_SMOOTHER_VANKA) vanka_setup(h);
   map_plan(h);
   autotune_levels(h);
-  map_build(h, plain.data());
+  map_build(h);
   AMG_CUDA(cudaStreamSynchronize(s));
 }
 

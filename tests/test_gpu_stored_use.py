@@ -62,3 +62,72 @@ def test_batched_statistics_name_the_stored_level(precision, tile, size, stored)
     x = torch.zeros_like(b)
     rc, st = B().solve_batched([h], [b], [x], 1, 1e-8)
     assert rc == 0 and st[0].stored_from == stored
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("size", [3, 9, 11])       # stored: level 0, level 1, more than 4,096
+def test_weight_changes(size, precision):
+    """Under new weights the cycle runs operation by operation, and repeated solves bring the
+    same stored level back; under the weights that the matrix holds it is in use at once."""
+    prob = fp.elasticity_problem(size, seed=3)
+    h, ops = handle(prob, precision=precision), handle(prob, precision=precision,
+                                                       cluster_from=0, cycle_kernel=1)
+    level = solve(h, prob).stored_from
+    assert level == (1 if size == 3 else 2)
+    h.set_weights(0.9, 1.1, 1.0)
+    ops.set_weights(0.9, 1.1, 1.0)
+    assert solve(h, prob).stored_from == 0
+    h.set_weights(1.0, 1.0, 1.0)
+    assert solve(h, prob).stored_from == level
+    h.set_weights(0.9, 1.1, 1.0)
+    want = solve(ops, prob).iterations
+    seen = []
+    for _ in range(10):
+        st = solve(h, prob)
+        assert abs(st.iterations - want) <= 1
+        seen.append(st.stored_from)
+    assert seen[0] == 0 and seen[-1] == level and seen == sorted(seen)
+    r = torch.from_numpy(np.random.default_rng(1).standard_normal(prob.n_dof)).cuda()
+    r[torch.from_numpy(np.repeat((prob.tags & fp.TAG_DIRICHLET) != 0, 3)).cuda()] = 0.0
+    z, ref = torch.zeros_like(r), torch.zeros_like(r)
+    h.apply_preconditioner(r, z)
+    ops.apply_preconditioner(r, ref)
+    # as in the tests of the stored cycle: at most 1000 (FP32: 200) roundings
+    tol = 1000 * 2.0 ** -53 if precision == 0 else 200 * 2.0 ** -24
+    assert float((z - ref).norm() / ref.norm()) <= tol
+
+
+@pytest.mark.parametrize("size,precision", [((4, 5, 3), 0), ((4, 5, 3), 1), (11, 0), (11, 1)])
+def test_a_weight_change_is_a_copy(size, precision):
+    """No matrix is filled by a change of weights itself (2 to 20 ms): well below 1 ms."""
+    import time
+    h = handle(fp.elasticity_problem(size, seed=3), precision=precision)
+    best = 1.0
+    for k in range(20):
+        t = time.perf_counter()
+        h.set_weights(0.9 + 0.01 * k, 1.1, 1.0)
+        best = min(best, time.perf_counter() - t)
+    assert best < 1e-3
+
+
+@pytest.mark.parametrize("size", [9, 12])          # 12: the batch has a matrix of its own
+def test_batched_weight_changes(size):
+    prob = fp.elasticity_problem(size, seed=3)
+    h = handle(prob, precision=1)
+    b = torch.from_numpy(np.ascontiguousarray(prob.rhs())).cuda()
+    x = torch.zeros_like(b)
+
+    def stored():
+        rc, st = B().solve_batched([h], [b], [x], 1, 1e-8)
+        assert rc == 0
+        return st[0].stored_from
+
+    level = stored()
+    assert level > 0
+    h.set_weights(0.9, 1.1, 1.0)
+    seen = [stored() for _ in range(6)]
+    assert seen[0] == 0 and seen[-1] == level
+    h.set_weights(1.0, 1.0, 1.0)
+    assert stored() == 0
+    h.set_weights(0.9, 1.1, 1.0)
+    assert stored() == level
