@@ -406,6 +406,17 @@ void learn_weights(amg_handle* h, const float* theta_host, amg_learned* out) {
   level_apply<double>(h, 0, ypad.p, bpad.p);
   launch_from_padded(bpad, b, l0.n, l0.np, s, h);
   int itp = 0, itl = 0;
+  struct Before {   // a probe that fails leaves the handle with the weights it had
+    amg_handle* h;
+    std::vector<double> w;
+    ~Before() {
+      if (!h) return;
+      try {
+        upload_weights(h, w);
+      } catch (const Error&) {   // the first error is the one reported
+      }
+    }
+  } before{h, h->weights};
   set_level_weights(h, plain.data(), nl);
   out->rho_plain = probe_rate(h, b, x, &itp);
   out->probe_iterations_plain = itp;
@@ -433,6 +444,7 @@ void learn_weights(amg_handle* h, const float* theta_host, amg_learned* out) {
   out->fell_back = keep == &plain ? 1 : 0;
   if (out->fell_back) out->rho_learned = out->rho_learned > 0 ? out->rho_learned : out->rho_plain;
   set_level_weights(h, keep->data(), nl);
+  before.h = nullptr;
   for (int l = 0; l < nl && l < AMG_MAX_LEVELS; ++l)
     for (int e = 0; e < 3; ++e) out->level_weights[3 * l + e] = (*keep)[3 * l + e];
   for (int e = 0; e < 3; ++e) out->weights[e] = (*keep)[e];

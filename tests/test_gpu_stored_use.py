@@ -131,3 +131,19 @@ def test_batched_weight_changes(size):
     assert stored() == 0
     h.set_weights(0.9, 1.1, 1.0)
     assert stored() == level
+
+
+def test_a_failing_probe_leaves_the_weights():
+    """learn_weights on a saddle handle whose Krylov method its probe solves refuse."""
+    prob = fp.mixed_elasticity_problem(4, nu=0.45, seed=4)
+    h = handle(prob, krylov=B().AMG_KRYLOV_PCG)
+    h.set_weights(0.8, 1.2, 0.7)
+    r = torch.from_numpy(np.random.default_rng(1).standard_normal(prob.n_dof)).cuda()
+    z, again = torch.zeros_like(r), torch.zeros_like(r)
+    h.apply_preconditioner(r, z)
+    w = h.weights()
+    with pytest.raises(Exception):
+        h.learn_weights(np.zeros(B().MLP_NPARAM, dtype=np.float32))
+    assert np.array_equal(h.weights(), w)
+    h.apply_preconditioner(r, again)
+    assert torch.equal(z, again)
