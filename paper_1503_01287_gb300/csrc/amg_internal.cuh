@@ -44,10 +44,14 @@ struct DBuf {
     return *this;
   }
   ~DBuf() { release(); }
-  void alloc(size_t count) {
+  void alloc(size_t count) {   // empty where there is no room
     release();
+    if (count) {
+      T* q = nullptr;
+      AMG_CUDA(cudaMalloc(&q, count * sizeof(T)));
+      p = q;
+    }
     n = count;
-    if (count) AMG_CUDA(cudaMalloc(&p, count * sizeof(T)));
   }
   void release() {
     if (p) cudaFree(p);

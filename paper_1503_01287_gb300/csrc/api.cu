@@ -475,7 +475,8 @@ int amg_apply_preconditioner(amg_handle* h, const double* r, double* z) {
     if (!h || !r || !z) fail(AMG_ERR_INVALID, "null argument");
     Level& lv = *h->L[0];
     const int64_t n4 = lv.dofs4();
-    if ((int64_t)h->kr.n < n4) { h->kr.alloc(n4); h->kz.alloc(n4); }
+    if ((int64_t)h->kr.n < n4) h->kr.alloc(n4);
+    if ((int64_t)h->kz.n < n4) h->kz.alloc(n4);
     map_refresh(h, h->map);
     h->map.used(1);
     launch_to_padded(r, h->kr, lv.n, lv.np, h->stream, h);
@@ -591,10 +592,12 @@ int amg_time_level_op(amg_handle* h, int32_t op, int32_t level, int32_t precisio
       xp.alloc(8 * (size_t)lv.n);
       AMG_CUDA(cudaMemsetAsync(xp.p, 0, xp.bytes(), h->stream));
     }
-    if (op == AMG_OP_PRECOND && (int64_t)h->kr.n < lv.dofs4()) {
-      h->kr.alloc(lv.dofs4());
-      h->kz.alloc(lv.dofs4());
-      AMG_CUDA(cudaMemsetAsync(h->kr.p, 0, h->kr.bytes(), h->stream));
+    if (op == AMG_OP_PRECOND) {
+      if ((int64_t)h->kr.n < lv.dofs4()) {
+        h->kr.alloc(lv.dofs4());
+        AMG_CUDA(cudaMemsetAsync(h->kr.p, 0, h->kr.bytes(), h->stream));
+      }
+      if ((int64_t)h->kz.n < lv.dofs4()) h->kz.alloc(lv.dofs4());
     }
     auto once = [&]() {
       switch (op) {

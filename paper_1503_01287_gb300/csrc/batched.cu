@@ -1022,6 +1022,11 @@ void alloc_batch(amg_handle* h) {
   if (h->saddle) fail(AMG_ERR_UNSUPPORTED, "batched solves are provided for the SPD kinds");
   h->batch_map = map_batch(h);
   if (!h->B.empty()) return;
+  // a call without room leaves none of it, so that the next one starts again
+  struct Undo {
+    amg_handle* h;
+    ~Undo() { if (h) h->B.clear(); }
+  } undo{h};
   h->B.resize(h->L.size());
   const bool f32 = h->opt.precision == AMG_FP32;
   auto z64 = [&](DBuf<double>& v, int64_t n) {
@@ -1069,6 +1074,7 @@ void alloc_batch(amg_handle* h) {
     BatchLevel& b = h->B[l];
     b.tile_gs = fixed >= 0 ? fixed : b.tile;
   }
+  undo.h = nullptr;
 }
 
 // initial block of one problem: x = 0, r = b, z = M r, rz, p = z, active set
