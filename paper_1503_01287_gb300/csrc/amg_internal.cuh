@@ -360,6 +360,18 @@ void map_follow(amg_handle* h);
 void map_refresh(amg_handle* h, CoarseMap& M);
 // the map of the batched solves: h->map, or h->bmap planned here; null: none
 CoarseMap* map_batch(amg_handle* h);
+// gives the maps' memory back (the cycle then runs operation by operation); false: none held
+bool map_release(amg_handle* h);
+// f(), and once more without the maps where the device had no room
+template <class F>
+auto giving_maps_back(amg_handle* h, F&& f) -> decltype(f()) {
+  try {
+    return f();
+  } catch (const Error& e) {
+    if (!h || e.code != AMG_ERR_NOMEM || !map_release(h)) throw;
+  }
+  return f();
+}
 // x = (the cycle from level map.from) b, vectors of that level in the padded layout
 template <typename T, typename IO>
 void map_apply(amg_handle* h, const IO* b, IO* x);

@@ -44,7 +44,7 @@ void max_dynamic_smem(const void* func, int bytes) {
 template <class F>
 int guarded(amg_handle* h, F&& f) {
   try {
-    return f();
+    return giving_maps_back(h, f);
   } catch (const Error& e) {
     g_last_error = e.msg;
     if (h) h->last_error = e.msg;
@@ -663,6 +663,14 @@ int amg_solve_batched(amg_handle* const* handles, int32_t n_problems, int32_t n_
     for (int p = 0; p < n_problems; ++p)
       if (!handles[p] || !B[p] || !X[p]) fail(AMG_ERR_INVALID, "null handle or vector");
     double ms = 0.0;
+    try {
+      return solve_batched(handles, n_problems, n_rhs, B, X, rel_tol, stats, &ms);
+    } catch (const Error& e) {   // no room: once more without the stored cycles of all problems
+      if (e.code != AMG_ERR_NOMEM) throw;
+      bool any = false;
+      for (int p = 0; p < n_problems; ++p) any |= map_release(handles[p]);
+      if (!any) throw;
+    }
     return solve_batched(handles, n_problems, n_rhs, B, X, rel_tol, stats, &ms);
   });
 }

@@ -703,6 +703,10 @@ constexpr float kMapMaxCond = 128.f;
 // (Mixed elasticity: 0.94 to 1.10 in FP32, 1.0 to 1.4 in FP64; elasticity and the Laplacian at
 // most 1 in FP32, in FP64 2 to 2.8 from level 0, at 5e-16, and 0.8 to 1.3 below.)
 constexpr int kMapStokesFrom = 2;
+// The share of the free device memory that a matrix may take: it is a gain in time only, and
+// the Krylov vectors, further handles and the caller's data need the rest.  (Where they do not
+// fit, the handle that asks gives its own matrices back: giving_maps_back.)
+constexpr int kMapMemoryShare = 32;
 // and the share of the coarsest solve (FP64) in the construction
 constexpr int64_t kMapCoarseWork = 4000000000ll;
 
@@ -723,6 +727,9 @@ void plan(amg_handle* h, CoarseMap& M, int most) {
     M.m = m;
     M.ld = (m + 31) / 32 * 32;
     const size_t count = (size_t)m * M.ld;
+    size_t free_bytes = 0, total_bytes = 0;
+    AMG_CUDA(cudaMemGetInfo(&free_bytes, &total_bytes));
+    if (count * (f32 ? sizeof(float) : sizeof(double)) > free_bytes / kMapMemoryShare) return;
     try {
       if (f32) M.m32.alloc(count);
       else M.m64.alloc(count);
@@ -803,6 +810,16 @@ void map_build(amg_handle* h) { fill(h, h->map); }
 void map_follow(amg_handle* h) {
   follow(h, h->map);
   follow(h, h->bmap);
+}
+
+bool map_release(amg_handle* h) {
+  if (h->map.level < 0 && h->bmap.level < 0) return false;
+  AMG_CUDA(cudaStreamSynchronize(h->stream));
+  drop_loops(h);
+  h->map = CoarseMap{};
+  h->bmap = CoarseMap{};
+  h->batch_map = nullptr;
+  return true;
 }
 
 void map_refresh(amg_handle* h, CoarseMap& M) {

@@ -1948,7 +1948,7 @@ void build_hierarchy(amg_handle* h, const amg_matrix* m, const int32_t* tags) {
   if (h->saddle && h->opt.smoother == AMG_SMOOTHER_BS) bs_setup(h);
   if (h->saddle && h->opt.smoother == AMG_SMOOTHER_VANKA) vanka_setup(h);
   map_plan(h);
-  autotune_levels(h);
+  giving_maps_back(h, [&] { autotune_levels(h); });
   map_build(h);
   AMG_CUDA(cudaStreamSynchronize(s));
 }
