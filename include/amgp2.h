@@ -157,9 +157,10 @@ typedef struct amg_options {
                                gs_* options below at -1: the levels from the first
                                of at most 10,240 unknowns (FP64 6,144; segregated
                                Gauss-Seidel 4,608) down as one stored matrix, the
-                               cycle's own linear map, built at setup (under
-                               other weights the operations, until solves have
-                               repaid building it for them; not for badly
+                               cycle's own linear map, built at setup and for
+                               weights set before the first solve (under others
+                               later the operations, until solves have repaid
+                               building it for them; not for badly
                                conditioned diagonal blocks, nor Stokes with the
                                FP32 cycle); else chosen by timing                */
   int32_t cycle_kernel;     /* 0: as cluster_from -1 (default); 1: one

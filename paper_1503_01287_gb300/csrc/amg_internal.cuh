@@ -225,7 +225,9 @@ struct CoarseMap {
   DBuf<double> m64;
   std::vector<double> w, seen;   // its levels' weights: as built, and the current ones
   int64_t waited = 0;            // applications without it since these are the current ones
+  bool fresh = false;            // filled by the setup, no application and no other weights yet
   void used(int64_t applications) {
+    fresh = false;
     if (level >= 0 && from < 0) waited += applications;
   }
 };
@@ -351,7 +353,7 @@ void set_subcycle(amg_handle* h, int from);
 // coarse_map.cu: the cycle below a level as one stored matrix
 // picks the level of h->map and allocates the matrix (before autotune_levels)
 void map_plan(amg_handle* h);
-// fills h->map for the current level weights
+// fills h->map for the current level weights where it holds others
 void map_build(amg_handle* h);
 // the level weights changed: the maps are in use where they were built with them
 void map_follow(amg_handle* h);

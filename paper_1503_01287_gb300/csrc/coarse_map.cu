@@ -8,8 +8,9 @@
 // level 1, for 8,538 unknowns; FP64 24^3: 690 us of 1317 us for 3,144).  M b instead reads
 // m^2 values once.  M is filled at setup by running the cycle's own recorded operations on
 // blocks of unit vectors, so it is the same operator, weights, smoother and cycle type, in the
-// cycle's precision.  Under other level weights the cycle runs operation by operation, until
-// M is filled for them (map_refresh); back under its own weights M is in use again.
+// cycle's precision.  It follows the weights that a program sets before its first solve.  Under
+// other weights later the cycle runs operation by operation, until M is filled for them
+// (map_refresh); back under its own weights M is in use again.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -30,12 +31,14 @@ namespace {
 // consecutive threads take consecutive vectors and every value of an operator is one
 // broadcast load for a warp.  A thread holds 2 vectors (16 bytes an entry).
 //
-// FP64 handles build in FP64.  FP32 handles build in FP32 pairs (hi + lo, as the Krylov
-// operator) with the cycle's own FP32 (or BF16) operator values: M is then the cycle of
-// those operators to about 2^-48, rounded once, and M b is no further from the 64-bit
-// cycle than the FP32 operations were.  Built in plain FP32, M doubled that error (32^3:
-// 7.1e-7 against 3.4e-7 relative).  FP64 would take the m nnz FMAs of three sweeps at
-// 0.5e12 a second (87 ms at 32^3); the pairs issue at the FP32 rate.
+// FP64 handles build in FP64.  FP32 handles build in FP32 pairs (hi + lo) with the cycle's own
+// FP32 (or BF16) operator values, to well below the rounding of M to FP32 that follows (mac
+// below: not to the 2^-48 of the Krylov operator's pairs).  M b is then about as far from the
+// FP64 cycle as the FP32 operations: 0.89 to 0.98 times for elasticity and the Laplacian,
+// 0.94 to 1.10 for mixed elasticity (kMapMaxCond and kMapStokesFrom say where it is further).
+// Built in plain FP32, M doubled that error (32^3: 7.1e-7 against 3.4e-7 relative).  FP64 would
+// take the m nnz FMAs of three sweeps at 0.5e12 a second (87 ms at 32^3); the pairs issue at
+// the FP32 rate.
 constexpr int kColThreads = 128;
 constexpr int kColN = 2;                             // vectors of a thread
 constexpr int kColBlock = kColThreads * kColN;       // vectors of a CTA
@@ -665,14 +668,21 @@ const T* matrix(const CoarseMap& M) {
 }
 
 // The largest level stored as a matrix.  Below these sizes M b is faster than the chain
-// of launches that it replaces: reading M takes 4 m^2 bytes at about 6 TB/s in FP32 (63 us
-// at 10,240) against 65 launches of 2 to 5 us and the levels below; in FP64 the m^2 FMAs
-// take 75 us at 6,144 (0.5e12 a second on this GPU).  They also bound the memory (420 and
-// 300 MB) and the time of the construction.
+// of launches that it replaces: reading M takes 4 m^2 bytes at 5.6 TB/s in FP32 (75 us at
+// 10,240; 52 us at 8,538, in place of 280 us) against 65 launches of 2 to 5 us and the levels
+// below; in FP64 the m^2 FMAs take 75 us at 6,144 (0.5e12 a second on this GPU).  They also
+// bound the memory (420 and 300 MB) and the time of the construction (20 ms at 8,538).
 constexpr int kMapMax32 = 10240;
 constexpr int kMapMax64 = 6144;
-// A segregated Gauss-Seidel level is 7 launches, not 65: Stokes 24^3 in FP64 gains 60 us of
-// 580 a preconditioner by its map of 4,159, built in 16 ms.
+// A segregated Gauss-Seidel level is 7 launches, not 65, so a large map saves less beyond the
+// next smaller one.  Mixed elasticity, an application with the map of the size given against
+// the next smaller, and its construction:
+//   FP32  3,065 (9^3) 70 against 117 us, 3.6 ms     4,159 (24^3) 251 against 295, 3.6 ms
+//         6,371 (28^3) 353 against 388, 7.8 ms      8,706 (13x11x15) 122 against 130, 13 ms
+//         9,267 (32^3) 485 against 499, 18 ms
+//   FP64  3,065 108 against 172 us, 7.0 ms          4,159 525 against 579, 15 ms
+// An FGMRES solve is 50 to 130 applications: up to 4,159 a solve repays it in FP32 (in FP64
+// three do), at 6,371 two to four, beyond that ten and more.
 constexpr int kMapMaxSgs = 4608;
 // Applications operation by operation, under weights that M was not built with, after which
 // it is filled for them: by then what M would have saved is about what filling it costs, so a
@@ -768,13 +778,18 @@ void fill(amg_handle* h, CoarseMap& M) {
   M.from = M.level;
 }
 
-// in use where the weights are those that it was built with
+// In use where the weights are those that it was built with.  The setup's matrix is filled
+// again for weights that a program sets before it uses the handle: it would be of no use.
 void follow(amg_handle* h, CoarseMap& M) {
   if (M.level < 0) return;
   const std::vector<double> now = own_weights(h, M);
   if (now != M.seen) M.waited = 0;
   M.seen = now;
   M.from = now == M.w ? M.level : -1;
+  if (M.from < 0 && M.fresh) {
+    M.fresh = false;
+    fill(h, M);
+  }
 }
 
 }  // namespace
@@ -805,7 +820,9 @@ CoarseMap* map_batch(amg_handle* h) {
   return &M;
 }
 
-void map_build(amg_handle* h) { fill(h, h->map); }
+void map_build(amg_handle* h) {
+  if (h->map.from < 0) fill(h, h->map);
+}
 
 void map_follow(amg_handle* h) {
   follow(h, h->map);

@@ -417,6 +417,7 @@ void learn_weights(amg_handle* h, const float* theta_host, amg_learned* out) {
       }
     }
   } before{h, h->weights};
+  h->map.fresh = false;   // not filled for weights that are only tried
   set_level_weights(h, plain.data(), nl);
   out->rho_plain = probe_rate(h, b, x, &itp);
   out->probe_iterations_plain = itp;
@@ -445,6 +446,7 @@ void learn_weights(amg_handle* h, const float* theta_host, amg_learned* out) {
   if (out->fell_back) out->rho_learned = out->rho_learned > 0 ? out->rho_learned : out->rho_plain;
   set_level_weights(h, keep->data(), nl);
   before.h = nullptr;
+  map_build(h);           // but for those that are kept
   for (int l = 0; l < nl && l < AMG_MAX_LEVELS; ++l)
     for (int e = 0; e < 3; ++e) out->level_weights[3 * l + e] = (*keep)[3 * l + e];
   for (int e = 0; e < 3; ++e) out->weights[e] = (*keep)[e];

@@ -1950,6 +1950,7 @@ void build_hierarchy(amg_handle* h, const amg_matrix* m, const int32_t* tags) {
   map_plan(h);
   giving_maps_back(h, [&] { autotune_levels(h); });
   map_build(h);
+  h->map.fresh = true;
   AMG_CUDA(cudaStreamSynchronize(s));
 }
 

@@ -1,4 +1,6 @@
 """Which solves run the coarse cycle as a stored matrix, as their statistics tell it."""
+import os
+
 import numpy as np
 import pytest
 
@@ -131,6 +133,31 @@ def test_batched_weight_changes(size):
     assert stored() == 0
     h.set_weights(0.9, 1.1, 1.0)
     assert stored() == level
+
+
+@pytest.mark.parametrize("size", [3, 11])
+def test_weights_set_after_setup(size):
+    """The matrix is filled for the weights that a program sets before its first solve, and
+    once only."""
+    prob = fp.elasticity_problem(size, seed=3)
+    h = handle(prob, precision=1)
+    h.set_weights(0.9, 1.1, 1.0)
+    assert solve(h, prob).stored_from > 0
+    h = handle(prob, precision=1)
+    h.set_weights(0.9, 1.1, 1.0)
+    h.set_weights(0.8, 1.1, 1.0)
+    assert solve(h, prob).stored_from == 0
+    h.set_weights(0.9, 1.1, 1.0)
+    assert solve(h, prob).stored_from > 0
+
+
+def test_learned_weights_are_stored():
+    prob = fp.elasticity_problem((4, 5, 3), seed=1)
+    h = handle(prob, precision=1)
+    solve(h, prob)
+    theta = np.load(os.path.join(os.path.dirname(B().__file__), "weights", "mlp_theta.npy"))
+    h.learn_weights(theta)
+    assert solve(h, prob).stored_from == 1
 
 
 def test_a_failing_probe_leaves_the_weights():
