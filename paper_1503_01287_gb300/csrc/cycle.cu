@@ -1921,7 +1921,6 @@ void launch_rows_v(const Phase& P, cudaStream_t s, bool pdl) {
   }
   if (pdl && P.mode == kGS && P.rows) {
     switch (P.G) {
-      case 4: launch_gs_pdl<T, 4, false, V>(P, s); return;
       case 8: launch_gs_pdl<T, 8, false, V>(P, s); return;
       case 16: launch_gs_pdl<T, 16, false, V>(P, s); return;
       default: launch_gs_pdl<T, 32, false, V>(P, s); return;
@@ -1929,7 +1928,6 @@ void launch_rows_v(const Phase& P, cudaStream_t s, bool pdl) {
   }
   if (pdl && P.mode == kFirst && P.rows) {
     switch (P.G) {
-      case 4: launch_gs_pdl<T, 4, true, V>(P, s); return;
       case 8: launch_gs_pdl<T, 8, true, V>(P, s); return;
       case 16: launch_gs_pdl<T, 16, true, V>(P, s); return;
       default: launch_gs_pdl<T, 32, true, V>(P, s); return;
@@ -2851,9 +2849,10 @@ void set_subcycle(amg_handle* h, int from) {
   h->sub_from = from;
 }
 
-// Lanes per block row (4, 8, 16 or 32) of every level, from timing the operator
-// kernel and, separately, one colour sweep; then the level from which the cycle
-// runs as one cluster launch, from timing whole preconditioner applications.
+// Lanes per block row (4, 8, 16 or 32) of the row kernels, from timing the operator on every
+// level that runs as operations; those of the colour kernels by gs_lanes.  Without a stored
+// coarse cycle also the other sweep kernels and the level from which the cycle runs as one
+// cluster launch, from timing sweeps and whole preconditioner applications.
 void autotune_levels(amg_handle* h) {
   cudaStream_t s = h->stream;
   cudaEvent_t e0, e1;
@@ -2870,7 +2869,9 @@ void autotune_levels(amg_handle* h) {
   const bool f32 = h->opt.precision == AMG_FP32;
   for (auto& lv : h->L)
     if (lv->ncolours > 0) lv->group_gs = gs_lanes(f32, (double)lv->n / lv->ncolours);
-  // levels that run as one stored matrix keep the default lanes per row
+  // levels that run as one stored matrix keep the default lanes per row (group_for), also for
+  // the time that they run as operations under other weights: within 1 % of the timed ones in
+  // a preconditioner application (elasticity 7x5x11 to 32^3, mixed and Stokes to 24^3)
   const size_t nl = h->map.level >= 0 ? std::max(h->map.level, 1) : h->L.size();
   for (size_t l = 0; l < nl; ++l) {
     Level& lv = *h->L[l];
@@ -2924,8 +2925,12 @@ void autotune_levels(amg_handle* h) {
         h->map.level == 0)
       continue;
     lv.gs_stream = 0;
-    if (h->map.level >= 0) continue;   // the other sweep kernels below were slower on every
-                                      // level that the stored matrix leaves to the chain
+    // With a stored cycle the other sweep kernels are not timed: of the levels that it leaves to
+    // the chain (elasticity 7x5x11 to 32^3, both precisions) timing chose one of them only on
+    // level 0 of 11^3 in FP64 (k_gs_stream, 82 against 93 us a sweep) and level 1 of 32^3 in
+    // FP64 (288 against 304), and with them the sweep from x = 0 reads all of A (32^3: 1926
+    // against 1684 us an application of operations).
+    if (h->map.level >= 0) continue;
     auto sweep_ms = [&]() {
       for (int r = 0; r < 7; ++r) {
         if (r == 2) AMG_CUDA(cudaEventRecord(e0, s));
